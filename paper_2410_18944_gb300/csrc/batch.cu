@@ -36,6 +36,8 @@ namespace {
 
 constexpr int kBatchPlainBlock = 128;
 constexpr int kBatchGuidedSmem = ws_smem_bytes(true);
+static_assert(kBatchGuidedSmem % alignof(CoopWarp) == 0, "query workspaces follow the tiles");
+constexpr int batch_guided_smem(int D, int W) { return kBatchGuidedSmem + coop_bytes(D, W); }
 // counter block of a plan (unsigned long long words)
 constexpr int kCtrStat = 8;       // [8, 15): launch statistics
 constexpr int kCtrRec = 16;       // [16, 18): records appended / dropped over all rounds
@@ -49,13 +51,13 @@ struct BatchGuidedArgs {
 
 template <int D>
 __global__ void __launch_bounds__(kBatchPlainBlock) batch_plain_kernel(const __grid_constant__ BatchArgs b) {
-    plain_loop<D>(BatchSrc<D>{b}, b.stat);
+    plain_loop<D, true>(coop_shared<D, kBatchPlainBlock / 32>(), BatchSrc<D>{b}, b.stat);
 }
 
 template <int D, int W>
 __global__ void __launch_bounds__(ws_threads(W), 1) batch_guided_kernel(const __grid_constant__ BatchGuidedArgs g) {
     extern __shared__ __align__(1024) uint8_t sm[];
-    guided_ws_body<D, true, W>(BatchSrc<D>{g.b}, g.o, sm);
+    guided_ws_body<D, true, W>(BatchSrc<D>{g.b}, g.o, sm, sm + kBatchGuidedSmem);
 }
 
 // job owning batch point i: the last job whose point_off <= i
@@ -70,13 +72,15 @@ __device__ __forceinline__ int find_job(const DevJob *jobs, int njobs, int64_t i
 }
 
 template <int D>
-__global__ void batch_classify_kernel(const DevJob *jobs, int njobs, int64_t n, uint8_t *status, double *shell,
+__global__ void __launch_bounds__(128) batch_classify_kernel(const DevJob *jobs, int njobs, int64_t n, uint8_t *status, double *shell,
                                       int *err) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const DevJob &J = jobs[find_job(jobs, njobs, i)];
+    const bool act = i < n;
+    const DevJob &J = jobs[find_job(jobs, njobs, act ? i : n - 1)];
     double val;
-    status[i] = classify_point<D>(J.sc, J.eps64, J.points + (i - J.point_off) * D, err, val);
+    const uint8_t st = classify_point<D, true>(coop_shared<D, 4>(), J.sc, J.eps64, J.points + (i - J.point_off) * D, act, err, val);
+    if (!act) return;
+    status[i] = st;
     shell[i] = val;
 }
 
@@ -178,10 +182,10 @@ struct wost_batch {
             g.o.stat = b.stat;
             constexpr int tn = ws_threads(kWsWalkerWarps), tw = ws_threads(kWsWalkersWide);
             const bool wide = walkers_ == kWsWalkersWide;
-            if (dim == 2 && wide) batch_guided_kernel<2, kWsWalkersWide><<<num_sms(), tw, kBatchGuidedSmem, st>>>(g);
-            else if (dim == 2) batch_guided_kernel<2, kWsWalkerWarps><<<num_sms(), tn, kBatchGuidedSmem, st>>>(g);
-            else if (wide) batch_guided_kernel<3, kWsWalkersWide><<<num_sms(), tw, kBatchGuidedSmem, st>>>(g);
-            else batch_guided_kernel<3, kWsWalkerWarps><<<num_sms(), tn, kBatchGuidedSmem, st>>>(g);
+            if (dim == 2 && wide) batch_guided_kernel<2, kWsWalkersWide><<<num_sms(), tw, batch_guided_smem(2, kWsWalkersWide), st>>>(g);
+            else if (dim == 2) batch_guided_kernel<2, kWsWalkerWarps><<<num_sms(), tn, batch_guided_smem(2, kWsWalkerWarps), st>>>(g);
+            else if (wide) batch_guided_kernel<3, kWsWalkersWide><<<num_sms(), tw, batch_guided_smem(3, kWsWalkersWide), st>>>(g);
+            else batch_guided_kernel<3, kWsWalkerWarps><<<num_sms(), tn, batch_guided_smem(3, kWsWalkerWarps), st>>>(g);
         }
         WOST_CUDA(cudaGetLastError());
         return WOST_OK;
@@ -431,11 +435,11 @@ wost_status build_plan(wost_batch *p) {
     if (p->guided) {
         const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
         if (D == 2) {
-            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<2, kWsWalkerWarps>, at, kBatchGuidedSmem));
-            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<2, kWsWalkersWide>, at, kBatchGuidedSmem));
+            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<2, kWsWalkerWarps>, at, batch_guided_smem(2, kWsWalkerWarps)));
+            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<2, kWsWalkersWide>, at, batch_guided_smem(2, kWsWalkersWide)));
         } else {
-            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<3, kWsWalkerWarps>, at, kBatchGuidedSmem));
-            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<3, kWsWalkersWide>, at, kBatchGuidedSmem));
+            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<3, kWsWalkerWarps>, at, batch_guided_smem(3, kWsWalkerWarps)));
+            WOST_CUDA(cudaFuncSetAttribute(batch_guided_kernel<3, kWsWalkersWide>, at, batch_guided_smem(3, kWsWalkersWide)));
         }
     }
     device_err_flag();   // created outside the capture

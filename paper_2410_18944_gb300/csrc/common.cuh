@@ -94,15 +94,15 @@ __device__ __forceinline__ float eval_fn(const DevFn &fn, const float *x) {
 }
 
 // ---------------------------------------------------------------------------
-// Scene view.  BVH node layout (binary BVH, child boxes stored in the parent):
-//   2D: 3 float4 = (c0.lo.x, c0.lo.y, c0.hi.x, c0.hi.y), (c1 ...), (ref0, ref1, -, -)
-//   3D: 4 float4 = (c0.lo.xyz, c0.hi.x), (c0.hi.yz, c1.lo.xy), (c1.lo.z, c1.hi.xyz), (ref0, ref1, -, -)
+// Scene view.  BVH node layouts: geom.cuh (2D: 3 float4 = (c0.lo.xy, c0.hi.xy),
+// (c1 ...), (ref0, ref1, -, -)).
 // ref >= 0: inner node index; ref < 0: leaf, ~ref = start << 4 | (count - 1).
 // Primitives are stored in leaf order:
 //   Dirichlet / Neumann 2D segment: 1 float4 (a.x, a.y, b.x, b.y)
 //   3D triangle: 3 float4 (a.xyz, b.x), (b.yz, c.xy), (c.z, -, -, -)
 //   silhouette 2D vertex: 2 float4 (v.xy, n0.xy), (n1.xy, always, -)
-//   silhouette 3D edge:   4 float4 (a.xyz, b.x), (b.yz, n0.xy), (n0.z, n1.xyz), (always, -, -, -)
+//   silhouette 3D edge:   3 float4 (a.xyz, b.x), (b.yz, n0.xy), (n0.z, n1.xyz); an edge that is always a
+//                         silhouette carries zero normals
 // n0/n1 are inward unit normals of the two adjacent Neumann primitives.
 // ---------------------------------------------------------------------------
 struct DevBVH {
@@ -112,6 +112,7 @@ struct DevBVH {
     const double *prims64; // FP64 copy of the primitive vertices (leaf order), 2D: 4, 3D: 9 doubles
     int nprims;
     int nnodes;
+    int need;             // 3D Dirichlet BVH: most stack entries a depth-first traversal of its caps holds
 };
 
 struct DevScene {
@@ -119,7 +120,8 @@ struct DevScene {
     float scale;          // bounding-box diagonal
     float tau;            // silhouette edge-on tolerance (1e-6 * scale)
     DevBVH dir, neu, sil;
-    const float4 *sil_cones;  // per silhouette-BVH node: one normal cone per child (axis.xyz, cos half-angle)
+    const float4 *dir_caps;   // per Dirichlet-BVH node: caps of the children and their references (layout at cap_f4)
+    const float4 *sil_facing; // per silhouette-BVH node: one facing bound per child (layout at facing_f4)
     const float *nin_neu; // inward normal of each Neumann prim, by leaf slot of the Neumann BVH (dim floats)
     DevFn g, f, h;
     int has_source;

@@ -13,6 +13,11 @@ namespace wost {
 
 constexpr int kStack = 64;
 
+// width of the band (relative to the scene scale) inside which an FP32
+// distance or hit parameter may be on the wrong side of its threshold:
+// 16 units of 2^-24
+constexpr float kRoundBand = 16.f * 5.9604645e-8f;
+
 // The closest-point, closest-silhouette and ray queries compiled out of line
 // (a call per query; the caller's live registers no longer add to the
 // traversal's), or inlined into the walk step.  Measured on one GB300,
@@ -28,29 +33,17 @@ constexpr int kStack = 64;
 #define WOST_QUERY_FN
 #endif
 
-// Children per BVH node, by dimension: 2 (binary, child boxes in the
-// parent) or 4 (the binary tree collapsed one level: four child boxes per
-// node, stored one coordinate of all four children per float4).  Width 4
-// halves the chain of dependent node loads from the root to a leaf.
-// Measured on one GB300: 3D walks 8-10% faster with width 4 (L2-resident
-// BVHs of 82k and 994k triangles); 2D walks 25-31% slower (the 4096-segment
-// scene's BVH sits in L1 or shared memory, and the wider visit costs more
-// instructions and registers than the shorter chain saves).
-#ifndef WOST_BVH_WIDTH_2D
-#define WOST_BVH_WIDTH_2D 2
-#endif
-#ifndef WOST_BVH_WIDTH_3D
-#define WOST_BVH_WIDTH_3D 4
-#endif
-__host__ __device__ constexpr int bvh_width(int d) { return d == 2 ? WOST_BVH_WIDTH_2D : WOST_BVH_WIDTH_3D; }
-static_assert((bvh_width(2) == 2 || bvh_width(2) == 4) && (bvh_width(3) == 2 || bvh_width(3) == 4),
-              "BVH width must be 2 or 4");
-constexpr int kEmptyRef = INT_MIN;   // child slot without a child (width 4)
+// BVH nodes.  2D: binary, child boxes in the parent (3 float4), one query per
+// lane (this file).  3D: four children per node, 4 x (lo.xyz, hi.x), then
+// 4 x (hi.yz, child, -), one query per group of lanes (coop.cuh; neumann_pick
+// one per lane).
+constexpr int lane_width(int d) { return d == 2 ? 2 : 4; }
+constexpr int kEmptyRef = INT_MIN;   // child slot without a child (wide nodes)
 
-// float4 per node: width 2: 2D 3, 3D 4; width 4: 2D 5, 3D 7
+// float4 per node
 template <int D>
 __host__ __device__ constexpr int node_f4() {
-    return bvh_width(D) == 2 ? (D == 2 ? 3 : 4) : (D == 2 ? 5 : 7);
+    return D == 2 ? 3 : 8;
 }
 
 // per-thread visit counts of the traversals (algorithmic-traffic accounting)
@@ -58,60 +51,51 @@ struct Visits {
     uint32_t nodes = 0, dprims = 0, sprims = 0, nprims = 0;
 };
 
-// squared distance from x to the two child boxes of a node
+// squared distance from the distances along the axes, with its rounding
+// spelled out: whether a box is opened is decided on this value
+__device__ __forceinline__ float box_d2(float dx, float dy, float dz) {
+    return __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
+}
+
+// keys of the children: squared distance from x to the child box (2D: the
+// binary nodes; 3D: the four-wide ones)
 template <int D>
-__device__ __forceinline__ void node_box_d2(const float4 *nodes, int node, const float *x,
-                                            float &d0, float &d1, int &r0, int &r1) {
-    if (D == 2) {
-        const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), r = ldn(nodes + 3 * node + 2);
+__device__ __forceinline__ void node_keys_d2(const float4 *nodes, int node, const float *x, float *k, int *r) {
+    if constexpr (D == 2) {
+        const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), q = ldn(nodes + 3 * node + 2);
         float ax = fmaxf(fmaxf(a.x - x[0], x[0] - a.z), 0.f), ay = fmaxf(fmaxf(a.y - x[1], x[1] - a.w), 0.f);
         float bx = fmaxf(fmaxf(b.x - x[0], x[0] - b.z), 0.f), by = fmaxf(fmaxf(b.y - x[1], x[1] - b.w), 0.f);
-        d0 = ax * ax + ay * ay;
-        d1 = bx * bx + by * by;
-        r0 = __float_as_int(r.x);
-        r1 = __float_as_int(r.y);
+        k[0] = ax * ax + ay * ay;
+        k[1] = bx * bx + by * by;
+        r[0] = __float_as_int(q.x);
+        r[1] = __float_as_int(q.y);
     } else {
-        const float4 a = ldn(nodes + 4 * node), b = ldn(nodes + 4 * node + 1);
-        const float4 c = ldn(nodes + 4 * node + 2), r = ldn(nodes + 4 * node + 3);
-        // child 0: lo = (a.x, a.y, a.z) hi = (a.w, b.x, b.y); child 1: lo = (b.z, b.w, c.x) hi = (c.y, c.z, c.w)
-        float ax = fmaxf(fmaxf(a.x - x[0], x[0] - a.w), 0.f);
-        float ay = fmaxf(fmaxf(a.y - x[1], x[1] - b.x), 0.f);
-        float az = fmaxf(fmaxf(a.z - x[2], x[2] - b.y), 0.f);
-        float bx = fmaxf(fmaxf(b.z - x[0], x[0] - c.y), 0.f);
-        float by = fmaxf(fmaxf(b.w - x[1], x[1] - c.z), 0.f);
-        float bz = fmaxf(fmaxf(c.x - x[2], x[2] - c.w), 0.f);
-        d0 = ax * ax + ay * ay + az * az;
-        d1 = bx * bx + by * by + bz * bz;
-        r0 = __float_as_int(r.x);
-        r1 = __float_as_int(r.y);
+        const float4 *p = nodes + (size_t)node_f4<3>() * node;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float4 a = ldn(p + c), b = ldn(p + 4 + c);
+            float dx = fmaxf(fmaxf(a.x - x[0], x[0] - a.w), 0.f);
+            float dy = fmaxf(fmaxf(a.y - x[1], x[1] - b.x), 0.f);
+            float dz = fmaxf(fmaxf(a.z - x[2], x[2] - b.y), 0.f);
+            k[c] = box_d2(dx, dy, dz);
+            r[c] = __float_as_int(b.z);
+        }
     }
 }
 
-// entry/exit of the ray o + t v (inv = 1/v) with the two child boxes
-// (exit casts: from t > -pad, boxes grown by pad on every side, so that
-// crossings within the rounding band of a primitive are not pruned)
-template <int D>
-__device__ __forceinline__ void node_box_ray(const float4 *nodes, int node, const float *o,
-                                             const float *inv, float tmax, float &t0, float &t1,
-                                             int &r0, int &r1, float pad = 0.f) {
-    float lo0[3], hi0[3], lo1[3], hi1[3];
-    if (D == 2) {
-        const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), r = ldn(nodes + 3 * node + 2);
-        lo0[0] = a.x; lo0[1] = a.y; hi0[0] = a.z; hi0[1] = a.w;
-        lo1[0] = b.x; lo1[1] = b.y; hi1[0] = b.z; hi1[1] = b.w;
-        r0 = __float_as_int(r.x);
-        r1 = __float_as_int(r.y);
-    } else {
-        const float4 a = ldn(nodes + 4 * node), b = ldn(nodes + 4 * node + 1);
-        const float4 c = ldn(nodes + 4 * node + 2), r = ldn(nodes + 4 * node + 3);
-        lo0[0] = a.x; lo0[1] = a.y; lo0[2] = a.z; hi0[0] = a.w; hi0[1] = b.x; hi0[2] = b.y;
-        lo1[0] = b.z; lo1[1] = b.w; lo1[2] = c.x; hi1[0] = c.y; hi1[1] = c.z; hi1[2] = c.w;
-        r0 = __float_as_int(r.x);
-        r1 = __float_as_int(r.y);
-    }
+// keys of the children of a binary 2D node: entry parameter of the ray
+// o + t v (inv = 1/v) into the child box grown by pad, from t > -pad, +inf if
+// it misses within tmax (exit casts grow the boxes, so that crossings within
+// the rounding band of a primitive are not pruned)
+__device__ __forceinline__ void node_keys_ray(const float4 *nodes, int node, const float *o, const float *inv,
+                                              float tmax, float *kk, int *r, float pad) {
+    const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), q = ldn(nodes + 3 * node + 2);
+    const float lo0[2] = {a.x, a.y}, hi0[2] = {a.z, a.w}, lo1[2] = {b.x, b.y}, hi1[2] = {b.z, b.w};
+    r[0] = __float_as_int(q.x);
+    r[1] = __float_as_int(q.y);
     float e0 = -pad, x0 = tmax, e1 = -pad, x1 = tmax;
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
+    for (int k = 0; k < 2; ++k) {
         float a0 = (lo0[k] - pad - o[k]) * inv[k], b0 = (hi0[k] + pad - o[k]) * inv[k];
         float a1 = (lo1[k] - pad - o[k]) * inv[k], b1 = (hi1[k] + pad - o[k]) * inv[k];
         e0 = fmaxf(e0, fminf(a0, b0));
@@ -119,84 +103,9 @@ __device__ __forceinline__ void node_box_ray(const float4 *nodes, int node, cons
         e1 = fmaxf(e1, fminf(a1, b1));
         x1 = fminf(x1, fmaxf(a1, b1));
     }
-    t0 = e0 <= x0 ? e0 : __int_as_float(0x7f800000);
-    t1 = e1 <= x1 ? e1 : __int_as_float(0x7f800000);
+    kk[0] = e0 <= x0 ? e0 : __int_as_float(0x7f800000);
+    kk[1] = e1 <= x1 ? e1 : __int_as_float(0x7f800000);
 }
-
-// ---- node visits of either width ---------------------------------------------
-// keys of the children: squared distance from x to the child box
-template <int D>
-__device__ __forceinline__ void node_keys_d2(const float4 *nodes, int node, const float *x, float *k, int *r) {
-    constexpr int kBW = bvh_width(D);
-    if (kBW == 2) {
-        node_box_d2<D>(nodes, node, x, k[0], k[1], r[0], r[1]);
-        return;
-    }
-    const float4 *p = nodes + (size_t)node_f4<D>() * node;
-    const float4 lx = ldn(p), ly = ldn(p + 1);
-    const float4 lz = D == 3 ? ldn(p + 2) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 hx = ldn(p + (D == 3 ? 3 : 2)), hy = ldn(p + (D == 3 ? 4 : 3));
-    const float4 hz = D == 3 ? ldn(p + 5) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 rr = ldn(p + (D == 3 ? 6 : 4));
-    const float LX[4] = {lx.x, lx.y, lx.z, lx.w}, LY[4] = {ly.x, ly.y, ly.z, ly.w}, LZ[4] = {lz.x, lz.y, lz.z, lz.w};
-    const float HX[4] = {hx.x, hx.y, hx.z, hx.w}, HY[4] = {hy.x, hy.y, hy.z, hy.w}, HZ[4] = {hz.x, hz.y, hz.z, hz.w};
-    const float RR[4] = {rr.x, rr.y, rr.z, rr.w};
-#pragma unroll
-    for (int c = 0; c < kBW; ++c) {
-        float dx = fmaxf(fmaxf(LX[c] - x[0], x[0] - HX[c]), 0.f);
-        float dy = fmaxf(fmaxf(LY[c] - x[1], x[1] - HY[c]), 0.f);
-        float d2 = dx * dx + dy * dy;
-        if (D == 3) {
-            float dz = fmaxf(fmaxf(LZ[c] - x[2], x[2] - HZ[c]), 0.f);
-            d2 += dz * dz;
-        }
-        k[c] = d2;
-        r[c] = __float_as_int(RR[c]);
-    }
-}
-
-// keys of the children: entry parameter of the ray o + t v (inv = 1/v) into
-// the child box grown by pad, from t > -pad, +inf if it misses within tmax
-template <int D>
-__device__ __forceinline__ void node_keys_ray(const float4 *nodes, int node, const float *o, const float *inv,
-                                              float tmax, float *k, int *r, float pad) {
-    constexpr int kBW = bvh_width(D);
-    if (kBW == 2) {
-        node_box_ray<D>(nodes, node, o, inv, tmax, k[0], k[1], r[0], r[1], pad);
-        return;
-    }
-    const float4 *p = nodes + (size_t)node_f4<D>() * node;
-    float4 lo4[3], hi4[3];
-    lo4[0] = ldn(p);
-    lo4[1] = ldn(p + 1);
-    lo4[2] = D == 3 ? ldn(p + 2) : make_float4(0.f, 0.f, 0.f, 0.f);
-    hi4[0] = ldn(p + (D == 3 ? 3 : 2));
-    hi4[1] = ldn(p + (D == 3 ? 4 : 3));
-    hi4[2] = D == 3 ? ldn(p + 5) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 rr = ldn(p + (D == 3 ? 6 : 4));
-    const float RR[4] = {rr.x, rr.y, rr.z, rr.w};
-    float e[4] = {-pad, -pad, -pad, -pad}, xm[4] = {tmax, tmax, tmax, tmax};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const float L[4] = {lo4[a].x, lo4[a].y, lo4[a].z, lo4[a].w};
-        const float H[4] = {hi4[a].x, hi4[a].y, hi4[a].z, hi4[a].w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float t0 = (L[c] - pad - o[a]) * inv[a], t1 = (H[c] + pad - o[a]) * inv[a];
-            e[c] = fmaxf(e[c], fminf(t0, t1));
-            xm[c] = fminf(xm[c], fmaxf(t0, t1));
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        k[c] = e[c] <= xm[c] ? e[c] : __int_as_float(0x7f800000);
-        r[c] = __float_as_int(RR[c]);
-    }
-}
-
-// box of child c (cone tests)
-template <int D>
-__device__ __forceinline__ void node_child_box(const float4 *nodes, int node, int c, float *lo, float *hi);
 
 // Continue at the nearest child with h[c] (ties: the lower child index) and
 // push the others, farthest first.  Returns false if no child is taken.
@@ -237,6 +146,38 @@ __device__ __forceinline__ bool take_children(const float *k, const int *r, cons
     }
     ref = rr[0];
     return true;
+}
+
+// ---- oriented caps ------------------------------------------------------------
+// Bound of the closest-point search: a cap around the primitives of a child,
+// centre c, axis a (their mean normal), half thickness h along a and radius r
+// across it (3D: a flat cylinder; 2D: an oriented box).  A boundary patch is
+// thin along its normal, so seen from the front, as walks see the boundary,
+// the cap's distance is that of the patch within curvature x r^2; the distance
+// to its axis-aligned box falls short by about r, and a search from afar has
+// to open every patch whose box is nearer than the closest point: patches
+// within about sqrt(r R) of it (R: the walk's distance) instead of a few r.
+// h and r carry a margin of 1e-6 x the scene's extent, more than the rounding
+// of this distance and of a primitive's own: every primitive at or below the
+// bound is tested, whatever the order of visits.
+// Per node: 2D (2 children) (c.xy, a.xy) of each, (h0, r0, h1, r1), (ref0,
+// ref1, -, -); 3D (8 children) 8 x (c.xyz, h), 8 x (a.xyz, r), 8 references.
+__host__ __device__ constexpr int cap_f4(int d) { return d == 2 ? 4 : 18; }
+
+// squared distance from x to the cap (c, a as loaded; 2D: c = (c.xy, a.xy))
+__device__ __forceinline__ float cap_d2_2(float4 c, float h, float r, const float *x) {
+    const float ux = x[0] - c.x, uy = x[1] - c.y;
+    const float s = fmaxf(fabsf(c.z * ux + c.w * uy) - h, 0.f), l = fmaxf(fabsf(c.z * uy - c.w * ux) - r, 0.f);
+    return s * s + l * l;
+}
+__device__ __forceinline__ float cap_d2_3(float4 c, float4 a, const float *x) {
+    const float u[3] = {x[0] - c.x, x[1] - c.y, x[2] - c.z};
+    const float q = a.x * u[0] + a.y * u[1] + a.z * u[2];
+    const float n = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    // squared distance to the axis, less the rounding of n and q^2
+    const float w = fmaxf(n * (1.f - 2e-6f) - q * q, 1e-30f);
+    const float s = fmaxf(fabsf(q) - c.w, 0.f), l = fmaxf(w * rsqrtf(w) - a.w, 0.f);
+    return s * s + l * l;
 }
 
 // ---- primitive distances ----------------------------------------------------
@@ -298,6 +239,50 @@ __device__ __forceinline__ R tri_d2(const R *a, const R *b, const R *c, const R 
     return s;
 }
 
+// The FP32 distance of tri_d2, bit for bit, without its branches: the region
+// selects base point, edge and quotient, and one division serves all regions
+// (the lanes of a group test different triangles and fall into different
+// regions, so every branch of tri_d2 would run, most with a division).  A zero
+// weight leaves a coordinate as it is: fma(0, e, a) = a.
+__device__ __forceinline__ float tri_d2_fast(const float *a, const float *b, const float *c, const float *p) {
+    float ab[3], ac[3], ap[3], bp[3], cp[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) { ab[i] = b[i] - a[i]; ac[i] = c[i] - a[i]; ap[i] = p[i] - a[i]; bp[i] = p[i] - b[i]; cp[i] = p[i] - c[i]; }
+    auto dot = [](const float *u, const float *v) { return u[0] * v[0] + u[1] * v[1] + u[2] * v[2]; };
+    const float d1 = dot(ab, ap), d2 = dot(ac, ap);
+    const float d3 = dot(ab, bp), d4 = dot(ac, bp);
+    const float d5 = dot(ab, cp), d6 = dot(ac, cp);
+    const float vc = d1 * d4 - d3 * d2, vb = d5 * d2 - d1 * d6, va = d3 * d6 - d5 * d4;
+    const float e43 = d4 - d3, e56 = d5 - d6;
+    // the first of tri_d2's regions that holds: A, B, AB, C, AC, BC, face
+    const bool rA = d1 <= 0.f && d2 <= 0.f;
+    const bool rB = !rA && d3 >= 0.f && d4 <= d3;
+    const bool rAB = !rA && !rB && vc <= 0.f && d1 >= 0.f && d3 <= 0.f;
+    const bool n3 = rA || rB || rAB;
+    const bool rC = !n3 && d6 >= 0.f && d5 <= d6;
+    const bool rAC = !n3 && !rC && vb <= 0.f && d2 >= 0.f && d6 <= 0.f;
+    const bool n5 = n3 || rC || rAC;
+    const bool rBC = !n5 && va <= 0.f && e43 >= 0.f && e56 >= 0.f;
+    const bool face = !n5 && !rBC;
+    float num = 0.f, den = 1.f;
+    if (rAB) { num = d1; den = d1 - d3; }
+    if (rAC) { num = d2; den = d2 - d6; }
+    if (rBC) { num = e43; den = e43 + e56; }
+    if (face) { num = 1.f; den = va + vb + vc; }
+    const float t = num / den;
+    const float v = face ? vb * t : (rAC ? 0.f : t), w = face ? vc * t : (rAC ? t : 0.f);
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float base = rB || rBC ? b[i] : (rC ? c[i] : a[i]);
+        const float dir = rBC ? c[i] - b[i] : ab[i];
+        const float q = __fmaf_rn(w, ac[i], __fmaf_rn(v, dir, base));
+        const float d = p[i] - q;
+        s += d * d;
+    }
+    return s;
+}
+
 __device__ __forceinline__ void load_tri(const float4 *__restrict__ P, int s, float *a, float *b, float *c) {
     float4 u = ldn(P + 3 * s), v = ldn(P + 3 * s + 1), w = ldn(P + 3 * s + 2);
     a[0] = u.x; a[1] = u.y; a[2] = u.z; b[0] = u.w; b[1] = v.x; b[2] = v.y; c[0] = v.z; c[1] = v.w; c[2] = w.x;
@@ -320,11 +305,11 @@ __device__ __forceinline__ void load_tri(const float4 *__restrict__ P, int s, fl
         if (!found_) done = true;                              \
     } while (0)
 
-// ---- closest Dirichlet primitive -------------------------------------------
+// ---- closest Dirichlet primitive (2D) ---------------------------------------
 // returns the leaf slot of the closest primitive (-1 if none); best = squared distance
-template <int D>
-__device__ WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const float *x, float &best, int *err, Visits *vis = nullptr) {
-    constexpr int kBW = bvh_width(D);
+__device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const float4 *caps, const float *x, float &best,
+                                                         int *err, Visits *vis = nullptr) {
+    constexpr int kBW = 2;
     best = __int_as_float(0x7f800000);
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
@@ -341,26 +326,24 @@ __device__ WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const float *x,
             float k[kBW];
             int r[kBW];
             bool h[kBW];
-            node_keys_d2<D>(bv.nodes, ref, x, k, r);
+            const float4 *p = caps + cap_f4(2) * ref;
+            const float4 hr = ldn(p + 2), q = ldn(p + 3);
+            k[0] = cap_d2_2(ldn(p), hr.x, hr.y, x);
+            k[1] = cap_d2_2(ldn(p + 1), hr.z, hr.w, x);
+            r[0] = __float_as_int(q.x);
+            r[1] = __float_as_int(q.y);
             if (vis) vis->nodes++;
 #pragma unroll
-            for (int c = 0; c < kBW; ++c) h[c] = r[c] != kEmptyRef && k[c] <= best;
+            for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
             if (!take_children<kBW>(k, r, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, best);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
             if (vis) vis->dprims += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
-                float d2;
-                if (D == 2) {
-                    float4 p = ldn(bv.prims + s);
-                    float qx, qy;
-                    d2 = seg_d2<float>(p.x, p.y, p.z, p.w, x[0], x[1], qx, qy);
-                } else {
-                    float a[3], b[3], c[3], q[3];
-                    load_tri(bv.prims, s, a, b, c);
-                    d2 = tri_d2<float>(a, b, c, x, q);
-                }
+                float4 p = ldn(bv.prims + s);
+                float qx, qy;
+                const float d2 = seg_d2<float>(p.x, p.y, p.z, p.w, x[0], x[1], qx, qy);
                 if (d2 <= best) {
                     int id = __ldg(bv.ids + s);
                     if (d2 < best || id < best_id) { best = d2; best_slot = s; best_id = id; }
@@ -398,69 +381,81 @@ __device__ __forceinline__ bool sil_rule(float o0, float o1, float tau) {
     return (c0 == -1 && c1 >= 0) || (c1 == -1 && c0 >= 0);
 }
 
-// Normal-cone test of a silhouette-BVH child: no element below it can be a
-// silhouette from x when every normal in its cone (axis a, half-angle t) is
-// strictly front- or strictly back-facing from every point of its box.  With
-// c = x - (box centre), view half-angle p = asin(R / |c|) (R = box
-// half-diagonal), that holds when |a . c/|c|| > sin(t + p); the margin
-// tau / dist keeps every |o| above the edge-on tolerance.
-template <int D>
-__device__ __forceinline__ bool cone_prunes(float4 cone, const float *lo, const float *hi, const float *x,
-                                            float dist2, float tau) {
-    if (cone.w <= 0.f || dist2 <= 0.f) return false;
-    float c[3], r2 = 0.f, cl2 = 0.f, ac = 0.f;
-    const float ax[3] = {cone.x, cone.y, cone.z};
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        float h = 0.5f * (hi[k] - lo[k]);
-        c[k] = x[k] - 0.5f * (hi[k] + lo[k]);
-        r2 += h * h;
-        cl2 += c[k] * c[k];
-        ac += ax[k] * c[k];
-    }
-    if (cl2 <= r2) return false;
-    float inv = rsqrtf(cl2);
-    float sp = sqrtf(r2) * inv, cp = sqrtf(fmaxf(0.f, 1.f - sp * sp));
-    float ct = cone.w, st = sqrtf(fmaxf(0.f, 1.f - ct * ct));
-    if (ct * cp - st * sp <= 0.f) return false;          // t + p >= 90 degrees
-    float s_tp = st * cp + ct * sp;                      // sin(t + p)
-    return fabsf(ac) * inv > s_tp + 2.f * tau * rsqrtf(dist2) + 1e-6f;
+// Facing bound of a silhouette-BVH child: no element below it can be a
+// silhouette from x when all of its planes are seen from the front (no
+// o < -tau) or all from the back (every o < -tau).  Per child the host stores
+// a unit axis a, s = sin t of the largest angle t between a and the normals
+// below it, and the range [d0, d1] of a . (v - lo) over the planes' points v
+// (lo: the child box's lower corner).  With A = a . (x - lo) - d1 > 0 every v
+// has a . (x - v) >= A, so x sees v under an angle from a whose cosine is at
+// least A / L, L the distance from x to the far corner of the box, and a
+// normal within t of a faces x when A >= L s (from the back: d0 - a . (x - lo)
+// in place of A).  The slab [d0, d1] is what makes the bound sharp for the
+// flat patches of a mesh: x may stand closer to a patch than the patch is
+// wide.  A bound from the patch's bounding sphere and normal cone alone
+// leaves every patch within about sqrt(2 rho / curvature) of a point on the
+// boundary unpruned (rho the patch radius), this one those within a few rho.
+// Rounding: o in a leaf, A and L err by less than 6e-7 L together, which the
+// stored s carries (scene.cu, facing_bound); planes seen from the front may lie up to tau
+// behind x, of which half is used (tau / 2, cos t >= 0.6), and from the back
+// every o has to be below -tau.
+// Per node: 2D (2 children) a.x, a.y, d0, d1 of each child, then both s^2;
+// 3D (4 children) 4 x (a.xyz, d0), then 4 x (d1, s^2).
+__host__ __device__ constexpr int facing_f4(int d) { return d == 2 ? 3 : 6; }
+
+// q = a . (x - lo), far2 = squared distance to the far corner of the box
+__device__ __forceinline__ bool facing_prunes(float q, float d0, float d1, float s2, float far2, float tau) {
+    const float m = fmaxf(q - d1 + 0.5f * tau, d0 - q - 1.01f * tau);
+    return m > 0.f && m * m >= s2 * far2;
 }
 
+// One inner node of the 2D silhouette search: keys of the children (squared
+// distance to the box) and which of them can hold a silhouette within best.
+__device__ __forceinline__ void node_keys_sil(const float4 *nodes, const float4 *facing, int node, const float *x,
+                                              float best, float tau, float *k, int *r, bool *h) {
+    const float4 bx[2] = {ldn(nodes + 3 * node), ldn(nodes + 3 * node + 1)}, q = ldn(nodes + 3 * node + 2);
+    const float4 f[2] = {ldn(facing + 3 * node), ldn(facing + 3 * node + 1)}, s = ldn(facing + 3 * node + 2);
+    r[0] = __float_as_int(q.x);
+    r[1] = __float_as_int(q.y);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const float ux = bx[c].x - x[0], vx = x[0] - bx[c].z, uy = bx[c].y - x[1], vy = x[1] - bx[c].w;
+        const float dx = fmaxf(fmaxf(ux, vx), 0.f), dy = fmaxf(fmaxf(uy, vy), 0.f);
+        const float fx = fmaxf(fabsf(ux), fabsf(vx)), fy = fmaxf(fabsf(uy), fabsf(vy));
+        k[c] = dx * dx + dy * dy;
+        h[c] = k[c] <= best && !facing_prunes(-(f[c].x * ux + f[c].y * uy), f[c].z, f[c].w, c == 0 ? s.x : s.y,
+                                              fx * fx + fy * fy, tau);
+    }
+}
+
+// Silhouette element s: whether it is a silhouette from x within best, and
+// its squared distance.  The facing tests come first: most elements of a
+// smooth boundary fail them, and skip the edge distance and its division.
+// An element without two neighbours ("always") carries zero normals.
 template <int D>
-__device__ __forceinline__ void child_boxes(const float4 *nodes, int node, float *lo0, float *hi0,
-                                            float *lo1, float *hi1) {
+__device__ __forceinline__ bool sil_elem(const float4 *prims, int s, const float *x, float tau, float best, float &d2) {
     if (D == 2) {
-        const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1);
-        lo0[0] = a.x; lo0[1] = a.y; hi0[0] = a.z; hi0[1] = a.w;
-        lo1[0] = b.x; lo1[1] = b.y; hi1[0] = b.z; hi1[1] = b.w;
-    } else {
-        const float4 a = ldn(nodes + 4 * node), b = ldn(nodes + 4 * node + 1), c = ldn(nodes + 4 * node + 2);
-        lo0[0] = a.x; lo0[1] = a.y; lo0[2] = a.z; hi0[0] = a.w; hi0[1] = b.x; hi0[2] = b.y;
-        lo1[0] = b.z; lo1[1] = b.w; lo1[2] = c.x; hi1[0] = c.y; hi1[1] = c.z; hi1[2] = c.w;
+        float4 e0 = ldn(prims + 2 * s), e1 = ldn(prims + 2 * s + 1);
+        float rx = x[0] - e0.x, ry = x[1] - e0.y;
+        d2 = rx * rx + ry * ry;
+        const float o0 = e0.z * rx + e0.w * ry;
+        const float o1 = e1.x * rx + e1.y * ry;
+        return d2 <= best && (e1.z != 0.f || sil_rule(o0, o1, tau));
     }
+    const float4 e0 = ldn(prims + 3 * s), e1 = ldn(prims + 3 * s + 1), e2 = ldn(prims + 3 * s + 2);
+    const float a[3] = {e0.x, e0.y, e0.z}, b[3] = {e0.w, e1.x, e1.y};
+    const float r[3] = {x[0] - a[0], x[1] - a[1], x[2] - a[2]};
+    const float o0 = e1.z * r[0] + e1.w * r[1] + e2.x * r[2];
+    const float o1 = e2.y * r[0] + e2.z * r[1] + e2.w * r[2];
+    const bool always = e1.z == 0.f && e1.w == 0.f && e2.x == 0.f;
+    if (!(always || sil_rule(o0, o1, tau))) return false;
+    d2 = seg3_d2<float>(a, b, x);
+    return d2 <= best;
 }
 
-template <int D>
-__device__ __forceinline__ void node_child_box(const float4 *nodes, int node, int c, float *lo, float *hi) {
-    if (bvh_width(D) == 2) {
-        float lo1[3], hi1[3];
-        if (c == 0) child_boxes<D>(nodes, node, lo, hi, lo1, hi1);
-        else child_boxes<D>(nodes, node, lo1, hi1, lo, hi);
-        return;
-    }
-    const float *p = reinterpret_cast<const float *>(nodes + (size_t)node_f4<D>() * node);
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        lo[a] = p[4 * a + c];
-        hi[a] = p[4 * (D + a) + c];
-    }
-}
-
-template <int D>
-__device__ WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const float *x, float tau, float &best, int *err,
-                                   Visits *vis = nullptr, const float4 *cones = nullptr) {
-    constexpr int kBW = bvh_width(D);
+__device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const float *x, float tau, float &best, int *err,
+                                   const float4 *facing, Visits *vis = nullptr) {
+    constexpr int kBW = 2;
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
     int best_slot = -1, best_id = 0x7fffffff;
@@ -476,43 +471,16 @@ __device__ WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const float *x
             float k[kBW];
             int r[kBW];
             bool h[kBW];
-            node_keys_d2<D>(bv.nodes, ref, x, k, r);
+            node_keys_sil(bv.nodes, facing, ref, x, best, tau, k, r, h);
             if (vis) vis->nodes++;
-#pragma unroll
-            for (int c = 0; c < kBW; ++c) {
-                h[c] = r[c] != kEmptyRef && k[c] <= best;
-                if (cones && h[c]) {
-                    float lo[3], hi[3];
-                    node_child_box<D>(bv.nodes, ref, c, lo, hi);
-                    if (cone_prunes<D>(ldn(cones + kBW * ref + c), lo, hi, x, k[c], tau)) h[c] = false;
-                }
-            }
             if (!take_children<kBW>(k, r, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, best);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
             if (vis) vis->sprims += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
-                float d2, o0, o1;
-                bool always;
-                if (D == 2) {
-                    float4 e0 = ldn(bv.prims + 2 * s), e1 = ldn(bv.prims + 2 * s + 1);
-                    float rx = x[0] - e0.x, ry = x[1] - e0.y;
-                    d2 = rx * rx + ry * ry;
-                    o0 = e0.z * rx + e0.w * ry;
-                    o1 = e1.x * rx + e1.y * ry;
-                    always = e1.z != 0.f;
-                } else {
-                    float4 e0 = ldn(bv.prims + 4 * s), e1 = ldn(bv.prims + 4 * s + 1);
-                    float4 e2 = ldn(bv.prims + 4 * s + 2), e3 = ldn(bv.prims + 4 * s + 3);
-                    float a[3] = {e0.x, e0.y, e0.z}, b[3] = {e0.w, e1.x, e1.y};
-                    d2 = seg3_d2<float>(a, b, x);
-                    float r[3] = {x[0] - a[0], x[1] - a[1], x[2] - a[2]};
-                    o0 = e1.z * r[0] + e1.w * r[1] + e2.x * r[2];
-                    o1 = e2.y * r[0] + e2.z * r[1] + e2.w * r[2];
-                    always = e3.x != 0.f;
-                }
-                if (d2 <= best && (always || sil_rule(o0, o1, tau))) {
+                float d2;
+                if (sil_elem<2>(bv.prims, s, x, tau, best, d2)) {
                     int id = __ldg(bv.ids + s);
                     if (d2 < best || id < best_id) { best = d2; best_slot = s; best_id = id; }
                 }
@@ -627,16 +595,16 @@ __device__ __forceinline__ bool ray_prim64(const DevBVH &bv, int s, const float 
 
 // first Neumann hit with 0 < t <= tmax, skipping leaf slot `skip`; returns
 // slot or -1 (kExit: exit hits only, from t > -tneg, see ray_prim)
-template <int D, bool kExit = false>
+template <bool kExit = false>
 __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const float *v, float tmax, int skip, float &thit,
                            int *err, Visits *vis = nullptr, float tneg = 0.f) {
-    constexpr int kBW = bvh_width(D);
+    constexpr int kBW = 2;
     thit = tmax;
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
     float inv[3];
 #pragma unroll
-    for (int k = 0; k < D; ++k) inv[k] = 1.f / v[k];   // +-inf for a zero component is fine in the slab test
+    for (int k = 0; k < 2; ++k) inv[k] = 1.f / v[k];   // +-inf for a zero component is fine in the slab test
     float best = tmax;
     int best_slot = -1, best_id = 0x7fffffff;
     int stack[kStack];
@@ -651,10 +619,10 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
             float k[kBW];
             int r[kBW];
             bool h[kBW];
-            node_keys_ray<D>(bv.nodes, ref, o, inv, best, k, r, kExit ? tneg : 0.f);
+            node_keys_ray(bv.nodes, ref, o, inv, best, k, r, kExit ? tneg : 0.f);
             if (vis) vis->nodes++;
 #pragma unroll
-            for (int c = 0; c < kBW; ++c) h[c] = r[c] != kEmptyRef && k[c] <= best;
+            for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
             if (!take_children<kBW>(k, r, h, ref, stack, st, sp, err)) WOST_POP(stack, st, sp, ref, done, best);
         }
         if (!done && ref < 0) {
@@ -662,7 +630,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
             if (vis) vis->nprims += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 float t;
-                if (s != skip && ray_prim<D, kExit>(bv.prims, s, o, v, t, tneg) && t <= best) {
+                if (s != skip && ray_prim<2, kExit>(bv.prims, s, o, v, t, tneg) && t <= best) {
                     int id = __ldg(bv.ids + s);
                     if (t < best || id < best_id) { best = t; best_slot = s; best_id = id; }
                 }
@@ -685,7 +653,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
 template <int D>
 __device__ int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t pid, uint32_t wid, uint32_t step,
                             uint32_t k0, uint32_t k1, float &W, int *err, Visits *vis = nullptr) {
-    constexpr int kBW = bvh_width(D);
+    constexpr int kBW = lane_width(D);
     W = 0.f;
     if (bv.nprims == 0) return -1;
     const float r2 = r * r;
@@ -741,15 +709,14 @@ __device__ int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t 
     return best_slot;
 }
 
-// number of crossings of the ray o + t v (t > 0) with all primitives of a BVH
-template <int D>
-__device__ int ray_count(const DevBVH &bv, const float *o, const float *v, int *err) {
-    constexpr int kBW = bvh_width(D);
+// number of crossings of the ray o + t v (t > 0) with all primitives of a 2D BVH
+__device__ inline int ray_count(const DevBVH &bv, const float *o, const float *v, int *err) {
+    constexpr int kBW = 2;
     if (bv.nprims == 0) return 0;
     const unsigned mask = __activemask();
     float inv[3];
 #pragma unroll
-    for (int k = 0; k < D; ++k) inv[k] = 1.f / v[k];
+    for (int k = 0; k < 2; ++k) inv[k] = 1.f / v[k];
     const float big = 3.0e38f;
     int cnt = 0, stack[kStack], sp = 0, ref = 0;
     float skey[kStack];
@@ -761,15 +728,15 @@ __device__ int ray_count(const DevBVH &bv, const float *o, const float *v, int *
             float k[kBW];
             int r[kBW];
             bool h[kBW];
-            node_keys_ray<D>(bv.nodes, ref, o, inv, big, k, r, 0.f);
+            node_keys_ray(bv.nodes, ref, o, inv, big, k, r, 0.f);
 #pragma unroll
-            for (int c = 0; c < kBW; ++c) h[c] = r[c] != kEmptyRef && k[c] <= big;
+            for (int c = 0; c < kBW; ++c) h[c] = k[c] <= big;
             if (!take_children<kBW>(k, r, h, ref, stack, skey, sp, err)) pop = true;
         } else {
             int s0 = leaf_start(ref), c = leaf_count(ref);
             for (int s = s0; s < s0 + c; ++s) {
                 float t;
-                cnt += ray_prim<D>(bv.prims, s, o, v, t) ? 1 : 0;
+                cnt += ray_prim<2>(bv.prims, s, o, v, t) ? 1 : 0;
             }
             pop = true;
         }

@@ -11,6 +11,8 @@ namespace wost {
 
 constexpr int kGuidedBlock = 256;
 constexpr int kWsSmem = ws_smem_bytes(false);
+static_assert(kWsSmem % 16 == 0 && ws_smem_bytes(false, kMaxKWide) % 16 == 0 && sizeof(CoopWarp) % 16 == 0,
+              "query workspaces and staged scene data follow the tiles");
 // the 16-lobe kernel's tiles take this much more shared memory (weight image
 // and output region), which its scene staging gives up
 constexpr int kWsSmemWideExtra = ws_smem_bytes(false, kMaxKWide) - kWsSmem;
@@ -24,7 +26,7 @@ struct GuidedArgs {
 };
 
 // Walker warps of the single-scene kernel (exec walker_warps 0): kWsWalkerWarps
-// (16) when the scene's traversal data (BVH nodes, cones, primitives) fits
+// (16) when the scene's traversal data (BVH nodes, facing bounds, primitives) fits
 // comfortably in L2 or shared memory, kWsWalkersWide beside the 4 servers
 // when it does not.
 // Measured on one GB300, one recording round: genus-3 solid (about 300 MB of
@@ -46,19 +48,19 @@ __global__ void __launch_bounds__(ws_threads(W), 1) guided_walk_kernel(const __g
     __shared__ DevScene staged;
     const DevScene *sc = &g.w.sc;
     if (g.stage_mask) {
-        stage_scene(g.w.sc, staged, reinterpret_cast<float4 *>(sm + ws_smem_bytes(false, KM)), g.stage_mask);
+        stage_scene(g.w.sc, staged, reinterpret_cast<float4 *>(sm + ws_smem_bytes(false, KM) + coop_bytes(D, W)), g.stage_mask);
         sc = &staged;
     }
-    guided_ws_body<D, false, W, KM>(SoloSrc<D>{g.w, &g.f, g.rd, sc}, g.o, sm);
+    guided_ws_body<D, false, W, KM>(SoloSrc<D>{g.w, &g.f, g.rd, sc}, g.o, sm, sm + ws_smem_bytes(false, KM));
 }
 
 // bytes of the scene's traversal data (the three BVHs' nodes and primitives
-// and the silhouette cones)
+// and the silhouette facing bounds)
 static size_t traversal_bytes(const DevScene &s) {
     const size_t nb = 16 * (size_t)(s.dim == 2 ? node_f4<2>() : node_f4<3>());
-    const size_t pd = s.dim == 2 ? 16 : 48, ps = s.dim == 2 ? 32 : 64;
-    return nb * ((size_t)s.dir.nnodes + s.neu.nnodes + s.sil.nnodes) + pd * ((size_t)s.dir.nprims + s.neu.nprims) +
-           ps * (size_t)s.sil.nprims + 16 * (size_t)bvh_width(s.dim) * s.sil.nnodes;
+    const size_t pd = s.dim == 2 ? 16 : 48, ps = s.dim == 2 ? 32 : 48;
+    return nb * ((size_t)s.neu.nnodes + s.sil.nnodes) + 16 * (size_t)cap_f4(s.dim) * s.dir.nnodes + pd * ((size_t)s.dir.nprims + s.neu.nprims) +
+           ps * (size_t)s.sil.nprims + 16 * (size_t)facing_f4(s.dim) * s.sil.nnodes;
 }
 
 // the walker-warp count of a scene's guided launches of `walks` walks
@@ -212,25 +214,25 @@ wost_status guided_occupancy(int dim, int *per_sm) {
     });
 }
 
-// regions of the scene to stage, and their size in float4 (km: lobe
-// capacity of the launch's kernel)
-static int stage_mask_for(const DevScene &sc, int *f4, int km = kMaxK) {
-    const int budget = stage_budget_bytes() - (km == kMaxK ? 0 : kWsSmemWideExtra);
+// regions of the scene to stage, and their size in float4 (walkers, km:
+// walker warps and lobe capacity of the launch's kernel)
+static int stage_mask_for(const DevScene &sc, int *f4, int walkers, int km = kMaxK) {
+    const int budget = stage_budget_bytes() - (km == kMaxK ? 0 : kWsSmemWideExtra) - coop_bytes(sc.dim, walkers);
     return stage_plan(sc, std::max(budget, 0) / 16, f4);
 }
 
 wost_status launch_guided(int dim, const GuidedArgs &g, int grid, cudaStream_t st, int walkers, int km = kMaxK) {
     int f4 = 0;
-    stage_mask_for(g.w.sc, &f4, km);
+    stage_mask_for(g.w.sc, &f4, walkers, km);
     constexpr int tn = ws_threads(kWsWalkerWarps), tw = ws_threads(kWsWalkersWide);
     if (km != kMaxK) {
-        const int smem16 = ws_smem_bytes(false, kMaxKWide) + f4 * 16;
+        const int smem16 = ws_smem_bytes(false, kMaxKWide) + coop_bytes(dim, kWsWalkerWarps) + f4 * 16;
         if (dim == 2) guided_walk_kernel<2, kWsWalkerWarps, kMaxKWide><<<grid, tn, smem16, st>>>(g);
         else guided_walk_kernel<3, kWsWalkerWarps, kMaxKWide><<<grid, tn, smem16, st>>>(g);
         WOST_CUDA(cudaGetLastError());
         return WOST_OK;
     }
-    const int smem = kWsSmem + f4 * 16;
+    const int smem = kWsSmem + coop_bytes(dim, walkers) + f4 * 16;
     const bool wide = walkers == kWsWalkersWide;
     if (dim == 2 && wide) guided_walk_kernel<2, kWsWalkersWide><<<grid, tw, smem, st>>>(g);
     else if (dim == 2) guided_walk_kernel<2, kWsWalkerWarps><<<grid, tn, smem, st>>>(g);
@@ -334,10 +336,6 @@ wost_status guided_solve(wost_scene *s, wost_field *f, WalkArgs &a, int nwalks, 
     }
     GuidedArgs g{};
     g.f = f->dev();
-    {
-        int f4 = 0;
-        g.stage_mask = stage_mask_for(s->dev, &f4, f->km);
-    }
     g.o.c_mode = ex.c_mode;
     g.o.c_fixed = ex.c_fixed;
     g.o.reflect = ex.reflect;
@@ -426,6 +424,8 @@ wost_status guided_solve(wost_scene *s, wost_field *f, WalkArgs &a, int nwalks, 
         // the largest launch of the solve: a training batch, or one walk per point
         const int walkers = ws_walkers_for_field(s->dev, f, ex.walker_warps,
                                                  (unsigned long long)a.npoints * (unsigned long long)(rounds > 0 ? bwpp : 1));
+        int f4 = 0;
+        g.stage_mask = stage_mask_for(s->dev, &f4, walkers, f->km);
         if (rounds > 0) {
             size_t scratch = (size_t)grid * (walkers * 32) * (size_t)std::max(a.maxsteps, 1) * kRecFloats *
                              sizeof(float);

@@ -215,8 +215,9 @@ __device__ __forceinline__ void end_recorded_walk(const RecDest &rd, const float
 // data misses L2 take more walkers to hide its latency); KM: lobe capacity of
 // the decoded output layout (8, or 16 for fields of 9..16 lobes; single-scene
 // launches only)
+// coop: the walkers' query workspaces in shared memory (3D; one per warp)
 template <int D, bool kMulti, int W = kWsWalkerWarps, int KM = kMaxK, class Src>
-__device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, uint8_t *sm) {
+__device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, uint8_t *sm, uint8_t *coop) {
     static_assert(!kMulti || KM == kMaxK, "multi-scene launches decode 8-lobe layouts");
     constexpr int kThreads = ws_threads(W);
     constexpr int kSlots = ws_weight_slots(kMulti);
@@ -422,11 +423,20 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
         const int slot = blockIdx.x * (W * 32) + (tid - 32 * kWsServerWarps);
         float *scratch_row = o.scratch + (size_t)slot * o.scratch_steps * kRecFloats;
         const float area = D == 2 ? 2.f * WOST_PI : 4.f * WOST_PI;
+        CoopWarp *sh = reinterpret_cast<CoopWarp *>(coop) + (D == 3 ? warp - kWsServerWarps : 0);
         Walk<D> w;
+        if (D == 3) {   // lanes without a walk take part in the groups' queries
+            w.job = 0;
+            w.prim = -1;
+            w.k = 0;
+            for (int i = 0; i < D; ++i) w.x[i] = 0.f;
+        }
         bool active = false, exhausted = false, failed = false;
+        WorkCursor cursor;
         for (;;) {
             if (!active && !exhausted) {
-                unsigned long long item = warp_fetch_add(src.work_ctr(), true);
+                unsigned long long item = cursor.next<D>(src.work_ctr(), (warp - kWsServerWarps) * gridDim.x + blockIdx.x,
+                                                         W * gridDim.x, 32);
                 if (item >= src.total()) exhausted = true;
                 else if (src.start(w, item)) { active = true; nwalks++; }
             }
@@ -439,16 +449,15 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             // unused).  Otherwise the geometry runs first and only walks that
             // go on are decoded.
             auto geometry = [&]() {
-                if (active) {
-                    nsteps++;
-                    float gv;
-                    bool trunc = false;
-                    if (step_geometry<D>(w, src.env(w), r, S, gv, trunc, &vis)) {
-                        src.finish(w);
-                        if (o.record) end_recorded_walk(src.rec(w), scratch_row, w.k, gv);
-                        ntrunc += trunc;
-                        active = false;
-                    }
+                if (D == 2 && !active) return;
+                nsteps += active;
+                float gv;
+                bool trunc = false;
+                if (step_geometry<D, kMulti>(sh, w, src.env(w), active, r, S, gv, trunc, &vis)) {
+                    src.finish(w);
+                    if (o.record) end_recorded_walk(src.rec(w), scratch_row, w.k, gv);
+                    ntrunc += trunc;
+                    active = false;
                 }
             };
             if (!kOverlap) geometry();
@@ -474,7 +483,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             __syncwarp();
             const bool live = active;
             if (!ws_wait(&ctl->done[b][quarter], k & 1u, o.wait_ns)) { failed = true; break; }
-            float nu[D];
+            float nu[D] = {};
             bool zero_density = false;
             float wgt = 1.f, ptil = 0.f;
             if (live) {
@@ -525,9 +534,9 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
                         rr[2] = make_float4(n2, ptil, wgt * roulette_scale(src.env(w), w.k), S);
                     }
                     w.T *= wgt;
-                    step_move<D>(w, src.env(w), nu, r, &vis);
                 }
             }
+            step_move<D, kMulti>(sh, w, src.env(w), live && !zero_density, nu, r, &vis);
         }
         if (failed) atomicOr(o.err, 2);
         __syncwarp();

@@ -14,18 +14,7 @@
 // same problem solved alone.
 #pragma once
 #include "field.cuh"
-#include "lanewalk.cuh"
 #include "walkstep.cuh"
-
-// plain walks in 3D: 1 = per-lane query state machine (lanewalk.cuh), 0 =
-// one warp-synchronous query at a time (plain_loop below).  Measured on
-// one GB300 the state machine is 8-11% faster on the 3D workloads (82k and
-// 994k triangles) and 26% slower in 2D (4096 segments), where its larger
-// register footprint costs more occupancy than its convergence gains; both
-// give identical results.
-#ifndef WOST_PLAIN_LANES
-#define WOST_PLAIN_LANES 1
-#endif
 
 namespace wost {
 
@@ -51,6 +40,7 @@ struct SoloSrc {
 
     __device__ __forceinline__ unsigned long long *work_ctr() const { return a.work_ctr; }
     __device__ __forceinline__ unsigned long long total() const { return a.total; }
+    __device__ __forceinline__ unsigned lanes() const { return a.lanes; }
     __device__ __forceinline__ bool start(Walk<D> &w, unsigned long long item) const {
         if (a.order) {   // the same walk index, another point
             const unsigned long long p = item % (unsigned long long)a.npoints;
@@ -77,18 +67,19 @@ struct SoloSrc {
 // chain of dependent loads of BVH nodes and leaf primitives, so their
 // latency is the step's latency; a kernel with shared memory to spare keeps
 // as much of the data there as fits.  Regions, in the order they are taken:
-// the three BVHs' nodes, the silhouette normal cones, then the Dirichlet,
+// the three BVHs' nodes (of the Dirichlet BVH its caps), the silhouette facing
+// bounds, then the Dirichlet,
 // Neumann and silhouette primitives.
 constexpr int kStageRegions = 7;
 
 __host__ __device__ __forceinline__ void stage_regions(const DevScene &s, const float4 **src, int *cnt) {
     const int nb = s.dim == 2 ? node_f4<2>() : node_f4<3>();   // float4 per node
     const int pd = s.dim == 2 ? 1 : 3;       // per Dirichlet / Neumann primitive
-    const int ps = s.dim == 2 ? 2 : 4;       // per silhouette element
-    src[0] = s.dir.nodes; cnt[0] = s.dir.nnodes * nb;
+    const int ps = s.dim == 2 ? 2 : 3;       // per silhouette element
+    src[0] = s.dir_caps; cnt[0] = s.dir.nnodes * cap_f4(s.dim);
     src[1] = s.neu.nodes; cnt[1] = s.neu.nnodes * nb;
     src[2] = s.sil.nodes; cnt[2] = s.sil.nnodes * nb;
-    src[3] = s.sil_cones; cnt[3] = s.sil_cones ? bvh_width(s.dim) * s.sil.nnodes : 0;
+    src[3] = s.sil_facing; cnt[3] = s.sil_facing ? facing_f4(s.dim) * s.sil.nnodes : 0;
     src[4] = s.dir.prims; cnt[4] = s.dir.nprims * pd;
     src[5] = s.neu.prims; cnt[5] = s.neu.nprims * pd;
     src[6] = s.sil.prims; cnt[6] = s.sil.nprims * ps;
@@ -130,10 +121,10 @@ __device__ __forceinline__ void stage_scene(const DevScene &in, DevScene &out, f
     if (threadIdx.x == 0) {
         out = in;
         auto take = [&](int r) { return (mask >> r & 1) && cnt[r] > 0; };
-        if (take(0)) out.dir.nodes = start[0];
+        if (take(0)) out.dir_caps = start[0];
         if (take(1)) out.neu.nodes = start[1];
         if (take(2)) out.sil.nodes = start[2];
-        if (take(3)) out.sil_cones = start[3];
+        if (take(3)) out.sil_facing = start[3];
         if (take(4)) out.dir.prims = start[4];
         if (take(5)) out.neu.prims = start[5];
         if (take(6)) out.sil.prims = start[6];
@@ -199,6 +190,7 @@ struct BatchSrc {
 
     __device__ __forceinline__ unsigned long long *work_ctr() const { return b.work_ctr; }
     __device__ __forceinline__ unsigned long long total() const { return b.total; }
+    __device__ __forceinline__ unsigned lanes() const { return 32; }
     __device__ __forceinline__ bool start(Walk<D> &w, unsigned long long item) const {
         const int s = find_seg(b.segs, b.nseg, item);
         const DevSeg sg = b.segs[s];
@@ -231,39 +223,76 @@ struct BatchSrc {
     __device__ __forceinline__ const float *b3(int j) const { return b.jobs[j].f.b3; }
 };
 
+// Walks per warp of a plain 3D launch of `total` walks on `warps` warps.  A
+// warp has four to eight queries in flight at a time, so more walks than that
+// amortise the step logic, but a warp that is left with many long walks holds
+// up the end of the launch: half the lanes where the launch has fewer than two
+// walks per lane.  The Neumann term runs per lane and wants all of them.
+// Measured on one GB300, 16 / 32 lanes: genus-3 (27 walks per warp) 66 / 72
+// ms, icosphere (77 per warp) 83 / 79 ms, flux slab 26.7 / 23.5 ms.
+inline int plain_lanes(const DevScene &s, unsigned long long total, long long warps) {
+    return s.dim == 2 || s.has_flux || total >= 64ull * (unsigned long long)warps ? 32 : 16;
+}
+
+// A lane's next work item.  2D: warp-aggregated from the launch's counter, so
+// a warp starts on consecutive points.  3D: the launch's first items go round
+// the warps (warp w's lane l takes item l * warps + w, `lanes` lanes of a warp
+// hold walks; the counter counts the items after those): long walks come in
+// runs of neighbouring points, or first where the launch is ordered, and a
+// warp that held a run of them would outlast all others.
+struct WorkCursor {
+    bool first = true;
+    template <int D>
+    __device__ __forceinline__ unsigned long long next(unsigned long long *ctr, unsigned warp, unsigned warps,
+                                                       unsigned lanes) {
+        if (D == 2) return warp_fetch_add(ctr, true);
+        if (first) {
+            first = false;
+            return (unsigned long long)(threadIdx.x & 31) * warps + warp;
+        }
+        return (unsigned long long)lanes * warps + warp_fetch_add(ctr, true);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // The plain persistent walk loop (uniform directions, Sec. 3.2).
 // Every lane of a warp stays in the loop until the whole warp is out of
 // work, and one loop iteration is one step of every active lane: lanes
 // cannot drift into different phases of the step, so the warp re-converges
-// after each query (a lane without a walk is predicated off).
+// after each query (2D: a lane without a walk is predicated off; 3D: it takes
+// part in the queries of the others, coop.cuh).
 // ---------------------------------------------------------------------------
-template <int D, class Src>
-__device__ __forceinline__ void plain_loop(const Src &src, unsigned long long *stat) {
-    if (WOST_PLAIN_LANES && D == 3) {
-        plain_loop_lanes<D>(src, stat);
-        return;
-    }
+template <int D, bool kMulti, class Src>
+__device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigned long long *stat) {
     Walk<D> w;
     Visits vis;
     bool active = false, exhausted = false;
     unsigned long long nsteps = 0, ntrunc = 0, nwalks = 0;
+    if (D == 3) {   // lanes without a walk take part in the groups' queries
+        w.job = 0;
+        w.prim = -1;
+        w.k = 0;
+        for (int i = 0; i < D; ++i) w.x[i] = 0.f;
+        exhausted = (threadIdx.x & 31) >= src.lanes();
+    }
+    WorkCursor cursor;
+    const unsigned warps = gridDim.x * (blockDim.x / 32), warp = (threadIdx.x / 32) * gridDim.x + blockIdx.x;
     for (;;) {
         if (!active && !exhausted) {
-            unsigned long long item = warp_fetch_add(src.work_ctr(), true);
+            unsigned long long item = cursor.next<D>(src.work_ctr(), warp, warps, src.lanes());
             if (item >= src.total()) exhausted = true;
             else if (src.start(w, item)) { active = true; nwalks++; }
         }
         if (!__any_sync(0xffffffffu, active || !exhausted)) break;
         __syncwarp();
-        if (!active) continue;
-        nsteps++;
+        if (D == 2 ? !active : !__any_sync(0xffffffffu, active)) continue;
+        nsteps += active;
         const StepEnv env = src.env(w);
-        float r, S, gv;
+        float r = 0.f, S, gv;
         bool trunc = false;
-        bool ended = step_geometry<D>(w, env, r, S, gv, trunc, &vis);
-        float nu[D];
-        if (!ended) {
+        bool ended = step_geometry<D, kMulti>(sh, w, env, active, r, S, gv, trunc, &vis);
+        float nu[D] = {};
+        if (active && !ended) {
             U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_DIR, env.key0, env.key1);
             uniform_dir<D>(u01(u.x), u01(u.y), nu);
             if (w.prim >= 0) {
@@ -272,13 +301,12 @@ __device__ __forceinline__ void plain_loop(const Src &src, unsigned long long *s
                 ended = dn == 0.f;   // zero density at the tangent plane (Eq. angular_req)
             }
         }
-        if (ended) {
+        if (active && ended) {
             src.finish(w);
             ntrunc += trunc;
             active = false;
-        } else {
-            step_move<D>(w, env, nu, r, &vis);
         }
+        step_move<D, kMulti>(sh, w, env, active, nu, r, &vis);
     }
     flush_stats(stat, nsteps, ntrunc, nwalks, vis);
 }

@@ -74,18 +74,20 @@ wost_status static_base(unsigned char **out) {
 }
 
 template <int D>
-__global__ void static_classify_kernel(WalkArgs a, double *shell_value) {
+__global__ void __launch_bounds__(128) static_classify_kernel(WalkArgs a, double *shell_value) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.npoints) return;
+    const bool act = i < a.npoints;
     double val;
-    const_cast<uint8_t *>(a.status)[i] = classify_point<D>(a.sc, a.eps64, a.points + i * D, a.err, val);
+    const uint8_t st = classify_point<D, false>(coop_shared<D, 4>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
+    if (!act) return;
+    const_cast<uint8_t *>(a.status)[i] = st;
     shell_value[i] = val;
 }
 
 // the plain persistent walk loop, on the static scratch
 template <int D>
 __global__ void __launch_bounds__(128) static_walk_kernel(const __grid_constant__ WalkArgs a) {
-    plain_loop<D>(SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
+    plain_loop<D, false>(coop_shared<D, 4>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
 }
 
 __global__ void static_finalize_kernel(const uint8_t *status, const double *shell_value, const double *sum,
@@ -148,6 +150,7 @@ extern "C" wost_status wost_solve_plain_static(wost_scene *s, const double *poin
     a.err = v.err;
     const int blocks = (int)((npoints + 127) / 128);
     const int grid = num_sms() * 8;
+    a.lanes = plain_lanes(s->dev, a.total, grid * 4);
     if (D == 2) {
         static_classify_kernel<2><<<blocks, 128, 0, st>>>(a, v.shell);
         static_walk_kernel<2><<<grid, 128, 0, st>>>(a);

@@ -7,19 +7,21 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <atomic>
 #include <numeric>
+#include <system_error>
+#include <thread>
 
-#include "geom.cuh"
+#include "coop.cuh"
 #include "internal.h"
 
 namespace wost {
 
 namespace {
 
-#ifndef WOST_BVH_LEAF
-#define WOST_BVH_LEAF 16
-#endif
-constexpr int kLeaf = WOST_BVH_LEAF;   // primitives per leaf (<= 16)
+// primitives per leaf (<= 16), and per leaf of the caps of a 3D scene (one
+// per lane of a query group)
+constexpr int kLeaf = 16, kLeafCaps = 8;
 constexpr int kBins = 16;
 constexpr int kSahDepth = 40;   // beyond this depth, median splits bound the tree depth
 
@@ -43,37 +45,139 @@ struct Item {
     Box b;
     float c[3];
     int idx;
-    // silhouette elements: inward normals of the two adjacent Neumann
-    // primitives; cone_free marks elements that are always silhouettes
-    float n0[3] = {0, 0, 0}, n1[3] = {0, 0, 0};
-    bool cone_free = false;
 };
 
-// Bounding cone (unit axis, cos of the half-angle) of the normals of items
-// [b, e); cos < 0 (half-angle beyond 90 degrees or an always-silhouette
-// element inside) disables pruning for that child.
-static float4 normal_cone(const std::vector<Item> &items, int b, int e, int d) {
+// silhouette element: inward normals of the two adjacent Neumann primitives
+// and the vertex both planes are taken through; free marks elements that are
+// always silhouettes
+struct SilData {
+    float n0[3] = {0, 0, 0}, n1[3] = {0, 0, 0}, v[3] = {0, 0, 0};
+    bool free = false;
+};
+
+// Facing bound of elements [b, e) relative to the box corner lo (geom.cuh,
+// facing_prunes): axis a (rounded to FP32), slab [d0, d1] of a . (v - lo) over
+// the planes' points v, and s^2, s the sine of the largest angle between a
+// and a normal (a normal of length 1 within FP32 rounding: |n x a|^2 is its
+// sine squared within 1e-6).  s^2 = infinity disables pruning: an
+// always-silhouette element inside, a degenerate normal, or normals spread
+// over more than a half space.
+struct Facing { float a[3] = {0, 0, 0}, d0 = 0, d1 = 0, s2 = INFINITY; };
+
+Facing facing_bound(const std::vector<SilData> &el, int b, int e, int d, const float *lo, double tau) {
+    const Facing off;
     double ax[3] = {0, 0, 0};
     for (int i = b; i < e; ++i) {
-        if (items[i].cone_free) return make_float4(0.f, 0.f, 0.f, -2.f);
-        for (int k = 0; k < d; ++k) ax[k] += items[i].n0[k] + items[i].n1[k];
+        if (el[i].free) return off;
+        for (int k = 0; k < d; ++k) ax[k] += el[i].n0[k] + el[i].n1[k];
     }
     double L = 0;
     for (int k = 0; k < d; ++k) L += ax[k] * ax[k];
     L = std::sqrt(L);
-    if (L < 1e-12) return make_float4(0.f, 0.f, 0.f, -2.f);
-    for (int k = 0; k < d; ++k) ax[k] /= L;
-    double cmin = 1.0;
-    for (int i = b; i < e; ++i)
-        for (const float *n : {items[i].n0, items[i].n1}) {
+    if (!(L > 1e-12)) return off;
+    Facing f;
+    for (int k = 0; k < d; ++k) { f.a[k] = (float)(ax[k] / L); ax[k] = f.a[k]; }
+    double s2 = 0, d0 = INFINITY, d1 = -INFINITY;
+    for (int i = b; i < e; ++i) {
+        for (const float *n : {el[i].n0, el[i].n1}) {
             double c = 0;
             for (int k = 0; k < d; ++k) c += ax[k] * n[k];
-            cmin = std::min(cmin, c);
+            if (!(c > 0)) return off;
+            const double x = n[1] * ax[2] - n[2] * ax[1], y = n[2] * ax[0] - n[0] * ax[2], z = n[0] * ax[1] - n[1] * ax[0];
+            s2 = std::max(s2, x * x + y * y + z * z);
         }
-    // shrink slightly so that FP32 rounding of the normals stays inside
-    cmin -= 1e-6;
-    if (cmin <= 0) return make_float4(0.f, 0.f, 0.f, -2.f);
-    return make_float4((float)ax[0], (float)ax[1], (float)ax[2], (float)cmin);
+        double h = 0;
+        for (int k = 0; k < d; ++k) h += ax[k] * ((double)el[i].v[k] - lo[k]);
+        d0 = std::min(d0, h);
+        d1 = std::max(d1, h);
+    }
+    // half of tau is used only while cos t >= 0.6; the rounding of o, A and L
+    // (below 6e-7 L together) goes into s
+    if (!(s2 < 0.64)) d1 += 0.5 * tau;
+    const double s = std::sqrt(s2) * (1 + 2e-6) + 1e-6;
+    f.d0 = std::nextafterf((float)d0, -INFINITY);
+    f.d1 = std::nextafterf((float)d1, INFINITY);
+    f.s2 = std::nextafterf((float)(s * s * (1 + 2e-6)), INFINITY);
+    return f;
+}
+
+// Oriented cap around primitives [b, e) (geom.cuh, cap_d2): centre c, axis a,
+// half thickness h along a, radius r across it.  The axis is the mean normal
+// (any axis bounds, that one is thin).  P: vertices in leaf order (d points
+// of d floats per primitive), N: unit normals.  margin: see cap_d2.
+struct Cap { float c[3] = {0, 0, 0}, a[3] = {1, 0, 0}, h = 0, r = 0; };
+
+Cap cap_of(const std::vector<float> &P, const std::vector<float> &N, int b, int e, int d, double margin) {
+    Cap o;
+    double ax[3] = {0, 0, 0}, lo[3], hi[3], L = 0;
+    for (int i = b; i < e; ++i)
+        for (int k = 0; k < d; ++k) ax[k] += N[(size_t)i * d + k];
+    for (int k = 0; k < d; ++k) L += ax[k] * ax[k];
+    L = std::sqrt(L);
+    if (L > 1e-3 * (e - b))
+        for (int k = 0; k < d; ++k) o.a[k] = (float)(ax[k] / L);
+    // frame: the axis and (2D) its perpendicular, or (3D) two axes across
+    double f[3][3] = {{o.a[0], o.a[1], o.a[2]}, {-o.a[1], o.a[0], 0}, {0, 0, 0}};
+    if (d == 3) {
+        const int m = std::fabs(f[0][0]) < std::fabs(f[0][1]) ? (std::fabs(f[0][0]) < std::fabs(f[0][2]) ? 0 : 2)
+                                                              : (std::fabs(f[0][1]) < std::fabs(f[0][2]) ? 1 : 2);
+        double t[3] = {0, 0, 0}, q = f[0][m], n = 0;
+        t[m] = 1;
+        for (int k = 0; k < 3; ++k) { t[k] -= q * f[0][k]; n += t[k] * t[k]; }
+        for (int k = 0; k < 3; ++k) f[1][k] = t[k] / std::sqrt(n);
+        f[2][0] = f[0][1] * f[1][2] - f[0][2] * f[1][1];
+        f[2][1] = f[0][2] * f[1][0] - f[0][0] * f[1][2];
+        f[2][2] = f[0][0] * f[1][1] - f[0][1] * f[1][0];
+    }
+    for (int j = 0; j < d; ++j) { lo[j] = INFINITY; hi[j] = -INFINITY; }
+    const size_t p0 = (size_t)b * d * d, p1 = (size_t)e * d * d;
+    for (size_t p = p0; p < p1; p += d)
+        for (int j = 0; j < d; ++j) {
+            double q = 0;
+            for (int k = 0; k < d; ++k) q += f[j][k] * P[p + k];
+            lo[j] = std::min(lo[j], q);
+            hi[j] = std::max(hi[j], q);
+        }
+    for (int k = 0; k < d; ++k) {
+        double c = 0;
+        for (int j = 0; j < d; ++j) c += 0.5 * (lo[j] + hi[j]) * f[j][k];
+        o.c[k] = (float)c;
+    }
+    double h = 0, r2 = 0;
+    for (size_t p = p0; p < p1; p += d) {
+        double q = 0, n = 0;
+        for (int k = 0; k < d; ++k) { const double u = P[p + k] - (double)o.c[k]; q += f[0][k] * u; n += u * u; }
+        h = std::max(h, std::fabs(q));
+        r2 = std::max(r2, n - q * q);
+    }
+    o.h = std::nextafterf((float)(h + margin), INFINITY);
+    o.r = std::nextafterf((float)(std::sqrt(r2) * (1 + 1e-6) + margin), INFINITY);
+    return o;
+}
+
+// fn(i) for i in [0, n), split over the host's cores
+template <class F>
+void parallel_for(int n, F fn) {
+    const int nt = (int)std::min<int64_t>(std::min<unsigned>(std::max(1u, std::thread::hardware_concurrency()), 16u), n / 64);
+    if (nt <= 1) {
+        for (int i = 0; i < n; ++i) fn(i);
+        return;
+    }
+    std::atomic<int> next{0};
+    auto work = [&] {
+        for (int i; (i = next.fetch_add(16)) < n;)
+            for (int j = i; j < std::min(n, i + 16); ++j) fn(j);
+    };
+    std::vector<std::thread> th;
+    for (int t = 1; t < nt; ++t) {
+        try {
+            th.emplace_back(work);
+        } catch (const std::system_error &) {
+            break;   // no more threads to be had: those there are do the work
+        }
+    }
+    work();
+    for (std::thread &t : th) t.join();
 }
 
 struct BNode {
@@ -84,6 +188,7 @@ struct BNode {
 
 struct Builder {
     int d;
+    int leaf = kLeaf;   // the tree is split down to this (<= kLeaf)
     std::vector<Item> items;
     std::vector<BNode> nodes;
     int maxdepth = 0;
@@ -105,10 +210,11 @@ struct Builder {
         return m;
     }
 
-    int rec(int b, int e, int depth) {
-        maxdepth = std::max(maxdepth, depth);
+    int rec(int b, int e, int depth, bool within_leaf = false) {
+        // (splits below kLeaf primitives do not count: the box tree has none)
+        if (!within_leaf) maxdepth = std::max(maxdepth, depth);
         int n = e - b;
-        if (n <= kLeaf) return leaf_ref(b, n);
+        if (n <= leaf) return leaf_ref(b, n);
         Box cb;
         for (int i = b; i < e; ++i) cb.grow(items[i].c, d);
         int axis = 0;
@@ -150,8 +256,8 @@ struct Builder {
         }
         int node = (int)nodes.size();
         nodes.push_back(BNode{});
-        int l = rec(b, mid, depth + 1);
-        int r = rec(mid, e, depth + 1);
+        int l = rec(b, mid, depth + 1, n <= kLeaf);
+        int r = rec(mid, e, depth + 1, n <= kLeaf);
         nodes[node].ref[0] = l;
         nodes[node].ref[1] = r;
         nodes[node].box[0] = range_box(b, mid);
@@ -166,7 +272,7 @@ struct Builder {
         nodes.clear();
         int n = (int)items.size();
         if (n == 0) return true;
-        if (n <= kLeaf) {
+        if (n <= leaf) {
             BNode r;
             r.ref[0] = leaf_ref(0, n);
             r.ref[1] = leaf_ref(0, 1);
@@ -182,116 +288,162 @@ struct Builder {
     }
 
     // ---- device layout ----
-    // Width 2: the binary nodes, child boxes in the parent.  Width 4: each
-    // node takes up to four descendants of a binary node (its children, with
-    // the inner child of the larger box surface opened until there are
-    // four); empty slots carry kEmptyRef and an inverted box.
-    struct Child { Box box; int ref; int range[2]; };
-    struct WNode { Child ch[4]; int n; };
-    std::vector<WNode> wide;
-    int wdepth = 0;
+    // Wide nodes: each takes up to W descendants of a binary node (its
+    // children, with the inner child of the larger box surface opened until
+    // there are W); empty slots carry kEmptyRef and an inverted box.
+    struct Child { Box box; int ref = kEmptyRef; int range[2] = {0, 0}; };
+    struct WNode { Child ch[8]; int n = 0; };
 
-    int collapse(int bnode, int depth) {
-        wdepth = std::max(wdepth, depth);
-        Child ch[4];
+    // (leaves of at most `lf` primitives)
+    int collapse(std::vector<WNode> &out, int W, int lf, int bnode) const {
+        Child ch[8];
         int n = 0;
-        for (int c = 0; c < 2; ++c)
-            ch[n++] = Child{nodes[bnode].box[c], nodes[bnode].ref[c], {nodes[bnode].range[c][0], nodes[bnode].range[c][1]}};
-        while (n < 4) {
+        auto child = [&](int b, int c) {
+            Child x;
+            x.box = nodes[b].box[c];
+            x.ref = nodes[b].ref[c];
+            x.range[0] = nodes[b].range[c][0];
+            x.range[1] = nodes[b].range[c][1];
+            if (x.ref >= 0 && x.range[1] - x.range[0] <= lf) x.ref = leaf_ref(x.range[0], x.range[1] - x.range[0]);
+            return x;
+        };
+        for (int c = 0; c < 2; ++c) ch[n++] = child(bnode, c);
+        while (n < W) {
             int pick = -1;
             float area = -1.f;
             for (int i = 0; i < n; ++i)
                 if (ch[i].ref >= 0 && ch[i].box.cost(d) > area) { pick = i; area = ch[i].box.cost(d); }
             if (pick < 0) break;
-            const BNode &b = nodes[ch[pick].ref];
-            Child c0{b.box[0], b.ref[0], {b.range[0][0], b.range[0][1]}};
-            Child c1{b.box[1], b.ref[1], {b.range[1][0], b.range[1][1]}};
-            ch[pick] = c0;
-            ch[n++] = c1;
+            const int b = ch[pick].ref;
+            ch[pick] = child(b, 0);
+            ch[n++] = child(b, 1);
         }
-        const int id = (int)wide.size();
-        wide.push_back(WNode{});
-        for (int i = 0; i < 4; ++i) {
-            Child c;
-            if (i < n) {
-                c = ch[i];
-                if (c.ref >= 0) c.ref = collapse(c.ref, depth + 1);
-            } else {
-                c = Child{Box{}, kEmptyRef, {0, 0}};
-            }
-            wide[id].ch[i] = c;
+        const int id = (int)out.size();
+        out.push_back(WNode{});
+        for (int i = 0; i < n; ++i) {
+            Child c = ch[i];
+            if (c.ref >= 0) c.ref = collapse(out, W, lf, c.ref);
+            else if (c.range[1] <= c.range[0]) c.ref = kEmptyRef;   // the unused child of a one-leaf tree
+            out[id].ch[i] = c;
         }
-        wide[id].n = n;
+        out[id].n = n;
         return id;
     }
 
     // most stack entries a traversal below wide node id can hold: a visit
     // pushes all but one of its taken children
-    int stack_need(int id) const {
+    static int stack_need(const std::vector<WNode> &w, int id) {
         int need = 0;
-        for (int c = 0; c < 4; ++c)
-            if (wide[id].ch[c].ref >= 0) need = std::max(need, stack_need(wide[id].ch[c].ref));
-        return need + std::max(wide[id].n - 1, 0);
+        for (int c = 0; c < w[id].n; ++c)
+            if (w[id].ch[c].ref >= 0) need = std::max(need, stack_need(w, w[id].ch[c].ref));
+        return need + std::max(w[id].n - 1, 0);
     }
 
-    // builds the wide tree (width 4); false if a traversal could overflow
-    // the device stack
-    bool widen() {
-        wide.clear();
-        wdepth = 0;
-        if (bvh_width(d) == 2 || nodes.empty()) return true;
-        collapse(0, 1);
-        return stack_need(0) < kStack;
+    // wide tree of at most W children per node and lf primitives per leaf
+    std::vector<WNode> widen(int W, int lf) const {
+        std::vector<WNode> out;
+        if (!nodes.empty()) collapse(out, W, lf, 0);
+        return out;
     }
 
-    int device_nodes() const { return bvh_width(d) == 2 ? (int)nodes.size() : (int)wide.size(); }
+    // a traversal's entries fit the device stack
+    static bool fits(const std::vector<WNode> &w) { return w.empty() || stack_need(w, 0) < kGrpStack; }
 
-    // one cone per child
-    std::vector<float4> cones() const {
+    static float bits(int r) { float f; std::memcpy(&f, &r, 4); return f; }
+
+    // 3D nodes (geom.cuh)
+    static std::vector<float4> pack_wide(const std::vector<WNode> &w) {
         std::vector<float4> out;
-        auto cone = [&](int b, int e) {
-            return e > b ? normal_cone(items, b, e, d) : make_float4(0.f, 0.f, 0.f, -2.f);
-        };
-        if (bvh_width(d) == 2) {
-            for (const BNode &nd : nodes)
-                for (int c = 0; c < 2; ++c) out.push_back(cone(nd.range[c][0], nd.range[c][1]));
-        } else {
-            for (const WNode &wn : wide)
-                for (int c = 0; c < 4; ++c) out.push_back(cone(wn.ch[c].range[0], wn.ch[c].range[1]));
+        out.reserve(w.size() * node_f4<3>());
+        for (const WNode &n : w) {
+            for (int c = 0; c < 4; ++c) {
+                const Box &b = n.ch[c].box;
+                out.push_back(make_float4(b.lo[0], b.lo[1], b.lo[2], b.hi[0]));
+            }
+            for (int c = 0; c < 4; ++c) {
+                const Box &b = n.ch[c].box;
+                out.push_back(make_float4(b.hi[1], b.hi[2], bits(n.ch[c].ref), 0.f));
+            }
         }
         return out;
     }
 
-    std::vector<float4> pack() const {
+    // binary 2D nodes, child boxes in the parent
+    std::vector<float4> pack_binary() const {
         std::vector<float4> out;
-        auto bits = [](int r) { float f; std::memcpy(&f, &r, 4); return f; };
-        if (bvh_width(d) == 4) {
-            // one coordinate of the four children per float4: lo x, lo y, (lo z,) hi x, hi y, (hi z,) refs
-            for (const WNode &wn : wide) {
-                for (int side = 0; side < 2; ++side)
-                    for (int a = 0; a < d; ++a) {
-                        float v[4];
-                        for (int c = 0; c < 4; ++c) v[c] = side == 0 ? wn.ch[c].box.lo[a] : wn.ch[c].box.hi[a];
-                        out.push_back(make_float4(v[0], v[1], v[2], v[3]));
-                    }
-                out.push_back(make_float4(bits(wn.ch[0].ref), bits(wn.ch[1].ref), bits(wn.ch[2].ref), bits(wn.ch[3].ref)));
-            }
-            return out;
-        }
         for (const BNode &nd : nodes) {
             const Box &a = nd.box[0], &b = nd.box[1];
-            float r0 = bits(nd.ref[0]), r1 = bits(nd.ref[1]);
-            if (d == 2) {
-                out.push_back(make_float4(a.lo[0], a.lo[1], a.hi[0], a.hi[1]));
-                out.push_back(make_float4(b.lo[0], b.lo[1], b.hi[0], b.hi[1]));
-                out.push_back(make_float4(r0, r1, 0.f, 0.f));
-            } else {
-                out.push_back(make_float4(a.lo[0], a.lo[1], a.lo[2], a.hi[0]));
-                out.push_back(make_float4(a.hi[1], a.hi[2], b.lo[0], b.lo[1]));
-                out.push_back(make_float4(b.lo[2], b.hi[0], b.hi[1], b.hi[2]));
-                out.push_back(make_float4(r0, r1, 0.f, 0.f));
-            }
+            out.push_back(make_float4(a.lo[0], a.lo[1], a.hi[0], a.hi[1]));
+            out.push_back(make_float4(b.lo[0], b.lo[1], b.hi[0], b.hi[1]));
+            out.push_back(make_float4(bits(nd.ref[0]), bits(nd.ref[1]), 0.f, 0.f));
         }
+        return out;
+    }
+
+    // facing bounds of every node's children (layout: facing_f4, geom.cuh)
+    static Facing facing_of(const std::vector<SilData> &el, const int *r, int d, const Box &bx, double tau) {
+        return r[1] > r[0] ? facing_bound(el, r[0], r[1], d, bx.lo, tau) : Facing{};
+    }
+    std::vector<float4> facing_binary(const std::vector<SilData> &el, double tau) const {
+        std::vector<float4> out(nodes.size() * facing_f4(2));
+        parallel_for((int)nodes.size(), [&](int i) {
+            const BNode &nd = nodes[i];
+            float4 *o = &out[(size_t)i * facing_f4(2)];
+            Facing f[2];
+            for (int c = 0; c < 2; ++c) {
+                f[c] = facing_of(el, nd.range[c], d, nd.box[c], tau);
+                o[c] = make_float4(f[c].a[0], f[c].a[1], f[c].d0, f[c].d1);
+            }
+            o[2] = make_float4(f[0].s2, f[1].s2, 0.f, 0.f);
+        });
+        return out;
+    }
+    static std::vector<float4> facing_wide(const std::vector<SilData> &el, const std::vector<WNode> &w, double tau) {
+        std::vector<float4> out(w.size() * facing_f4(3));
+        parallel_for((int)w.size(), [&](int i) {
+            float4 *o = &out[(size_t)i * facing_f4(3)];
+            Facing f[4];
+            for (int c = 0; c < 4; ++c) {
+                f[c] = facing_of(el, w[i].ch[c].range, 3, w[i].ch[c].box, tau);
+                o[c] = make_float4(f[c].a[0], f[c].a[1], f[c].a[2], f[c].d0);
+            }
+            for (int c = 0; c < 4; c += 2) o[4 + c / 2] = make_float4(f[c].d1, f[c].s2, f[c + 1].d1, f[c + 1].s2);
+        });
+        return out;
+    }
+
+    // caps of every node's children, with the child references (layout:
+    // cap_f4, geom.cuh); P, N as cap_of
+    std::vector<float4> caps_binary(const std::vector<float> &P, const std::vector<float> &N, double margin) const {
+        std::vector<float4> out(nodes.size() * cap_f4(2));
+        parallel_for((int)nodes.size(), [&](int i) {
+            const BNode &nd = nodes[i];
+            float4 *o = &out[(size_t)i * cap_f4(2)];
+            Cap c[2];
+            for (int k = 0; k < 2; ++k) {
+                if (nd.range[k][1] > nd.range[k][0]) c[k] = cap_of(P, N, nd.range[k][0], nd.range[k][1], 2, margin);
+                else c[k].c[0] = 1e30f;   // the unused child of a one-leaf tree: far away
+                o[k] = make_float4(c[k].c[0], c[k].c[1], c[k].a[0], c[k].a[1]);
+            }
+            o[2] = make_float4(c[0].h, c[0].r, c[1].h, c[1].r);
+            o[3] = make_float4(bits(nd.ref[0]), bits(nd.ref[1]), 0.f, 0.f);
+        });
+        return out;
+    }
+    static std::vector<float4> caps_wide(const std::vector<WNode> &w, const std::vector<float> &P,
+                                          const std::vector<float> &N, double margin) {
+        std::vector<float4> out(w.size() * cap_f4(3));
+        parallel_for((int)w.size(), [&](int i) {
+            float4 *o = &out[(size_t)i * cap_f4(3)];
+            const Child *ch = w[i].ch;
+            for (int k = 0; k < 8; ++k) {
+                const Cap c = ch[k].range[1] > ch[k].range[0] ? cap_of(P, N, ch[k].range[0], ch[k].range[1], 3, margin) : Cap{};
+                o[k] = make_float4(c.c[0], c.c[1], c.c[2], c.h);
+                o[8 + k] = make_float4(c.a[0], c.a[1], c.a[2], c.r);
+            }
+            for (int k = 0; k < 8; k += 4)
+                o[16 + k / 4] = make_float4(bits(ch[k].ref), bits(ch[k + 1].ref), bits(ch[k + 2].ref), bits(ch[k + 3].ref));
+        });
         return out;
     }
 };
@@ -411,6 +563,8 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
     auto build_prims = [&](int bcv, DevBVH &bv, int &count, int &depth, std::vector<int> *slot_of) -> wost_status {
         Builder B;
         B.d = d;
+        // (the caps' smaller leaves subdivide those of the boxes)
+        B.leaf = d == 3 && bcv == 0 ? kLeafCaps : kLeaf;
         for (int64_t i = 0; i < np; ++i) {
             if (desc->bc[i] != bcv) continue;
             Item it;
@@ -425,7 +579,20 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
             B.items.push_back(it);
         }
         count = (int)B.items.size();
-        if (!B.build() || !B.widen()) { set_error("wost_create_scene: BVH too deep"); return WOST_ERR_INVALID_ARG; }
+        std::vector<Builder::WNode> wide, caps;
+        bool ok = B.build();
+        if (ok && d == 3) {
+            wide = B.widen(4, kLeaf);
+            ok = Builder::fits(wide);
+            if (bcv == 0) {
+                // a very deep tree takes fewer children per node, then the
+                // larger leaves (always fits: the binary depth is below 62)
+                for (int W : {8, 4, 2})
+                    if (W == 8 || !Builder::fits(caps)) caps = B.widen(W, kLeafCaps);
+                if (!Builder::fits(caps)) caps = B.widen(2, kLeaf);
+            }
+        }
+        if (!ok) { set_error("wost_create_scene: BVH too deep"); return WOST_ERR_INVALID_ARG; }
         depth = B.maxdepth;
         std::vector<float4> prims;
         std::vector<double> p64;
@@ -447,8 +614,22 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
             }
         }
         wost_status st;
-        if ((st = upload(s, B.pack(), &bv.nodes)) != WOST_OK) return st;
-        bv.nnodes = B.device_nodes();
+        if ((st = upload(s, d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK) return st;
+        bv.nnodes = (int)(d == 2 ? B.nodes.size() : (bcv == 0 ? caps.size() : wide.size()));
+        bv.need = caps.empty() ? 0 : Builder::stack_need(caps, 0);
+        if (bcv == 0) {
+            std::vector<float> vp((size_t)count * d * d), vn((size_t)count * d);
+            for (int i = 0; i < count; ++i) {
+                const int id = B.items[i].idx;
+                for (int j = 0; j < d; ++j)
+                    for (int k = 0; k < d; ++k) vp[((size_t)i * d + j) * d + k] = fv(P[(size_t)id * d + j], k);
+                for (int k = 0; k < d; ++k) vn[(size_t)i * d + k] = (float)nin[(size_t)id * d + k];
+            }
+            double far = diag;
+            for (int k = 0; k < d; ++k) far = std::max(far, std::max(std::fabs(lo[k]), std::fabs(hi[k])));
+            if ((st = upload(s, d == 2 ? B.caps_binary(vp, vn, 1e-6 * far) : Builder::caps_wide(caps, vp, vn, 1e-6 * far),
+                             &s->dev.dir_caps)) != WOST_OK) return st;
+        }
         if ((st = upload(s, prims, &bv.prims)) != WOST_OK) return st;
         if ((st = upload(s, ids, &bv.ids)) != WOST_OK) return st;
         if ((st = upload(s, p64, &bv.prims64)) != WOST_OK) return st;
@@ -511,29 +692,36 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
             if (d == 2) it.b.lo[2] = it.b.hi[2] = 0.f;
             for (int k = 0; k < 3; ++k) it.c[k] = 0.5f * (pa[k] + pb[k]);
             it.idx = (int)e;
-            it.cone_free = el[e].f0 < 0 || el[e].f1 < 0;
-            for (int k = 0; k < d; ++k) {
-                if (el[e].f0 >= 0) it.n0[k] = (float)nin[(size_t)el[e].f0 * d + k];
-                if (el[e].f1 >= 0) it.n1[k] = (float)nin[(size_t)el[e].f1 * d + k];
-            }
             B.items.push_back(it);
         }
         s->nsil = (int)el.size();
-        if (!B.build() || !B.widen()) { set_error("wost_create_scene: BVH too deep"); delete s; return WOST_ERR_INVALID_ARG; }
+        std::vector<Builder::WNode> wide;
+        bool ok = B.build();
+        if (ok && d == 3) {
+            wide = B.widen(4, kLeaf);
+            ok = Builder::fits(wide);
+        }
+        if (!ok) { set_error("wost_create_scene: BVH too deep"); delete s; return WOST_ERR_INVALID_ARG; }
         s->depth_sil = B.maxdepth;
         std::vector<float4> prims;
         std::vector<int> ids;
         std::vector<int64_t> keys;
+        std::vector<SilData> data;
+        data.reserve(B.items.size());
         for (const Item &it : B.items) {
             const Elem &e = el[it.idx];
             ids.push_back(it.idx);
             keys.push_back(e.key);
-            bool always = e.f0 < 0 || e.f1 < 0;
+            const bool always = e.f0 < 0 || e.f1 < 0;   // 3D: marked by the zero normals
             float n0[3] = {0, 0, 0}, n1[3] = {0, 0, 0};
             for (int k = 0; k < d; ++k) {
                 if (e.f0 >= 0) n0[k] = (float)nin[(size_t)e.f0 * d + k];
                 if (e.f1 >= 0) n1[k] = (float)nin[(size_t)e.f1 * d + k];
             }
+            SilData sd;
+            for (int k = 0; k < d; ++k) { sd.n0[k] = n0[k]; sd.n1[k] = n1[k]; sd.v[k] = fv(e.a, k); }
+            sd.free = always;
+            data.push_back(sd);
             if (d == 2) {
                 prims.push_back(make_float4(fv(e.a, 0), fv(e.a, 1), n0[0], n0[1]));
                 prims.push_back(make_float4(n1[0], n1[1], always ? 1.f : 0.f, 0.f));
@@ -541,17 +729,18 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
                 prims.push_back(make_float4(fv(e.a, 0), fv(e.a, 1), fv(e.a, 2), fv(e.b, 0)));
                 prims.push_back(make_float4(fv(e.b, 1), fv(e.b, 2), n0[0], n0[1]));
                 prims.push_back(make_float4(n0[2], n1[0], n1[1], n1[2]));
-                prims.push_back(make_float4(always ? 1.f : 0.f, 0.f, 0.f, 0.f));
             }
         }
         DevBVH &bv = s->dev.sil;
-        if ((st = upload(s, B.cones(), &s->dev.sil_cones)) != WOST_OK) { delete s; return st; }
-        if ((st = upload(s, B.pack(), &bv.nodes)) != WOST_OK ||
+        const double tau = (float)(1e-6 * diag);
+        if ((st = upload(s, d == 2 ? B.facing_binary(data, tau) : Builder::facing_wide(data, wide, tau), &s->dev.sil_facing)) != WOST_OK) { delete s; return st; }
+        if ((st = upload(s, d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK ||
             (st = upload(s, prims, &bv.prims)) != WOST_OK || (st = upload(s, ids, &bv.ids)) != WOST_OK) {
             delete s;
             return st;
         }
-        bv.nnodes = B.device_nodes();
+        bv.nnodes = (int)(d == 2 ? B.nodes.size() : wide.size());
+        bv.need = 0;
         const int64_t *kp = nullptr;
         if ((st = upload(s, keys, &kp)) != WOST_OK) { delete s; return st; }
         s->sil_key = const_cast<int64_t *>(kp);

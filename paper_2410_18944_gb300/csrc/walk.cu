@@ -24,7 +24,7 @@ namespace wost {
 double walk_alg_bytes(int D, bool guided, const unsigned long long *hs, int64_t records) {
     // bytes per item of the leaf-order arrays (see common.cuh)
     const double node_b = 16.0 * (D == 2 ? node_f4<2>() : node_f4<3>()), prim_b = D == 2 ? 16 : 48,
-                 sil_b = D == 2 ? 32 : 64;
+                 sil_b = D == 2 ? 32 : 48;
     double b = hs[3] * node_b + hs[4] * prim_b + hs[5] * sil_b + hs[6] * prim_b;
     b += (double)hs[2] * (D * 8.0 + 2 * 8.0);          // start point, FP64 sum and sum of squares
     if (guided) {
@@ -82,18 +82,20 @@ void DevBuf::release() {
 constexpr int kPlainBlock = 128;
 
 template <int D>
-__global__ void __launch_bounds__(kPlainBlock) plain_walk_kernel(const __grid_constant__ WalkArgs a) {
-    plain_loop<D>(SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
+__global__ void __launch_bounds__(kPlainBlock, D == 3 ? 8 : 0) plain_walk_kernel(const __grid_constant__ WalkArgs a) {
+    plain_loop<D, false>(coop_shared<D, kPlainBlock / 32>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
 }
 
 // status of every query point: 2 outside (odd/even crossing count of a ray
 // against all primitives), 1 inside the epsilon-shell (value g(xbar)), 0 walk
 template <int D>
-__global__ void classify_kernel(WalkArgs a, double *shell_value) {
+__global__ void __launch_bounds__(kPlainBlock) classify_kernel(WalkArgs a, double *shell_value) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.npoints) return;
+    const bool act = i < a.npoints;
     double val;
-    const_cast<uint8_t *>(a.status)[i] = classify_point<D>(a.sc, a.eps64, a.points + i * D, a.err, val);
+    const uint8_t st = classify_point<D, false>(coop_shared<D, kPlainBlock / 32>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
+    if (!act) return;
+    const_cast<uint8_t *>(a.status)[i] = st;
     shell_value[i] = val;
 }
 
@@ -108,11 +110,14 @@ __global__ void finalize_kernel(const uint8_t *status, const double *shell_value
 template <int D>
 __global__ void q_closest_kernel(DevScene sc, const double *p, int64_t n, int32_t *oid, float *od, int *err) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x[D];
-    for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
+    const bool act = i < n;
+    if (D == 2 && !act) return;
+    float x[D] = {};
+    if (act)
+        for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
     float b;
-    int s = closest_dirichlet<D>(sc.dir, x, b, err);
+    const int s = query_dirichlet<D, false>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
+    if (!act) return;
     oid[i] = s >= 0 ? sc.dir.ids[s] : -1;
     od[i] = sqrtf(b);
 }
@@ -121,11 +126,14 @@ template <int D>
 __global__ void q_sil_kernel(DevScene sc, const int64_t *keys, const double *p, int64_t n, int64_t *oid,
                              float *od, int *err) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x[D];
-    for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
+    const bool act = i < n;
+    if (D == 2 && !act) return;
+    float x[D] = {};
+    if (act)
+        for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
     float b = __int_as_float(0x7f800000);
-    int s = closest_silhouette<D>(sc.sil, x, sc.tau, b, err, nullptr, sc.sil_cones);
+    const int s = query_silhouette<D, false>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
+    if (!act) return;
     oid[i] = s >= 0 ? keys[s] : -1;
     od[i] = s >= 0 ? sqrtf(b) : b;
 }
@@ -139,27 +147,31 @@ __global__ void q_ray_kernel(DevScene sc, const double *o, const double *v, cons
                              const int32_t *skip_id, const int *slot_of_id, int64_t n, int32_t *oid, float *ot,
                              int *err) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x[D], d[D];
-    for (int k = 0; k < D; ++k) { x[k] = (float)o[i * D + k]; d[k] = (float)v[i * D + k]; }
-    int skip = skip_id && skip_id[i] >= 0 ? slot_of_id[skip_id[i]] : -1;
-    float t;
-    float tm = (float)tmax[i];
-    int s;
+    const bool act = i < n;
+    if (D == 2 && !act) return;
+    CoopWarp *sh = coop_shared<D, kPlainBlock / 32>();
+    float x[D] = {}, d[D] = {}, tm = 0.f, t;
+    int skip = -1, s;
+    if (act) {
+        for (int k = 0; k < D; ++k) { x[k] = (float)o[i * D + k]; d[k] = (float)v[i * D + k]; }
+        skip = skip_id && skip_id[i] >= 0 ? slot_of_id[skip_id[i]] : -1;
+        tm = (float)tmax[i];
+    }
     if (kExit) {
-        const float tneg = kRoundBand * sc.scale;
-        s = ray_neumann<D, true>(sc.neu, x, d, tm, skip, t, err, nullptr, tneg);
-        if (s >= 0 && tm - t <= kRoundBand * (sc.scale + tm)) {
-            double t64;
-            if (!ray_prim64<D, true>(sc.neu, s, x, d, t64, tneg) || t64 > (double)tm) s = -1;
-        }
+        s = query_exit<D, false>(sh, sc, act, x, d, tm, skip, t, err, nullptr);
     } else {
-        s = ray_neumann<D>(sc.neu, x, d, tm, skip, t, err);
+        if constexpr (D == 2) {
+            s = ray_neumann<false>(sc.neu, x, d, tm, skip, t, err);
+        } else {
+            t = tm;
+            s = coop_run<kCoopAny, false>(*sh, sc, act, x, d, t, skip, err, nullptr);
+        }
         if (s >= 0) {
             double t64;
             if (!ray_prim64<D>(sc.neu, s, x, d, t64) || t64 > tmax[i]) s = -1;
         }
     }
+    if (!act) return;
     oid[i] = s >= 0 ? sc.neu.ids[s] : -1;
     ot[i] = s >= 0 ? t : __int_as_float(0x7f800000);
 }
@@ -309,6 +321,7 @@ extern "C" wost_status wost_solve(wost_scene *s, wost_field *field, const double
         }
         int cps = ex.ctas_per_sm > 0 ? std::min(ex.ctas_per_sm, occ[D]) : occ[D];
         int grid = num_sms() * cps;
+        a.lanes = plain_lanes(s->dev, a.total, grid * (kPlainBlock / 32));
         tm.mark(tm.walk, st);
         if (D == 2) plain_walk_kernel<2><<<grid, kPlainBlock, 0, st>>>(a);
         else plain_walk_kernel<3><<<grid, kPlainBlock, 0, st>>>(a);

@@ -11,14 +11,9 @@
 //   5. first Neumann hit within r (FP64 re-test of the winner) or x + r nu.
 // Random numbers: Philox4x32-10, counter (point, walk, step, purpose).
 #pragma once
-#include "geom.cuh"
+#include "coop.cuh"
 
 namespace wost {
-
-// width of the band (relative to the scene scale) inside which an FP32
-// distance or hit parameter may be on the wrong side of its threshold:
-// 16 units of 2^-24
-constexpr float kRoundBand = 16.f * 5.9604645e-8f;
 
 struct WalkArgs {
     DevScene sc;
@@ -43,6 +38,7 @@ struct WalkArgs {
     // take in this launch
     const uint32_t *order;
     unsigned *plen;
+    int lanes;                 // plain 3D walks: walks per warp (plain_lanes)
 };
 
 // what one step needs besides the walk state: the walk's scene and the
@@ -179,92 +175,138 @@ __device__ __forceinline__ float neumann_term(const Walk<D> &w, const DevScene &
     return G * eval_fn<D>(sc.h, z) * W * (w.prim >= 0 ? 2.f : 1.f);
 }
 
-// Steps 1-3.  Returns true if the walk ended (its value already added;
-// term_value 0 after a lost roulette draw).  On return false: r (star
-// radius) and S (this step's source and Neumann terms, times the step's
-// roulette scale, as the suffix pass of a recorded walk takes them).
-template <int D>
-__device__ __forceinline__ bool step_geometry(Walk<D> &w, const StepEnv &a, float &r, float &S,
-                                              float &term_value, bool &truncated, Visits *vis) {
-    const DevScene &sc = a.sc;
-    float bd2;
-    int slot = closest_dirichlet<D>(sc.dir, w.x, bd2, a.err, vis);
-    float RD = sqrtf(bd2);
-    // eps-shell decision: in FP64 when the FP32 distance lies within its
-    // rounding band around eps (elsewhere both precisions agree)
-    double q64[3];
-    bool have64 = false, shell;
-    if (fabsf(RD - a.eps) <= kRoundBand * (sc.scale + RD)) {
-        shell = dirichlet_dist64<D>(sc.dir, slot, w.x, q64) <= a.eps64;
-        have64 = true;
+// The queries of a step: per lane in 2D (called by the lanes that want one),
+// by groups of lanes in 3D (called by the whole warp).  kMulti: the lanes'
+// scenes may differ.
+template <int D, bool kMulti>
+__device__ __forceinline__ int query_dirichlet(CoopWarp *sh, const DevScene &sc, bool want, const float *x, float &d2,
+                                               int *err, Visits *vis) {
+    if constexpr (D == 2) {
+        return closest_dirichlet(sc.dir, sc.dir_caps, x, d2, err, vis);
     } else {
-        shell = RD <= a.eps;
+        return coop_closest<kMulti>(*sh, sc, want, x, d2, err, vis);
     }
-    if (shell || w.k >= a.maxsteps) {
-        if (!have64) dirichlet_dist64<D>(sc.dir, slot, w.x, q64);
-        float xb[3] = {(float)q64[0], (float)q64[1], D == 3 ? (float)q64[2] : 0.f};
-        term_value = eval_fn<D>(sc.g, xb);
-        w.acc += w.T * term_value;
-        truncated = !shell;
-        return true;
-    }
-    if (roulette_on(a, w.k)) {
-        if (!roulette_survives(a, w.pid, w.wid, w.k)) {
-            term_value = 0.f;
-            truncated = false;
-            return true;
-        }
-        w.T *= 1.f / a.rr_q;
-    }
-    float bs = RD * RD;
-    closest_silhouette<D>(sc.sil, w.x, sc.tau, bs, a.err, vis, sc.sil_cones);
-    float R = fminf(sqrtf(bs), RD);
-    r = fmaxf(R, a.eps);
-    S = 0.f;
-    if (sc.has_source) {
-        U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_SRC, a.key0, a.key1);
-        float vs[D];
-        uniform_dir<D>(u01(u.x), u01(u.y), vs);
-        if (w.prim >= 0 && dotv<D>(vs, w.n) < 0.f) reflect<D>(vs, w.n);
-        float rho = D == 2 ? r * sqrtf(u01(u.z) * u01(u.w)) : r * beta22_inv(u01(u.z));
-        float th;
-        const float tneg = kRoundBand * sc.scale;
-        int hs = ray_neumann<D, true>(sc.neu, w.x, vs, rho, w.prim, th, a.err, vis, tneg);
-        if (hs >= 0 && rho - th <= kRoundBand * (sc.scale + rho)) {
-            double t64;
-            if (!ray_prim64<D, true>(sc.neu, hs, w.x, vs, t64, tneg) || t64 > (double)rho) hs = -1;
-        }
-        if (hs < 0) {
-            float y[3];
-#pragma unroll
-            for (int i = 0; i < D; ++i) y[i] = w.x[i] + rho * vs[i];
-            S = -(r * r / (2.f * D)) * eval_fn<D>(sc.f, y);
-        }
-        if (!sc.has_flux) w.acc += w.T * S;
-    }
-    if (sc.has_flux) {
-        S -= neumann_term<D>(w, sc, r, a.key0, a.key1, a.err, vis);
-        w.acc += w.T * S;
-    }
-    S *= roulette_scale(a, w.k);
-    return false;
 }
 
-// Step 5: ray cast within r and move.
-template <int D>
-__device__ __forceinline__ void step_move(Walk<D> &w, const StepEnv &a, const float *nu, float r, Visits *vis) {
+template <int D, bool kMulti>
+__device__ __forceinline__ int query_silhouette(CoopWarp *sh, const DevScene &sc, bool want, const float *x, float &d2,
+                                                 int *err, Visits *vis) {
+    if constexpr (D == 2) return closest_silhouette(sc.sil, x, sc.tau, d2, err, sc.sil_facing, vis);
+    else return coop_run<kCoopSil, kMulti>(*sh, sc, want, x, x, d2, -1, err, vis);
+}
+
+// first exit through the Neumann boundary within tmax, re-tested in FP64 when
+// the FP32 hit lies within its rounding band below tmax
+template <int D, bool kMulti>
+__device__ __forceinline__ int query_exit(CoopWarp *sh, const DevScene &sc, bool want, const float *x, const float *v,
+                                          float tmax, int skip, float &th, int *err, Visits *vis) {
+    const float tneg = kRoundBand * sc.scale;
+    int hit;
+    if constexpr (D == 2) {
+        hit = ray_neumann<true>(sc.neu, x, v, tmax, skip, th, err, vis, tneg);
+    } else {
+        th = tmax;
+        hit = coop_run<kCoopExit, kMulti>(*sh, sc, want, x, v, th, skip, err, vis);
+    }
+    if (hit >= 0 && tmax - th <= kRoundBand * (sc.scale + tmax)) {
+        double t64;
+        if (!ray_prim64<D, true>(sc.neu, hit, x, v, t64, tneg) || t64 > (double)tmax) hit = -1;
+    }
+    return hit;
+}
+
+// Steps 1-3 of the lanes with `act` (3D: the whole warp calls).  Returns true
+// if the walk ended (its value already added; term_value 0 after a lost
+// roulette draw).  On return false: r (star radius) and S (this step's source
+// and Neumann terms, times the step's roulette scale, as the suffix pass of a
+// recorded walk takes them).
+template <int D, bool kMulti>
+__device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const StepEnv &a, bool act, float &r, float &S,
+                                              float &term_value, bool &truncated, Visits *vis) {
+    if (D == 2 && !act) return false;
+    const DevScene &sc = a.sc;
+    float bd2;
+    const int slot = query_dirichlet<D, kMulti>(sh, sc, act, w.x, bd2, a.err, vis);
+    const float RD = sqrtf(bd2);
+    bool ended = false;
+    if (act) {
+        // eps-shell decision: in FP64 when the FP32 distance lies within its
+        // rounding band around eps (elsewhere both precisions agree)
+        double q64[3];
+        bool have64 = false, shell;
+        if (fabsf(RD - a.eps) <= kRoundBand * (sc.scale + RD)) {
+            shell = dirichlet_dist64<D>(sc.dir, slot, w.x, q64) <= a.eps64;
+            have64 = true;
+        } else {
+            shell = RD <= a.eps;
+        }
+        if (shell || w.k >= a.maxsteps) {
+            if (!have64) dirichlet_dist64<D>(sc.dir, slot, w.x, q64);
+            float xb[3] = {(float)q64[0], (float)q64[1], D == 3 ? (float)q64[2] : 0.f};
+            term_value = eval_fn<D>(sc.g, xb);
+            w.acc += w.T * term_value;
+            truncated = !shell;
+            ended = true;
+        } else if (roulette_on(a, w.k)) {
+            if (!roulette_survives(a, w.pid, w.wid, w.k)) {
+                term_value = 0.f;
+                truncated = false;
+                ended = true;
+            } else {
+                w.T *= 1.f / a.rr_q;
+            }
+        }
+    }
+    if (D == 2 && ended) return true;
+    const bool go = act && !ended;
+    float bs = RD * RD;
+    query_silhouette<D, kMulti>(sh, sc, go, w.x, bs, a.err, vis);
+    if (go) {
+        float R = fminf(sqrtf(bs), RD);
+        r = fmaxf(R, a.eps);
+        S = 0.f;
+    }
+    const bool source = go && sc.has_source;
+    if (D == 2 ? source : __any_sync(0xffffffffu, source)) {
+        float vs[D] = {}, rho = 0.f;
+        if (source) {
+            U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_SRC, a.key0, a.key1);
+            uniform_dir<D>(u01(u.x), u01(u.y), vs);
+            if (w.prim >= 0 && dotv<D>(vs, w.n) < 0.f) reflect<D>(vs, w.n);
+            rho = D == 2 ? r * sqrtf(u01(u.z) * u01(u.w)) : r * beta22_inv(u01(u.z));
+        }
+        float th;
+        const int hs = query_exit<D, kMulti>(sh, sc, source, w.x, vs, rho, w.prim, th, a.err, vis);
+        if (source) {
+            if (hs < 0) {
+                float y[3];
+#pragma unroll
+                for (int i = 0; i < D; ++i) y[i] = w.x[i] + rho * vs[i];
+                S = -(r * r / (2.f * D)) * eval_fn<D>(sc.f, y);
+            }
+            if (!sc.has_flux) w.acc += w.T * S;
+        }
+    }
+    if (go) {
+        if (sc.has_flux) {
+            S -= neumann_term<D>(w, sc, r, a.key0, a.key1, a.err, vis);
+            w.acc += w.T * S;
+        }
+        S *= roulette_scale(a, w.k);
+    }
+    return ended;
+}
+
+// Step 5 of the lanes with `act` (3D: the whole warp calls): ray cast within
+// r and move.
+template <int D, bool kMulti>
+__device__ __forceinline__ void step_move(CoopWarp *sh, Walk<D> &w, const StepEnv &a, bool act, const float *nu, float r,
+                                          Visits *vis) {
+    if (D == 2 && !act) return;
     const DevScene &sc = a.sc;
     float th;
-    // the first exit through the Neumann boundary (ray_prim, kExit), from
-    // t > -(rounding band of a position)
-    const float tneg = kRoundBand * sc.scale;
-    int hit = ray_neumann<D, true>(sc.neu, w.x, nu, r, w.prim, th, a.err, vis, tneg);
-    // hit-or-reach-r decision: in FP64 when the FP32 hit lies within its
-    // rounding band below r
-    if (hit >= 0 && r - th <= kRoundBand * (sc.scale + r)) {
-        double t64;
-        if (!ray_prim64<D, true>(sc.neu, hit, w.x, nu, t64, tneg) || t64 > (double)r) hit = -1;
-    }
+    const int hit = query_exit<D, kMulti>(sh, sc, act, w.x, nu, r, w.prim, th, a.err, vis);
+    if (!act) return;
     if (hit >= 0) {
         // an exit hit arrives from the inside, the side the walk is on, so
         // the walker's normal is the primitive's inward normal (Sec. 4.1,
@@ -272,6 +314,7 @@ __device__ __forceinline__ void step_move(Walk<D> &w, const StepEnv &a, const fl
         // hit point moved tneg along that normal: a rounded hit point may lie
         // on either side of the boundary, and every later query (silhouettes,
         // exit casts near a vertex) needs a start point inside the domain.
+        const float tneg = kRoundBand * sc.scale;
         th = fmaxf(th, 0.f);
 #pragma unroll
         for (int i = 0; i < D; ++i) {
@@ -287,26 +330,47 @@ __device__ __forceinline__ void step_move(Walk<D> &w, const StepEnv &a, const fl
     w.k++;
 }
 
+// crossings of the ray x + t v (t > 0) with the whole boundary
+template <int D, bool kMulti>
+__device__ __forceinline__ int count_crossings(CoopWarp *sh, const DevScene &sc, bool want, const float *x,
+                                               const float *v, int *err) {
+    if constexpr (D == 2) {
+        return ray_count(sc.dir, x, v, err) + ray_count(sc.neu, x, v, err);
+    } else {
+        float far = 3.0e38f;
+        const int n = coop_run<kCoopCount, kMulti>(*sh, sc, want, x, v, far, 1, err, nullptr);
+        return n + coop_run<kCoopCount, kMulti>(*sh, sc, want, x, v, far, 0, err, nullptr);
+    }
+}
+
 // Status of a query point: 2 outside (odd/even crossing count of a fixed
 // ray against all primitives), 1 inside the epsilon-shell (val = g at the
 // closest Dirichlet point, FP64 distance test), 0 to be walked.
-template <int D>
-__device__ __forceinline__ uint8_t classify_point(const DevScene &sc, double eps64, const double *p, int *err,
-                                                  double &val) {
-    float x[D];
-    for (int k = 0; k < D; ++k) x[k] = (float)p[k];
+// (3D: the whole warp calls, `act`: the lanes with a point)
+template <int D, bool kMulti>
+__device__ __forceinline__ uint8_t classify_point(CoopWarp *sh, const DevScene &sc, double eps64, const double *p,
+                                                  bool act, int *err, double &val) {
+    float x[D] = {};
+    if (act)
+        for (int k = 0; k < D; ++k) x[k] = (float)p[k];
     const float dir[3] = {0.5377844f, 0.7924136f, 0.2876523f};
     float v[D], nn = 0.f;
     for (int k = 0; k < D; ++k) { v[k] = dir[k]; nn += v[k] * v[k]; }
     for (int k = 0; k < D; ++k) v[k] *= rsqrtf(nn);
-    int c = ray_count<D>(sc.dir, x, v, err) + ray_count<D>(sc.neu, x, v, err);
+    if (D == 2 && !act) return 0;
+    const int c = count_crossings<D, kMulti>(sh, sc, act, x, v, err);
     val = 0.0;
-    if ((c & 1) == 0) {
+    const bool inside = act && (c & 1) != 0;
+    if (D == 2 && !inside) {
         val = __longlong_as_double(0x7ff8000000000000LL);
         return 2;
     }
     float bd2;
-    int slot = closest_dirichlet<D>(sc.dir, x, bd2, err);
+    const int slot = query_dirichlet<D, kMulti>(sh, sc, inside, x, bd2, err, nullptr);
+    if (!inside) {
+        val = __longlong_as_double(0x7ff8000000000000LL);
+        return 2;
+    }
     double q[3];
     if (dirichlet_dist64<D>(sc.dir, slot, x, q) <= eps64) {
         float xb[3] = {(float)q[0], (float)q[1], D == 3 ? (float)q[2] : 0.f};

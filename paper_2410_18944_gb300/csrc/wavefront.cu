@@ -38,6 +38,11 @@ namespace {
 constexpr int kWfBlock = 128;
 constexpr int kThetaStride = kOutPad;   // FP16 decoded outputs per decode row
 constexpr int kWfChunk = 8;             // iterations between host checks
+#ifndef WOST_WF_LANES3
+#define WOST_WF_LANES3 8
+#endif
+constexpr int kWfLanes3 = WOST_WF_LANES3;   // 3D: walks per warp of the step kernel
+constexpr int wf_walks_per_block(int d) { return kWfBlock / 32 * (d == 2 ? 32 : kWfLanes3); }
 
 // Iteration k's step kernel reads the decode list of iteration k-1 (entry j
 // is an active walk whose pending step decoded into row j of theta) and
@@ -88,15 +93,17 @@ __device__ __forceinline__ void store_walk(const WfSlots &S, int s, const Walk<D
     S.ids[s] = make_int4((int)w.pid, (int)w.wid, w.k, w.prim);
 }
 
-template <int D, class Src>
-__device__ __forceinline__ void wf_step_body(const Src &src, const WsOpts &o, const WfSlots &S, int parity,
-                                             bool first) {
+template <int D, bool kMulti, class Src>
+__device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const WsOpts &o, const WfSlots &S,
+                                             int parity, bool first) {
     // one thread per entry of the previous iteration's decode list (or per
     // slot in the first iteration); blocks past the list's end leave at once
     const unsigned n_in = first ? (unsigned)S.nslots : S.dcount[parity ^ 1];
-    const unsigned j = blockIdx.x * kWfBlock + threadIdx.x;
-    if (blockIdx.x * kWfBlock >= n_in) return;
-    const bool valid = j < n_in;
+    // (3D: kWfLanes3 entries per warp, see walk_lanes)
+    constexpr unsigned L = D == 2 ? 32 : kWfLanes3;
+    const unsigned j = (blockIdx.x * (kWfBlock / 32) + threadIdx.x / 32) * L + threadIdx.x % 32;
+    if (blockIdx.x * (kWfBlock / 32) * L >= n_in) return;
+    const bool valid = threadIdx.x % 32 < L && j < n_in;
     // decoded rows are staged in shared memory (stride of 25 words: the
     // scalar reads of the mixture evaluation are free of bank conflicts)
     __shared__ __half rows[kWfBlock * kYStride];
@@ -106,8 +113,14 @@ __device__ __forceinline__ void wf_step_body(const Src &src, const WsOpts &o, co
     unsigned long long nsteps = 0, ntrunc = 0, nwalks = 0;
     const int s = valid ? (first ? (int)j : S.dlist[parity ^ 1][j]) : 0;
     Walk<D> w;
+    if (D == 3) {   // lanes without a walk take part in the groups' queries
+        w.job = 0;
+        w.prim = -1;
+        w.k = 0;
+        for (int i = 0; i < D; ++i) w.x[i] = 0.f;
+    }
     bool active = valid && !first;
-    float r = 0.f, Sx = 0.f;
+    float r = 0.f, Sx = 0.f, nu[D] = {};
     if (active) {
         load_walk<D>(S, s, w);
         w.job = S.job[s];
@@ -126,7 +139,6 @@ __device__ __forceinline__ void wf_step_body(const Src &src, const WsOpts &o, co
         m.init(myrow);
         const float c = o.c_mode ? o.c_fixed : m.c();
         const StepEnv env = src.env(w);
-        float nu[D];
         const bool from_guide =
             sample_direction_row<D, 8>(m, c, w.pid, w.wid, (uint32_t)w.k, env.key0, env.key1, nu);
         const bool onN = w.prim >= 0;
@@ -166,23 +178,24 @@ __device__ __forceinline__ void wf_step_body(const Src &src, const WsOpts &o, co
                 rr[2] = make_float4(n2, ptil, wgt * roulette_scale(env, w.k), Sx);
             }
             w.T *= wgt;
-            step_move<D>(w, env, nu, r, &vis);
         }
     }
+    if (D == 2 ? active : !first) step_move<D, kMulti>(sh, w, src.env(w), active, nu, r, &vis);
     // ---- the next step's geometry; an ended walk hands its slot to the next item ----
+    bool settled = !valid;   // this lane's geometry is done, or there is no work for it
     for (;;) {
-        if (!active) {
-            if (!valid) break;
+        if (!active && !settled) {
             const unsigned long long item = warp_fetch_add(src.work_ctr(), true);
-            if (item >= src.total()) break;
-            if (!src.start(w, item)) continue;
-            active = true;
-            nwalks++;
+            if (item >= src.total()) settled = true;
+            else if (src.start(w, item)) { active = true; nwalks++; }
         }
-        nsteps++;
+        if (!__any_sync(0xffffffffu, !settled)) break;
+        const bool run = active && !settled;
+        if (D == 2 ? !run : !__any_sync(0xffffffffu, run)) continue;
+        nsteps += run;
         float gv;
         bool trunc = false;
-        if (step_geometry<D>(w, src.env(w), r, Sx, gv, trunc, &vis)) {
+        if (step_geometry<D, kMulti>(sh, w, src.env(w), run, r, Sx, gv, trunc, &vis)) {
             src.finish(w);
             // the suffix pass of a recorded walk waits for the end of the
             // launch (a recording launch gives every slot one walk, so its
@@ -191,9 +204,9 @@ __device__ __forceinline__ void wf_step_body(const Src &src, const WsOpts &o, co
             if (o.record) S.ended[s] = make_int2(w.k, __float_as_int(gv));
             ntrunc += trunc;
             active = false;
-            continue;
+        } else if (run) {
+            settled = true;
         }
-        break;
     }
     if (active) {
         store_walk<D>(S, s, w);
@@ -215,7 +228,8 @@ __global__ void wf_suffix_kernel(RecDest rd, const float *scratch, int scratch_s
 
 template <int D>
 __global__ void __launch_bounds__(kWfBlock) wf_step_kernel(const __grid_constant__ WfSoloArgs g) {
-    wf_step_body<D>(SoloSrc<D>{g.w, &g.f, g.rd, &g.w.sc}, g.o, g.S, g.parity, g.first != 0);
+    wf_step_body<D, false>(coop_shared<D, kWfBlock / 32>(), SoloSrc<D>{g.w, &g.f, g.rd, &g.w.sc}, g.o, g.S, g.parity,
+                           g.first != 0);
 }
 
 // decode rows [0, dcount[parity]) of the list into FP16 rows; clears the
@@ -327,7 +341,7 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
     }
     // one thread per list entry (at most one per slot): the block scheduler
     // balances the uneven step costs
-    const int gs = (nslots + kWfBlock - 1) / kWfBlock;
+    const int gs = (nslots + wf_walks_per_block(D) - 1) / wf_walks_per_block(D);
     const int gd = std::min(grid_dec[D], (nslots + 255) / 256);
     WfSoloArgs g{};
     g.w = a;
