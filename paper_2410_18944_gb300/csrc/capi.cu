@@ -212,7 +212,7 @@ extern "C" wost_status wost_create_field(const wost_field_desc *desc, wost_field
     for (void **p : bufs) if (rc == WOST_OK) rc = alloc(p, ng * sizeof(float));
     void **mbufs[] = {(void **)&f->mlp32, (void **)&f->mlp_m, (void **)&f->mlp_v, (void **)&f->mlp_g};
     for (void **p : mbufs) if (rc == WOST_OK) rc = alloc(p, nm * sizeof(float));
-    if (rc == WOST_OK) rc = alloc((void **)&f->grid16, (ng / 2) * sizeof(__half2));
+    if (rc == WOST_OK) rc = alloc((void **)&f->grid16, ((ng / 2 + 3) / 4) * 4 * sizeof(__half2));
     if (rc == WOST_OK) rc = alloc((void **)&f->wimg, wimg_bytes(f->km));
     if (rc == WOST_OK) rc = alloc((void **)&f->b3pad, out_pad(f->km) * sizeof(float));
     if (rc == WOST_OK) rc = alloc((void **)&f->loss_acc, 3 * sizeof(double));

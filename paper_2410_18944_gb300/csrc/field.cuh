@@ -172,6 +172,72 @@ __device__ __forceinline__ void encode_row(const DevField &f, const float *x, ui
     }
 }
 
+// The same row with the corners fetched in pairs.  The two corners of an edge
+// along x are neighbours in the table: entries id and id + 1 on a densely
+// indexed level, id and id ^ (v ^ (v + 1)) on a hashed one (prime 1), so three
+// quarters of the pairs lie in one aligned group of four entries, which one
+// 16-byte load brings; the rest take a second load.  The gathers are bound by
+// the rate of L1 lookups (one per lane and load, the table serves from L2), so
+// 1.25 loads per pair take the place of two (figures at decode_kernel; the
+// training step's two passes over 2^18 3D records 1473 -> 1338 us per call).  Costs 8 more registers per
+// level in flight, which the walkers of the warp-specialised kernel do not
+// have.  Same features bit for bit: the corners are added in the same order.
+template <int D>
+__device__ __forceinline__ void encode_row_pairs(const DevField &f, const float *x, uint8_t *xtile, int row) {
+    float u[D];
+    unit_coords<D>(f, x, u);
+    constexpr int P = 1 << (D - 1);
+#pragma unroll 1
+    for (int l4 = 0; l4 < kMaxLevels; l4 += 4) {
+        float feat[8];
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            uint4 q[2][P];
+            uint32_t far[2][P];
+            float w[2][2 * P];
+            uint32_t i0[2][P], i1[2][P];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int l = l4 + h + j;
+                uint32_t idx[2 * P];
+                level_corners<D>(f, l, u, idx, w[j]);
+                const uint32_t off = f.level_off[l];
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    i0[j][p] = off + idx[2 * p];
+                    i1[j][p] = off + idx[2 * p + 1];
+                    q[j][p] = __ldcg(reinterpret_cast<const uint4 *>(f.grid16) + (i0[j][p] >> 2));
+                    far[j][p] = 0u;
+                    if ((i0[j][p] ^ i1[j][p]) >> 2)
+                        far[j][p] = __ldcg(reinterpret_cast<const uint32_t *>(f.grid16) + i1[j][p]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float a0 = 0.f, a1 = 0.f;
+                auto add = [&](uint32_t bits, float wt) {
+                    const float2 g = __half22float2(*reinterpret_cast<const __half2 *>(&bits));
+                    a0 = fmaf(wt, g.x, a0);
+                    a1 = fmaf(wt, g.y, a1);
+                };
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    const uint4 v = q[j][p];
+                    auto pick = [&](uint32_t i) {
+                        const uint32_t lo = (i & 1u) ? v.y : v.x, hi = (i & 1u) ? v.w : v.z;
+                        return (i & 2u) ? hi : lo;
+                    };
+                    add(pick(i0[j][p]), w[j][2 * p]);
+                    add((i0[j][p] ^ i1[j][p]) >> 2 ? far[j][p] : pick(i1[j][p]), w[j][2 * p + 1]);
+                }
+                feat[2 * (h + j)] = a0;
+                feat[2 * (h + j) + 1] = a1;
+            }
+        }
+        st_row8_bf16(xtile, row, 2 * l4, kFeat, feat);
+    }
+}
+
 // One 128-row tile: X (128 x 32) -> H1 -> H2 -> Y (128 x out_pad(KM)) in
 // TMEM columns [tcol, tcol + tile_tmem_cols(KM)).  Called by all 128 threads
 // of the tile; thread `row` owns row `row`.  `issuer` issues the MMAs.  On

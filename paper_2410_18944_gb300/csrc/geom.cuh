@@ -193,6 +193,17 @@ __device__ __forceinline__ R seg_d2(R ax, R ay, R bx, R by, R px, R py, R &qx, R
     return dx * dx + dy * dy;
 }
 
+// the FP32 distance of seg_d2, bit for bit, dividing only where the foot lies
+// inside the segment (few of a leaf's segments; star of 4096: 21.7 -> 21.1 ms)
+__device__ __forceinline__ float seg_d2_fast(float4 s, const float *x) {
+    const float ex = s.z - s.x, ey = s.w - s.y;
+    const float ee = ex * ex + ey * ey, dot = (x[0] - s.x) * ex + (x[1] - s.y) * ey;
+    float t = dot > 0.f ? 1.f : 0.f;
+    if (dot > 0.f && dot < ee) t = dot / ee;
+    const float dx = x[0] - __fmaf_rn(t, ex, s.x), dy = x[1] - __fmaf_rn(t, ey, s.y);
+    return dx * dx + dy * dy;
+}
+
 template <typename R>
 __device__ __forceinline__ R seg3_d2(const R *a, const R *b, const R *p) {
     R e[3], ap[3], ee = 0, t = 0;
@@ -342,8 +353,7 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
             if (vis) vis->dprims += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 float4 p = ldn(bv.prims + s);
-                float qx, qy;
-                const float d2 = seg_d2<float>(p.x, p.y, p.z, p.w, x[0], x[1], qx, qy);
+                const float d2 = seg_d2_fast(p, x);
                 if (d2 <= best) {
                     int id = __ldg(bv.ids + s);
                     if (d2 < best || id < best_id) { best = d2; best_slot = s; best_id = id; }

@@ -89,27 +89,53 @@ static int ws_walkers_for_field(const DevScene &s, const wost_field *f, int req,
 
 // decode of arbitrary points: the same tile forward as inside the walk
 // (KM: lobe capacity of the field's internal output layout)
+// Bound by the corner gathers (L1 lookups) and the output rows, once written a
+// row per thread: 41 stores of 32 sectors each per warp.  Measured on one
+// GB300, 10^6 positions, 8 lobes: 3D 714 -> 369 us, 2D 457 -> 258 us with the
+// corners in pairs (encode_row_pairs) and the rows staged; three CTAs per SM
+// (85 registers, spilling) 558 us.
+constexpr int kDecodeCtas = 2;                // CTAs per SM
+constexpr int kStageFloats = 32 * kHid / 2;   // floats in a warp's quarter of the hidden tile
+
 template <int D, int KM>
-__global__ void __launch_bounds__(kGuidedBlock, 1) decode_kernel(DevField f, const double *pts, int64_t n,
+__global__ void __launch_bounds__(kGuidedBlock, KM <= kMaxK ? kDecodeCtas : 1) decode_kernel(DevField f, const double *pts, int64_t n,
                                                                  float *out, int nout, int *err) {
     extern __shared__ __align__(1024) uint8_t sm[];
     CtaTiles ct = cta_tiles_setup<KM>(sm, f);
     const int tid = threadIdx.x, tile = tid >> 7, row = tid & 127;
     TileCtx t{ct.xt + tile * kXTileBytes, ct.ht + tile * kHTileBytes, ct.wimg, &ct.mbar[tile],
               *ct.tptr + (uint32_t)(tile * tile_tmem_cols(KM)), 0u, 1 + tile};
+    // a warp's finished rows go out through shared memory (its quarter of the
+    // hidden tile, dead by then) in whole lines
+    float *stage = reinterpret_cast<float *>(t.htile) + (row >> 5) * kStageFloats;
+    const int lane = tid & 31, per = kStageFloats / nout;
     for (int64_t base = (int64_t)blockIdx.x * kGuidedBlock; base < n; base += (int64_t)gridDim.x * kGuidedBlock) {
         int64_t i = base + tid;
         float x[D];
         if (i < n) {
             for (int k = 0; k < D; ++k) x[k] = (float)pts[i * D + k];
-            encode_row<D>(f, x, t.xtile, row);
+            encode_row_pairs<D>(f, x, t.xtile, row);
         } else {
             zero_row(t.xtile, row, kFeat);
         }
         float raw[out_pad(KM)];
         if (!mlp_tile_forward<KM>(t, f, row, row == 0, raw, err)) break;
-        if (i < n)
-            for (int k = 0; k < nout; ++k) out[i * nout + k] = raw[exchange_to_out_row(k, D, f.K, KM)];
+        // (every thread of the tile waited for the last MMA, which read the tile)
+        const int64_t first = i - lane;
+        const int rows = (int)max((int64_t)0, min((int64_t)32, n - first));
+        for (int r0 = 0; r0 < rows; r0 += per) {
+            const int cnt = min(per, rows - r0);
+            if (lane >= r0 && lane < r0 + cnt)
+#pragma unroll
+                for (int r = 0; r < out_pad(KM); ++r) {
+                    const int e = out_row_to_exchange(r, D, f.K, KM);
+                    if (e >= 0 && r <= KM * (D + 2)) stage[(lane - r0) * nout + e] = raw[r];
+                }
+            __syncwarp();
+            float *o = out + (first + r0) * nout;
+            for (int k = lane; k < cnt * nout; k += 32) __stcs(o + k, stage[k]);
+            __syncwarp();
+        }
     }
     cta_tiles_teardown<KM>(ct);
 }
@@ -520,7 +546,7 @@ extern "C" wost_status wost_field_decode(wost_field *f, const double *points, in
         WOST_CUDA(cudaMalloc(&dout, n * f->nout * sizeof(float)));
         own_o = true;
     }
-    int grid = (int)std::min<int64_t>((n + kGuidedBlock - 1) / kGuidedBlock, (int64_t)num_sms() * 2);
+    int grid = (int)std::min<int64_t>((n + kGuidedBlock - 1) / kGuidedBlock, (int64_t)num_sms() * kDecodeCtas);
     auto launch = [&](auto kern, int smem) -> wost_status {
         WOST_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         kern<<<grid, kGuidedBlock, smem, st>>>(f->dev(), dp, n, dout, f->nout, device_err_flag());

@@ -266,7 +266,9 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
             rec[0] = r0.x; rec[1] = r0.y; rec[2] = r0.z; rec[3] = r0.w;
             rec[4] = r1.x; rec[5] = r1.y; rec[6] = r1.z; rec[7] = r1.w;
             rec[8] = r2.x; rec[9] = r2.y; rec[10] = r2.z; rec[11] = r2.w;
-            encode_row<D>(a.f, rec, t.X, row);
+            // (the 16-lobe kernel has no registers for the pairs: 968 -> 1012 us)
+            if constexpr (KM <= kMaxK) encode_row_pairs<D>(a.f, rec, t.X, row);
+            else encode_row<D>(a.f, rec, t.X, row);
         } else {
             for (int i = 0; i < 12; ++i) rec[i] = 0.f;
             for (int c = 0; c < kFeat; c += 8) *reinterpret_cast<uint4 *>(t.X + cm_offset(row, c, kFeat)) = make_uint4(0, 0, 0, 0);

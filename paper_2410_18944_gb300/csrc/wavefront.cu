@@ -38,10 +38,9 @@ namespace {
 constexpr int kWfBlock = 128;
 constexpr int kThetaStride = kOutPad;   // FP16 decoded outputs per decode row
 constexpr int kWfChunk = 8;             // iterations between host checks
-#ifndef WOST_WF_LANES3
-#define WOST_WF_LANES3 8
-#endif
-constexpr int kWfLanes3 = WOST_WF_LANES3;   // 3D: walks per warp of the step kernel
+// 3D: walks per warp of the step kernel (icosphere, 64k walks: 109 / 79 / 67 ms
+// with 32 / 16 / 8)
+constexpr int kWfLanes3 = 8;
 constexpr int wf_walks_per_block(int d) { return kWfBlock / 32 * (d == 2 ? 32 : kWfLanes3); }
 
 // Iteration k's step kernel reads the decode list of iteration k-1 (entry j
@@ -59,6 +58,7 @@ struct WfSlots {
     __half *theta;     // [rows][kThetaStride] decoded outputs of the last list
     int2 *ended;       // recording launches: (records, terminal value bits) of the slot's ended walk
     int nslots;
+    int warps;         // 3D: warps of the step kernel the GPU holds at once
 };
 
 struct WfSoloArgs {
@@ -99,8 +99,13 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
     // one thread per entry of the previous iteration's decode list (or per
     // slot in the first iteration); blocks past the list's end leave at once
     const unsigned n_in = first ? (unsigned)S.nslots : S.dcount[parity ^ 1];
-    // (3D: kWfLanes3 entries per warp, see walk_lanes)
-    constexpr unsigned L = D == 2 ? 32 : kWfLanes3;
+    // 3D: at most kWfLanes3 entries per warp, fewer once the list is short
+    // (a warp answers four to eight queries at a time, coop.cuh)
+    unsigned L = 32;
+    if (D == 3) {
+        L = kWfLanes3;
+        while (L > 1 && n_in * 2u <= L * (unsigned)S.warps) L >>= 1;
+    }
     const unsigned j = (blockIdx.x * (kWfBlock / 32) + threadIdx.x / 32) * L + threadIdx.x % 32;
     if (blockIdx.x * (kWfBlock / 32) * L >= n_in) return;
     const bool valid = threadIdx.x % 32 < L && j < n_in;
@@ -128,12 +133,12 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
         const float2 rs = S.rS[s];
         r = rs.x;
         Sx = rs.y;
-        const uint2 *src_row = reinterpret_cast<const uint2 *>(S.theta + (size_t)j * kThetaStride);
+        const uint4 *src_row = reinterpret_cast<const uint4 *>(S.theta + (size_t)j * kThetaStride);
 #pragma unroll
-        for (int i = 0; i < kThetaStride / 4; ++i) {
-            const uint2 v = __ldcs(src_row + i);
-            reinterpret_cast<uint32_t *>(myrow)[2 * i] = v.x;
-            reinterpret_cast<uint32_t *>(myrow)[2 * i + 1] = v.y;
+        for (int i = 0; i < kThetaStride / 8; ++i) {
+            const uint4 v = __ldcs(src_row + i);
+            uint32_t *dst = reinterpret_cast<uint32_t *>(myrow) + 4 * i;
+            dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
         }
         RowMixture<D, 8> m;
         m.init(myrow);
@@ -251,18 +256,23 @@ __global__ void __launch_bounds__(256, 1) wf_decode_kernel(DevField f, WfSlots S
             const int s = S.dlist[parity][i];
             const float4 xT = S.xT[s];
             const float x[3] = {xT.x, xT.y, xT.z};
-            encode_row<D>(f, x, t.xtile, row);
+            encode_row_pairs<D>(f, x, t.xtile, row);
         } else {
             zero_row(t.xtile, row, kFeat);
         }
         float raw[kOutPad];
         if (!mlp_tile_forward(t, f, row, row == 0, raw, err)) break;
         if (valid) {
-            uint2 *dst = reinterpret_cast<uint2 *>(S.theta + (size_t)i * kThetaStride);
+            uint4 *dst = reinterpret_cast<uint4 *>(S.theta + (size_t)i * kThetaStride);
 #pragma unroll
-            for (int c = 0; c < kOutPad; c += 4) {
-                __half2 a = __floats2half2_rn(raw[c], raw[c + 1]), b = __floats2half2_rn(raw[c + 2], raw[c + 3]);
-                __stcs(dst + c / 4, make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b)));
+            for (int c = 0; c < kOutPad; c += 8) {
+                uint32_t h[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __half2 a = __floats2half2_rn(raw[c + 2 * k], raw[c + 2 * k + 1]);
+                    h[k] = *reinterpret_cast<const uint32_t *>(&a);
+                }
+                __stcs(dst + c / 8, make_uint4(h[0], h[1], h[2], h[3]));
             }
         }
     }
@@ -325,7 +335,7 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
 
     // decode grid: the attribute is set, and the occupancy taken, once per
     // device (the device model, and so the grid, is the same on all of them)
-    static int grid_dec[4] = {0, 0, 0, 0};
+    static int grid_dec[4] = {0, 0, 0, 0}, step_warps[4] = {0, 0, 0, 0};
     {
         wost_status rc = once_per_device(300 + D, [&]() -> wost_status {
             if (D == 2) {
@@ -334,6 +344,7 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
             } else {
                 WOST_CUDA(cudaFuncSetAttribute(wf_decode_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCtaTilesSmem));
                 grid_dec[D] = occupancy_grid(wf_decode_kernel<3>, 256, kCtaTilesSmem);
+                step_warps[D] = occupancy_grid(wf_step_kernel<3>, kWfBlock, 0) * (kWfBlock / 32);
             }
             return WOST_OK;
         });
@@ -341,7 +352,8 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
     }
     // one thread per list entry (at most one per slot): the block scheduler
     // balances the uneven step costs
-    const int gs = (nslots + wf_walks_per_block(D) - 1) / wf_walks_per_block(D);
+    S.warps = step_warps[D];
+    const int gs = std::max((nslots + wf_walks_per_block(D) - 1) / wf_walks_per_block(D), step_warps[D] / (kWfBlock / 32));
     const int gd = std::min(grid_dec[D], (nslots + 255) / 256);
     WfSoloArgs g{};
     g.w = a;
