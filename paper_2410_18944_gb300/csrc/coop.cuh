@@ -23,8 +23,9 @@
 // Silhouettes and rays: groups of four lanes over four-wide nodes of boxes,
 // depth first, children nearest first.  An edge's or a hit's FP32 value can
 // lie below its box's by rounding (a ray hit by its edge slack, ray_prim), so
-// the result can depend on which box was opened first: the order of visits is
-// part of the query, and is that of neumann_pick's per-lane traversal.
+// the result can depend on which box was opened first, and the summed weight of
+// the Neumann sample on the order of its terms: the order of visits is part of
+// these queries.
 // All lanes of the warp run every call together.
 #pragma once
 #include "geom.cuh"
@@ -52,7 +53,7 @@ __device__ __forceinline__ CoopWarp *coop_shared() {
 }
 __host__ __device__ constexpr int coop_bytes(int D, int warps) { return D == 3 ? warps * (int)sizeof(CoopWarp) : 0; }
 
-enum : int { kCoopPoint = 0, kCoopPointBox = 1, kCoopSil = 2, kCoopExit = 3, kCoopAny = 4, kCoopCount = 5 };
+enum : int { kCoopPoint = 0, kCoopPointBox = 1, kCoopSil = 2, kCoopExit = 3, kCoopAny = 4, kCoopCount = 5, kCoopPick = 6 };
 
 // monotonic map of a float (not NaN) to an int
 __device__ __forceinline__ int order_key(float f) {
@@ -76,6 +77,7 @@ template <int kKind>
 __device__ __forceinline__ const DevBVH &coop_bvh(const DevScene &sc, bool dirichlet = false) {
     if (kKind == kCoopPoint || kKind == kCoopPointBox) return sc.dir;
     if (kKind == kCoopSil) return sc.sil;
+    if (kKind == kCoopPick) return sc.neu;
     if (kKind == kCoopCount) return dirichlet ? sc.dir : sc.neu;
     return sc.neu;
 }
@@ -89,6 +91,8 @@ __device__ __forceinline__ const DevBVH &coop_bvh(const DevScene &sc, bool diric
 //               (ray_prim, kExit), aux: slot skipped
 //   kCoopAny    first hit of either orientation, aux: slot skipped
 //   kCoopCount  crossings along v (returned), aux != 0: of the Dirichlet BVH
+//   kCoopPick   neumann_pick: best_io: in r^2, out W; v: the bits of point, walk
+//               and step, aux and key1: the key
 // Returns the leaf slot (-1: none within the bound).  kMulti: the lanes'
 // scenes may differ.
 // Out of line: the walk's state is saved once around the call instead of
@@ -101,13 +105,14 @@ struct CoopResult {
 };
 template <int kKind, bool kMulti>
 __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *scene_p, bool want, float x0, float x1,
-                                              float x2, float v0, float v1, float v2, float best_io, int aux, int *err) {
+                                              float x2, float v0, float v1, float v2, float best_io, int aux, uint32_t key1,
+                                              int *err) {
     CoopWarp &sh = *reinterpret_cast<CoopWarp *>(__cvta_shared_to_generic(sh_addr));
     const DevScene &scene = *scene_p;
     const float x[3] = {x0, x1, x2}, v[3] = {v0, v1, v2};
     CoopResult res{kKind == kCoopCount ? 0 : -1, best_io, 0u, 0u};
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr bool kRay = kKind >= kCoopExit;
+    constexpr bool kRay = kKind >= kCoopExit && kKind <= kCoopCount;
     constexpr int G = kKind == kCoopPoint ? 8 : 4, NG = 32 / G;   // lanes per group, groups
     const int lane = threadIdx.x & 31, sub = lane & (G - 1), g = lane / G, base = g * G;
     uint2 *stack = sh.stack[g];
@@ -123,11 +128,13 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
     // the group's query
     bool busy = false;
     int cur = 0, ref = 0, sp = 0, gaux = -1;
+    uint32_t gkey1 = 0;        // kCoopPick
     float best = 0.f, gx[3] = {0.f, 0.f, 0.f}, gv[3] = {0.f, 0.f, 0.f}, ginv[3] = {0.f, 0.f, 0.f};
     const DevScene *gs = &scene;
     // this lane's candidate of the group's query
     float lb = 0.f;
     int ls = -1, lid = INT_MAX;
+    float W = 0.f;             // kCoopPick: summed weight of the group's query
     for (;;) {
         const unsigned idle = __ballot_sync(kFull, !busy);
         if (todo && idle) {
@@ -142,14 +149,13 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
             const int from = take ? __ffs(mine) - 1 : lane;
             const float b0 = __shfl_sync(kFull, best_io, from);
             const int a0 = __shfl_sync(kFull, aux, from);
+            const uint32_t nk1 = kKind == kCoopPick ? __shfl_sync(kFull, key1, from) : 0u;
             float nx[3], nv[3], ni[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 nx[k] = __shfl_sync(kFull, x[k], from);
-                if (kRay) {
-                    nv[k] = __shfl_sync(kFull, v[k], from);
-                    ni[k] = __shfl_sync(kFull, inv[k], from);
-                }
+                if (kRay || kKind == kCoopPick) nv[k] = __shfl_sync(kFull, v[k], from);
+                if (kRay) ni[k] = __shfl_sync(kFull, inv[k], from);
             }
             const DevScene *ns = gs;
             if (kMulti)
@@ -162,11 +168,14 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                 sp = 0;
                 best = b0;
                 gaux = a0;
+                gkey1 = nk1;
+                W = 0.f;
                 gs = ns;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     gx[k] = nx[k];
-                    if (kRay) { gv[k] = nv[k]; ginv[k] = ni[k]; }
+                    if (kRay || kKind == kCoopPick) gv[k] = nv[k];
+                    if (kRay) ginv[k] = ni[k];
                 }
                 lb = __int_as_float(0x7f800000);
                 ls = -1;
@@ -275,7 +284,7 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                             far2 += df * df;
                         }
                         key = box_d2(dd[0], dd[1], dd[2]);
-                        ok = cref != kEmptyRef && key <= best;
+                        ok = cref != kEmptyRef && (kKind == kCoopPick ? key < best : key <= best);
                         if constexpr (kKind == kCoopSil) {
                             const float4 *fp = sc.sil_facing + (size_t)facing_f4(3) * ref;
                             const float4 f = ldn(fp + sub);   // axis, d0
@@ -328,6 +337,7 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
         const int s0 = leaf_start(ref), cnt = at ? leaf_count(ref) : 0;
         for (int b = 0; __any_sync(kFull, b < cnt); b += G) {
             const int s = s0 + b + sub;
+            float wt = 0.f;
             if (b + sub < cnt) {
                 float t;
                 bool cand;
@@ -342,6 +352,12 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                     cand = s != gaux && ray_prim<3, true>(bv.prims, s, gx, gv, t, tneg) && t <= best;
                 } else if (kKind == kCoopAny) {
                     cand = s != gaux && ray_prim<3>(bv.prims, s, gx, gv, t) && t <= best;
+                } else if (kKind == kCoopPick) {
+                    wt = neumann_weight<3>(bv, s, gx, best);
+                    cand = wt > 0.f;
+                    if (cand)
+                        t = neumann_key(__ldg(bv.ids + s), wt, __float_as_uint(gv[0]), __float_as_uint(gv[1]),
+                                        __float_as_uint(gv[2]), (uint32_t)gaux, gkey1);
                 } else {
                     lid += ray_prim<3>(bv.prims, s, gx, gv, t) ? 1 : 0;
                     cand = false;
@@ -351,9 +367,13 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                     if (t < lb || id < lid) { lb = t; ls = s; lid = id; }
                 }
             }
+            if constexpr (kKind == kCoopPick) {   // in the order of the primitives
+#pragma unroll
+                for (int j = 0; j < G; ++j) W += __shfl_sync(kFull, wt, base + j);
+            }
         }
         if (sub == 0) res.prims += cnt;
-        if (kKind != kCoopCount) best = fminf(best, group_min<G>(at ? lb : __int_as_float(0x7f800000)));
+        if (kKind != kCoopCount && kKind != kCoopPick) best = fminf(best, group_min<G>(at ? lb : __int_as_float(0x7f800000)));
         pop(at);
 
         // ---- results ----
@@ -364,8 +384,10 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                 for (int o = G / 2; o; o >>= 1) n += __shfl_xor_sync(kFull, n, o);
                 if (fin && sub == 0) sh.slot[cur] = n;
             } else {
-                const int id = ls >= 0 && lb == best ? lid : INT_MAX;
+                const float top = kKind == kCoopPick ? group_min<G>(lb) : best;
+                const int id = ls >= 0 && lb == top ? lid : INT_MAX;
                 const int mid = group_min<G>(id);
+                if (kKind == kCoopPick && fin) best = W;   // (returned in place of the bound)
                 if (fin) {
                     if (mid == INT_MAX) {
                         if (sub == 0) { sh.best[cur] = best; sh.slot[cur] = -1; }
@@ -389,9 +411,9 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
 // the call, with the visits added to the lane's counters
 template <int kKind, bool kMulti>
 __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool want, const float *x, const float *v,
-                                        float &best, int aux, int *err, Visits *vis) {
+                                        float &best, int aux, int *err, Visits *vis, uint32_t key1 = 0) {
     const CoopResult r = coop_query<kKind, kMulti>((uint32_t)__cvta_generic_to_shared(&sh), &sc, want, x[0], x[1], x[2],
-                                                   v[0], v[1], v[2], best, aux, err);
+                                                   v[0], v[1], v[2], best, aux, key1, err);
     best = r.best;
     if (vis) {
         vis->nodes += r.nodes;

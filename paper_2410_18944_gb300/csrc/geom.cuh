@@ -35,9 +35,7 @@ constexpr float kRoundBand = 16.f * 5.9604645e-8f;
 
 // BVH nodes.  2D: binary, child boxes in the parent (3 float4), one query per
 // lane (this file).  3D: four children per node, 4 x (lo.xyz, hi.x), then
-// 4 x (hi.yz, child, -), one query per group of lanes (coop.cuh; neumann_pick
-// one per lane).
-constexpr int lane_width(int d) { return d == 2 ? 2 : 4; }
+// 4 x (hi.yz, child, -), one query per group of lanes (coop.cuh).
 constexpr int kEmptyRef = INT_MIN;   // child slot without a child (wide nodes)
 
 // float4 per node
@@ -57,30 +55,15 @@ __device__ __forceinline__ float box_d2(float dx, float dy, float dz) {
     return __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
 }
 
-// keys of the children: squared distance from x to the child box (2D: the
-// binary nodes; 3D: the four-wide ones)
-template <int D>
+// keys of the children of a binary 2D node: squared distance from x to the box
 __device__ __forceinline__ void node_keys_d2(const float4 *nodes, int node, const float *x, float *k, int *r) {
-    if constexpr (D == 2) {
-        const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), q = ldn(nodes + 3 * node + 2);
-        float ax = fmaxf(fmaxf(a.x - x[0], x[0] - a.z), 0.f), ay = fmaxf(fmaxf(a.y - x[1], x[1] - a.w), 0.f);
-        float bx = fmaxf(fmaxf(b.x - x[0], x[0] - b.z), 0.f), by = fmaxf(fmaxf(b.y - x[1], x[1] - b.w), 0.f);
-        k[0] = ax * ax + ay * ay;
-        k[1] = bx * bx + by * by;
-        r[0] = __float_as_int(q.x);
-        r[1] = __float_as_int(q.y);
-    } else {
-        const float4 *p = nodes + (size_t)node_f4<3>() * node;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float4 a = ldn(p + c), b = ldn(p + 4 + c);
-            float dx = fmaxf(fmaxf(a.x - x[0], x[0] - a.w), 0.f);
-            float dy = fmaxf(fmaxf(a.y - x[1], x[1] - b.x), 0.f);
-            float dz = fmaxf(fmaxf(a.z - x[2], x[2] - b.y), 0.f);
-            k[c] = box_d2(dx, dy, dz);
-            r[c] = __float_as_int(b.z);
-        }
-    }
+    const float4 a = ldn(nodes + 3 * node), b = ldn(nodes + 3 * node + 1), q = ldn(nodes + 3 * node + 2);
+    float ax = fmaxf(fmaxf(a.x - x[0], x[0] - a.z), 0.f), ay = fmaxf(fmaxf(a.y - x[1], x[1] - a.w), 0.f);
+    float bx = fmaxf(fmaxf(b.x - x[0], x[0] - b.z), 0.f), by = fmaxf(fmaxf(b.y - x[1], x[1] - b.w), 0.f);
+    k[0] = ax * ax + ay * ay;
+    k[1] = bx * bx + by * by;
+    r[0] = __float_as_int(q.x);
+    r[1] = __float_as_int(q.y);
 }
 
 // keys of the children of a binary 2D node: entry parameter of the ray
@@ -660,10 +643,37 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
 // traversal visits the candidates in (weighted sampling with keys,
 // Efraimidis & Spirakis 2006); ties go to the smaller id.  Returns the leaf
 // slot of the choice (-1 if there is no candidate) and W.
+//
+// weight of leaf slot s, 0 if it is not within the ball (r2 = r^2)
 template <int D>
-__device__ int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t pid, uint32_t wid, uint32_t step,
-                            uint32_t k0, uint32_t k1, float &W, int *err, Visits *vis = nullptr) {
-    constexpr int kBW = lane_width(D);
+__device__ __forceinline__ float neumann_weight(const DevBVH &bv, int s, const float *x, float r2) {
+    float d2, w;
+    if (D == 2) {
+        float4 p = ldn(bv.prims + s);
+        float qx, qy;
+        d2 = seg_d2<float>(p.x, p.y, p.z, p.w, x[0], x[1], qx, qy);
+        w = sqrtf((p.z - p.x) * (p.z - p.x) + (p.w - p.y) * (p.w - p.y));
+    } else {
+        float a[3], b[3], c[3];
+        load_tri(bv.prims, s, a, b, c);
+        d2 = tri_d2_fast(a, b, c, x);
+        float e1[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]}, e2[3] = {c[0] - a[0], c[1] - a[1], c[2] - a[2]};
+        float n0 = e1[1] * e2[2] - e1[2] * e2[1], n1 = e1[2] * e2[0] - e1[0] * e2[2], n2 = e1[0] * e2[1] - e1[1] * e2[0];
+        w = 0.5f * sqrtf(n0 * n0 + n1 * n1 + n2 * n2);
+    }
+    return d2 < r2 && w > 0.f ? w : 0.f;
+}
+__device__ __forceinline__ float neumann_key(int id, float w, uint32_t pid, uint32_t wid, uint32_t step, uint32_t k0,
+                                             uint32_t k1) {
+    U4 u = philox(pid, wid, step, P_NKEY | (uint32_t)id, k0, k1);
+    const float uu = ((float)(u.x >> 8) + 1.f) * (1.0f / 16777216.0f);   // (0, 1]
+    return -logf(uu) / w;
+}
+
+// 2D (one query per lane; 3D: kCoopPick, coop.cuh)
+__device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t pid, uint32_t wid, uint32_t step,
+                                   uint32_t k0, uint32_t k1, float &W, int *err, Visits *vis = nullptr) {
+    constexpr int kBW = 2;
     W = 0.f;
     if (bv.nprims == 0) return -1;
     const float r2 = r * r;
@@ -681,35 +691,20 @@ __device__ int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t 
             float k[kBW];
             int rr[kBW];
             bool h[kBW];
-            node_keys_d2<D>(bv.nodes, ref, x, k, rr);
+            node_keys_d2(bv.nodes, ref, x, k, rr);
             if (vis) vis->nodes++;
 #pragma unroll
-            for (int c = 0; c < kBW; ++c) h[c] = rr[c] != kEmptyRef && k[c] < r2;
+            for (int c = 0; c < kBW; ++c) h[c] = k[c] < r2;
             if (!take_children<kBW>(k, rr, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, lim);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
             if (vis) vis->nprims += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
-                float d2, w;
-                if (D == 2) {
-                    float4 p = ldn(bv.prims + s);
-                    float qx, qy;
-                    d2 = seg_d2<float>(p.x, p.y, p.z, p.w, x[0], x[1], qx, qy);
-                    w = sqrtf((p.z - p.x) * (p.z - p.x) + (p.w - p.y) * (p.w - p.y));
-                } else {
-                    float a[3], b[3], c[3], q[3];
-                    load_tri(bv.prims, s, a, b, c);
-                    d2 = tri_d2<float>(a, b, c, x, q);
-                    float e1[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]}, e2[3] = {c[0] - a[0], c[1] - a[1], c[2] - a[2]};
-                    float n0 = e1[1] * e2[2] - e1[2] * e2[1], n1 = e1[2] * e2[0] - e1[0] * e2[2], n2 = e1[0] * e2[1] - e1[1] * e2[0];
-                    w = 0.5f * sqrtf(n0 * n0 + n1 * n1 + n2 * n2);
-                }
-                if (!(d2 < r2) || !(w > 0.f)) continue;
+                const float w = neumann_weight<2>(bv, s, x, r2);
+                if (!(w > 0.f)) continue;
                 const int id = __ldg(bv.ids + s);
-                U4 u = philox(pid, wid, step, P_NKEY | (uint32_t)id, k0, k1);
-                const float uu = ((float)(u.x >> 8) + 1.f) * (1.0f / 16777216.0f);   // (0, 1]
-                const float key = -logf(uu) / w;
+                const float key = neumann_key(id, w, pid, wid, step, k0, k1);
                 W += w;
                 if (key < best_key || (key == best_key && id < best_id)) { best_key = key; best_slot = s; best_id = id; }
             }

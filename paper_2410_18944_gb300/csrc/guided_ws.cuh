@@ -435,8 +435,8 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
         WorkCursor cursor;
         for (;;) {
             if (!active && !exhausted) {
-                unsigned long long item = cursor.next<D>(src.work_ctr(), (warp - kWsServerWarps) * gridDim.x + blockIdx.x,
-                                                         W * gridDim.x, 32);
+                unsigned long long item = cursor.next(src.work_ctr(), (warp - kWsServerWarps) * gridDim.x + blockIdx.x,
+                                                      W * gridDim.x, D == 2 ? 0 : 32);
                 if (item >= src.total()) exhausted = true;
                 else if (src.start(w, item)) { active = true; nwalks++; }
             }

@@ -190,7 +190,7 @@ struct BatchSrc {
 
     __device__ __forceinline__ unsigned long long *work_ctr() const { return b.work_ctr; }
     __device__ __forceinline__ unsigned long long total() const { return b.total; }
-    __device__ __forceinline__ unsigned lanes() const { return 32; }
+    __device__ __forceinline__ unsigned lanes() const { return D == 2 ? 0 : 32; }
     __device__ __forceinline__ bool start(Walk<D> &w, unsigned long long item) const {
         const int s = find_seg(b.segs, b.nseg, item);
         const DevSeg sg = b.segs[s];
@@ -223,30 +223,33 @@ struct BatchSrc {
     __device__ __forceinline__ const float *b3(int j) const { return b.jobs[j].f.b3; }
 };
 
-// Walks per warp of a plain 3D launch of `total` walks on `warps` warps.  A
-// warp has four to eight queries in flight at a time, so more walks than that
-// amortise the step logic, but a warp that is left with many long walks holds
-// up the end of the launch: half the lanes where the launch has fewer than two
-// walks per lane.  The Neumann term runs per lane and wants all of them.
+// How a plain launch of `total` walks on `warps` warps hands out its items
+// (WorkCursor).  2D: 0, from the counter, so that a warp starts on consecutive
+// points and shares the nodes of their first step; a launch of less than one
+// walk per lane goes round the warps instead (32), which leaves each warp fewer
+// lanes to wait for (64-segment problem, 52k walks: see plain_walk_kernel).
+// 3D: round the warps, the lanes of a warp that hold walks: a warp has four to
+// eight queries in flight at a time, so more walks than that only amortise the
+// step logic, but a warp that is left with many long walks holds up the end of
+// the launch; half the lanes where there are fewer than two walks per lane.
 // Measured on one GB300, 16 / 32 lanes: genus-3 (27 walks per warp) 66 / 72
-// ms, icosphere (77 per warp) 83 / 79 ms, flux slab 26.7 / 23.5 ms.
+// ms, icosphere (77 per warp) 83 / 79 ms.
 inline int plain_lanes(const DevScene &s, unsigned long long total, long long warps) {
-    return s.dim == 2 || s.has_flux || total >= 64ull * (unsigned long long)warps ? 32 : 16;
+    const unsigned long long lanes = 32ull * (unsigned long long)warps;
+    if (s.dim == 2) return total <= lanes ? 32 : 0;
+    return total >= 2 * lanes ? 32 : 16;
 }
 
-// A lane's next work item.  2D: warp-aggregated from the launch's counter, so
-// a warp starts on consecutive points.  3D: the launch's first items go round
-// the warps (warp w's lane l takes item l * warps + w, `lanes` lanes of a warp
-// hold walks; the counter counts the items after those): long walks come in
-// runs of neighbouring points, or first where the launch is ordered, and a
-// warp that held a run of them would outlast all others.
+// A lane's next work item: from the launch's counter, warp-aggregated, after
+// (lanes > 0) the first items have gone round the warps (warp w's lane l takes
+// item l * warps + w; the counter then counts the items after those).  Long
+// walks come in runs of neighbouring points, or first where the launch is
+// ordered, and in 3D a warp that held a run of them would outlast all others.
 struct WorkCursor {
     bool first = true;
-    template <int D>
     __device__ __forceinline__ unsigned long long next(unsigned long long *ctr, unsigned warp, unsigned warps,
                                                        unsigned lanes) {
-        if (D == 2) return warp_fetch_add(ctr, true);
-        if (first) {
+        if (first && lanes > 0) {
             first = false;
             return (unsigned long long)(threadIdx.x & 31) * warps + warp;
         }
@@ -279,7 +282,7 @@ __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigne
     const unsigned warps = gridDim.x * (blockDim.x / 32), warp = (threadIdx.x / 32) * gridDim.x + blockIdx.x;
     for (;;) {
         if (!active && !exhausted) {
-            unsigned long long item = cursor.next<D>(src.work_ctr(), warp, warps, src.lanes());
+            unsigned long long item = cursor.next(src.work_ctr(), warp, warps, src.lanes());
             if (item >= src.total()) exhausted = true;
             else if (src.start(w, item)) { active = true; nwalks++; }
         }

@@ -38,7 +38,7 @@ struct WalkArgs {
     // take in this launch
     const uint32_t *order;
     unsigned *plen;
-    int lanes;                 // plain 3D walks: walks per warp (plain_lanes)
+    int lanes;                 // plain walks: plain_lanes
 };
 
 // what one step needs besides the walk state: the walk's scene and the
@@ -142,11 +142,19 @@ __device__ __forceinline__ void finish_walk(const WalkArgs &a, uint32_t pid, flo
 //   <N> = G(x, z) h(z) W / alpha,  G = ln(r / |z - x|) / 2 pi  (2D),
 //                                      (1 / |z - x| - 1 / r) / 4 pi  (3D),
 // h the flux along the normal into the domain, alpha = 1/2 on a Neumann point.
-template <int D>
-__device__ __forceinline__ float neumann_term(const Walk<D> &w, const DevScene &sc, float r, uint32_t k0,
-                                              uint32_t k1, int *err, Visits *vis) {
+// Lanes with `act` (3D: the whole warp calls).
+template <int D, bool kMulti>
+__device__ __forceinline__ float neumann_term(CoopWarp *sh, const Walk<D> &w, const DevScene &sc, bool act, float r,
+                                              uint32_t k0, uint32_t k1, int *err, Visits *vis) {
     float W;
-    const int js = neumann_pick<D>(sc.neu, w.x, r, w.pid, w.wid, (uint32_t)w.k, k0, k1, W, err, vis);
+    int js;
+    if constexpr (D == 2) {
+        js = neumann_pick(sc.neu, w.x, r, w.pid, w.wid, (uint32_t)w.k, k0, k1, W, err, vis);
+    } else {
+        const float ctr[3] = {__uint_as_float(w.pid), __uint_as_float(w.wid), __int_as_float(w.k)};
+        W = r * r;
+        js = coop_run<kCoopPick, kMulti>(*sh, sc, act, w.x, ctr, W, (int)k0, err, vis, k1);
+    }
     if (js < 0) return 0.f;
     U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_NEU, k0, k1);
     const float u0 = u01(u.x), u1 = u01(u.y);
@@ -287,13 +295,15 @@ __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const St
             if (!sc.has_flux) w.acc += w.T * S;
         }
     }
-    if (go) {
-        if (sc.has_flux) {
-            S -= neumann_term<D>(w, sc, r, a.key0, a.key1, a.err, vis);
+    const bool flux = go && sc.has_flux;
+    if (D == 2 ? flux : __any_sync(0xffffffffu, flux)) {
+        const float N = neumann_term<D, kMulti>(sh, w, sc, flux, r, a.key0, a.key1, a.err, vis);
+        if (flux) {
+            S -= N;
             w.acc += w.T * S;
         }
-        S *= roulette_scale(a, w.k);
     }
+    if (go) S *= roulette_scale(a, w.k);
     return ended;
 }
 
