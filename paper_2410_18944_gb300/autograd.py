@@ -40,7 +40,11 @@ def _fp(t):
 
 
 def _load_params(lib, field, tensors):
-    torch.cuda.current_stream().synchronize()
+    # the field's copies run on the legacy default stream, in order after work
+    # of torch's default stream; tensors of another stream have to be ready
+    stream = torch.cuda.current_stream()
+    if stream.cuda_stream != 0:
+        stream.synchronize()
     check(lib.wost_field_set_params(field._h, *[_fp(t) for t in tensors]))
 
 
@@ -78,7 +82,9 @@ class FieldLoss(torch.autograd.Function):
         grads = [torch.empty_like(t) for t in params]
         loss = C.c_float()
         check(lib.wost_train_grad(ctx.field._h, C.byref(_exec(lib)), C.byref(loss), *[_fp(g) for g in grads]))
-        return (None,) + tuple(gout * g for g in grads)
+        if torch.is_grad_enabled() and gout.requires_grad:   # a graph of the gradients is asked for
+            return (None,) + tuple(gout * g for g in grads)
+        return (None,) + tuple(g.mul_(gout) for g in grads)
 
 
 def field_loss(field, grid, W1, W2, W3, b3):

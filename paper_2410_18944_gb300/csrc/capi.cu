@@ -32,6 +32,8 @@ wost_status check_device(int device, const char *who) {
 }
 
 wost_status refresh_inference_copy(wost_field *f, cudaStream_t st);
+wost_status load_params_device(wost_field *f, const float *grid, const float *const *w, cudaStream_t st);
+wost_status train_grad_launch(wost_field *f, int dim, cudaStream_t st, long long off, bool loss_only, float *g_grid);
 wost_status train_launch(wost_field *f, int dim, cudaStream_t st, bool apply_adam, float *loss_out_dev,
                          long long off = -1);
 wost_status train_loss_launch(wost_field *f, int dim, cudaStream_t st, float *out_dev);
@@ -245,10 +247,30 @@ extern "C" wost_status wost_destroy_field(wost_field *f) {
     return WOST_OK;
 }
 
+// a pointer into memory of `device` (its own allocations, not managed or
+// peer memory), aligned to `align` bytes
+static bool on_device(const void *p, int device, size_t align) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 extern "C" wost_status wost_field_set_params(wost_field *f, const float *grid, const float *W1, const float *W2,
                                              const float *W3, const float *b3) {
     if (!f || !grid || !W1 || !W2 || !W3 || !b3) { set_error("wost_field_set_params: null argument"); return WOST_ERR_INVALID_ARG; }
     if (wost_status dc = check_device(f->device, "wost_field_set_params")) return dc;
+    const float *mlp[4] = {W1, W2, W3, b3};
+    bool dev = on_device(grid, f->device, 16);
+    for (const float *p : mlp) dev = dev && on_device(p, f->device, 4);
+    if (dev) {
+        wost_status rc = load_params_device(f, grid, mlp, 0);
+        if (rc != WOST_OK) return rc;
+        WOST_CUDA(cudaDeviceSynchronize());
+        return WOST_OK;
+    }
     const int H = f->desc.hidden, nin = f->desc.levels * f->desc.features;
     float *d = f->mlp32;
     WOST_CUDA(cudaMemcpy(f->grid32, grid, f->n_grid() * sizeof(float), cudaMemcpyDefault));
@@ -364,8 +386,11 @@ extern "C" wost_status wost_train_grad(wost_field *f, const wost_exec *exec, flo
     if (!f->rec || !f->rec_ctr) { set_error("wost_train_grad: no training records"); return WOST_ERR_INVALID_ARG; }
     cudaStream_t st = exec ? (cudaStream_t)exec->stream : 0;
     if (exec) f->t_samples = exec->train_samples;
-    wost_status rc = train_launch(f, f->desc.dim, st, false, nullptr);
+    // the grid's gradient is accumulated in the caller's array where it can be
+    const bool direct = g_grid && on_device(g_grid, f->device, 16);
+    wost_status rc = train_grad_launch(f, f->desc.dim, st, -1, false, direct ? g_grid : nullptr);
     if (rc != WOST_OK) return rc;
+    if (direct) g_grid = nullptr;
     if ((rc = read_loss(f, st, out_loss)) != WOST_OK) return rc;
     if ((rc = device_check(st)) != WOST_OK) return rc;
     const int H = f->desc.hidden, nin = f->desc.levels * f->desc.features;

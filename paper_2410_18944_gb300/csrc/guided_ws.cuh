@@ -188,22 +188,43 @@ __device__ __forceinline__ void zero_row(uint8_t *tile, int row, int C) {
     for (int c = 0; c < C; c += 8) *reinterpret_cast<uint4 *>(tile + cm_offset(row, c, C)) = make_uint4(0, 0, 0, 0);
 }
 
-// suffix pass of a finished recorded walk (Sec. 4.1): v_k = w_k v_{k+1} + S_k,
-// target of record k = |v_{k+1}|; appends the nrec records to the buffer
-// (or counts them as dropped when it is full)
+// Suffix pass of one finished recorded walk (Sec. 4.1): v_k = w_k v_{k+1} + S_k
+// from v_n = term, target of record k = |v_{k+1}|; appends the nrec records to
+// the buffer (or counts them as dropped when it is full).  The whole warp
+// calls with the same walk: 32 records at a time are loaded one per lane, the
+// recurrence runs down their (w, S) by shuffles, and each lane writes its
+// record.  (One lane walking its records back paid a memory round trip each
+// while the warp waited: star, batch of 4 walks per point, see
+// guided_walk_kernel.)
 __device__ __forceinline__ void end_recorded_walk(const RecDest &rd, const float *base, int nrec, float term) {
-    unsigned long long at = atomicAdd(rd.ctr, (unsigned long long)nrec);
-    bool keep = (long long)(at + nrec) <= rd.cap;
-    if (!keep) atomicAdd(rd.ctr + 1, (unsigned long long)nrec);
+    constexpr unsigned kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned long long at = 0;
+    if (lane == 0) {
+        at = atomicAdd(rd.ctr, (unsigned long long)nrec);
+        if ((long long)(at + nrec) > rd.cap) atomicAdd(rd.ctr + 1, (unsigned long long)nrec);
+    }
+    at = __shfl_sync(kFull, at, 0);
+    if ((long long)(at + nrec) > rd.cap) return;
     float v = term;
-    for (int k = nrec - 1; k >= 0; --k) {
-        const float4 *r = reinterpret_cast<const float4 *>(base + (size_t)k * kRecFloats);
-        float4 a = r[0], b = r[1], c = r[2];   // x0 x1 x2 v0 | v1 v2 n0 n1 | n2 q w S
-        float tgt = fabsf(v);
-        v = c.z * v + c.w;
-        if (keep) {
+    for (int top = nrec; top > 0; top -= 32) {
+        const int k = top - 1 - lane;   // lane 0 holds the last record of the run
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;   // x0 x1 x2 v0 | v1 v2 n0 n1 | n2 q w S
+        if (k >= 0) {
+            const float4 *r = reinterpret_cast<const float4 *>(base + (size_t)k * kRecFloats);
+            a = __ldcs(r);
+            b = __ldcs(r + 1);
+            c = __ldcs(r + 2);
+        }
+        float tgt = 0.f;
+        const int n = min(top, 32);
+        for (int j = 0; j < n; ++j) {
+            if (lane == j) tgt = fabsf(v);
+            v = __shfl_sync(kFull, c.z, j) * v + __shfl_sync(kFull, c.w, j);
+        }
+        if (k >= 0) {
             float4 *o = reinterpret_cast<float4 *>(rd.out + (size_t)(at + k) * kRecFloats);
-            float onN = (b.z != 0.f || b.w != 0.f || c.x != 0.f) ? 1.f : 0.f;
+            const float onN = (b.z != 0.f || b.w != 0.f || c.x != 0.f) ? 1.f : 0.f;
             o[0] = a;
             o[1] = b;
             o[2] = make_float4(c.x, onN, c.y, tgt);
@@ -425,12 +446,12 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
         const float area = D == 2 ? 2.f * WOST_PI : 4.f * WOST_PI;
         CoopWarp *sh = reinterpret_cast<CoopWarp *>(coop) + (D == 3 ? warp - kWsServerWarps : 0);
         Walk<D> w;
-        if (D == 3) {   // lanes without a walk take part in the groups' queries
-            w.job = 0;
-            w.prim = -1;
-            w.k = 0;
-            for (int i = 0; i < D; ++i) w.x[i] = 0.f;
-        }
+        // lanes without a walk take part in the groups' queries (3D) and in the
+        // suffix passes of the others
+        w.job = 0;
+        w.prim = -1;
+        w.k = 0;
+        for (int i = 0; i < D; ++i) w.x[i] = 0.f;
         bool active = false, exhausted = false, failed = false;
         WorkCursor cursor;
         for (;;) {
@@ -442,7 +463,8 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             }
             if (!__any_sync(0xffffffffu, active || !exhausted)) break;
             __syncwarp();
-            float r = 0.f, S = 0.f;
+            float r = 0.f, S = 0.f, gv = 0.f;
+            bool ended = false;
             // The decode needs only the walk's position: with kOverlap the
             // row is submitted first and the step's geometry runs while the
             // tile fills and decodes (a walk that then ends leaves its row
@@ -451,16 +473,40 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             auto geometry = [&]() {
                 if (D == 2 && !active) return;
                 nsteps += active;
-                float gv;
                 bool trunc = false;
                 if (step_geometry<D, kMulti>(sh, w, src.env(w), active, r, S, gv, trunc, &vis)) {
                     src.finish(w);
-                    if (o.record) end_recorded_walk(src.rec(w), scratch_row, w.k, gv);
+                    ended = true;
                     ntrunc += trunc;
                     active = false;
                 }
             };
-            if (!kOverlap) geometry();
+            // the suffix passes of the walks that have just ended (the whole
+            // warp; each lane's records stay in its scratch row till here)
+            auto suffix = [&](bool mine, float term) {
+                __syncwarp();
+                for (unsigned m = __ballot_sync(0xffffffffu, mine && w.k > 0); m; m &= m - 1u) {
+                    const int e = __ffs(m) - 1;
+                    const int nrec = __shfl_sync(0xffffffffu, w.k, e);
+                    const float t = __shfl_sync(0xffffffffu, term, e);
+                    const float *rows = o.scratch + (size_t)(slot - lane + e) * o.scratch_steps * kRecFloats;
+                    if constexpr (kMulti) {
+                        const RecDest mineRd = src.rec(w);
+                        RecDest rd;
+                        rd.out = reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(mineRd.out), e));
+                        rd.ctr = reinterpret_cast<unsigned long long *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(mineRd.ctr), e));
+                        rd.cap = __shfl_sync(0xffffffffu, mineRd.cap, e);
+                        end_recorded_walk(rd, rows, nrec, t);
+                    } else {
+                        end_recorded_walk(src.rec(w), rows, nrec, t);
+                    }
+                    __syncwarp();
+                }
+            };
+            if (!kOverlap) {
+                geometry();
+                if (o.record) suffix(ended, gv);
+            }
             const bool enc = active;
             if (!__any_sync(0xffffffffu, enc)) continue;
             // claim a quarter of a decode tile
@@ -477,7 +523,10 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             fence_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->full[b]);
-            if (kOverlap) geometry();
+            if (kOverlap) {
+                geometry();
+                if (o.record) suffix(ended, gv);
+            }
             // reconverge before polling: lanes without a step must not spin
             // on the barrier while the others' geometry runs
             __syncwarp();
@@ -522,7 +571,6 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
             if (live) {
                 if (zero_density) {
                     src.finish(w);
-                    if (o.record) end_recorded_walk(src.rec(w), scratch_row, w.k, S);
                     active = false;
                 } else {
                     if (o.record) {
@@ -536,6 +584,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
                     w.T *= wgt;
                 }
             }
+            if (o.record) suffix(live && zero_density, S);
             step_move<D, kMulti>(sh, w, src.env(w), live && !zero_density, nu, r, &vis);
         }
         if (failed) atomicOr(o.err, 2);

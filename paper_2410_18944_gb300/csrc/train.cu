@@ -527,6 +527,58 @@ wost_status refresh_inference_copy(wost_field *f, cudaStream_t st) {
     return refresh_weight_image(f, st);
 }
 
+// New parameters from device arrays in one pass: FP32 masters, FP16 grid copy
+// and cleared Adam state (then the weight image).  Copies, clears and the
+// conversion as calls of their own took 64 us of launches and, for a 3D field,
+// 127 us in all; one GB300, see wost_field_set_params.
+struct ParamSrc {
+    const float *grid, *w[4];   // W1, W2, W3, b3
+    int64_t end[4];             // prefix ends of the MLP parts
+};
+__global__ void load_params_kernel(ParamSrc s, float *g32, float *gm, float *gv, __half2 *g16, int64_t ng, float *m32,
+                                   float *mm, float *mv, int64_t nm, unsigned long long *step, int grid_blocks) {
+    if ((int)blockIdx.x >= grid_blocks) {
+        const int64_t i = (int64_t)(blockIdx.x - grid_blocks) * blockDim.x + threadIdx.x;
+        if (i == 0) *step = 0;
+        if (i >= nm) return;
+        int p = 0;
+        while (i >= s.end[p]) ++p;
+        m32[i] = s.w[p][i - (p ? s.end[p - 1] : 0)];
+        mm[i] = 0.f;
+        mv[i] = 0.f;
+        return;
+    }
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i + 4 <= ng) {
+        const float4 p = __ldcs(reinterpret_cast<const float4 *>(s.grid + i));
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4 *>(g32 + i) = p;
+        *reinterpret_cast<float4 *>(gm + i) = z;
+        *reinterpret_cast<float4 *>(gv + i) = z;
+        g16[i / 2] = __floats2half2_rn(p.x, p.y);
+        g16[i / 2 + 1] = __floats2half2_rn(p.z, p.w);
+    } else if (i < ng) {   // the ragged end (an even number of floats)
+        for (int j = 0; j < 2; ++j) {
+            g32[i + j] = s.grid[i + j];
+            gm[i + j] = 0.f;
+            gv[i + j] = 0.f;
+        }
+        g16[i / 2] = __floats2half2_rn(s.grid[i], s.grid[i + 1]);
+    }
+}
+
+wost_status load_params_device(wost_field *f, const float *grid, const float *const *w, cudaStream_t st) {
+    const int H = f->desc.hidden, nin = f->desc.levels * f->desc.features;
+    const int64_t ng = f->n_grid(), nm = f->n_mlp(), part[4] = {(int64_t)H * nin, (int64_t)H * H, (int64_t)f->nout * H, f->nout};
+    ParamSrc s{grid, {w[0], w[1], w[2], w[3]}, {}};
+    for (int k = 0; k < 4; ++k) s.end[k] = part[k] + (k ? s.end[k - 1] : 0);
+    const int gb = (int)((ng + 1023) / 1024), mb = (int)((nm + 255) / 256);
+    load_params_kernel<<<gb + mb, 256, 0, st>>>(s, f->grid32, f->grid_m, f->grid_v, f->grid16, ng, f->mlp32, f->mlp_m,
+                                                f->mlp_v, nm, f->adam_step(), gb);
+    WOST_CUDA(cudaGetLastError());
+    return refresh_weight_image(f, st);
+}
+
 // sums each privatised level's gradient copies into copy 0 and clears the
 // others (one thread per used entry of those levels)
 __global__ void priv_reduce_kernel(float2 *g, GradCopies gc) {
@@ -592,10 +644,13 @@ wost_status train_prepare(int dim) {
 }
 
 // gradient of the mean loss over the record buffer into f->grid_g / f->mlp_g
-// (loss_only: the loss alone, the gradient buffers untouched)
-wost_status train_grad_launch(wost_field *f, int dim, cudaStream_t st, long long off, bool loss_only = false) {
+// (loss_only: the loss alone, the gradient buffers untouched; g_grid: another
+// device array of the grid's size to take the grid's gradient)
+wost_status train_grad_launch(wost_field *f, int dim, cudaStream_t st, long long off, bool loss_only = false,
+                              float *g_grid = nullptr) {
+    if (!g_grid) g_grid = f->grid_g;
     if (!loss_only) {
-        WOST_CUDA(cudaMemsetAsync(f->grid_g, 0, f->n_grid() * sizeof(float), st));
+        WOST_CUDA(cudaMemsetAsync(g_grid, 0, f->n_grid() * sizeof(float), st));
         WOST_CUDA(cudaMemsetAsync(f->mlp_g, 0, f->n_mlp() * sizeof(float), st));
     }
     WOST_CUDA(cudaMemsetAsync(f->loss_acc, 0, sizeof(double), st));
@@ -608,7 +663,7 @@ wost_status train_grad_launch(wost_field *f, int dim, cudaStream_t st, long long
     a.c_fixed = f->t_c_fixed;
     a.reflect = f->t_reflect;
     a.e_sel = f->desc.e_sel;
-    a.g_grid = f->grid_g;
+    a.g_grid = g_grid;
     a.g_W1 = f->mlp_g;
     a.g_W2 = a.g_W1 + kHid * kFeat;
     a.g_W3 = a.g_W2 + kHid * kHid;
@@ -634,7 +689,7 @@ wost_status train_grad_launch(wost_field *f, int dim, cudaStream_t st, long long
         else train_kernel<3, kMaxKWide><<<num_sms(), b16, s16, st>>>(a);
     }
     if (!loss_only && a.gc.n > 0)
-        priv_reduce_kernel<<<(a.gc.start[a.gc.n] + 255) / 256, 256, 0, st>>>(reinterpret_cast<float2 *>(f->grid_g), a.gc);
+        priv_reduce_kernel<<<(a.gc.start[a.gc.n] + 255) / 256, 256, 0, st>>>(reinterpret_cast<float2 *>(g_grid), a.gc);
     WOST_CUDA(cudaGetLastError());
     return WOST_OK;
 }

@@ -222,9 +222,9 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
     flush_stats(o.stat, nsteps, ntrunc, nwalks, vis);
 }
 
-// suffix passes of the walks of a recording launch (one per slot)
+// suffix passes of the walks of a recording launch (one per slot, a warp each)
 __global__ void wf_suffix_kernel(RecDest rd, const float *scratch, int scratch_steps, const int2 *ended, int n) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     if (s >= n) return;
     const int2 e = ended[s];
     if (e.x > 0)
@@ -388,7 +388,7 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
         }
     }
     if (o.record) {
-        wf_suffix_kernel<<<(nslots + 255) / 256, 256, 0, st>>>(rd, o.scratch, o.scratch_steps, S.ended, nslots);
+        wf_suffix_kernel<<<(nslots + 7) / 8, 256, 0, st>>>(rd, o.scratch, o.scratch_steps, S.ended, nslots);
         WOST_CUDA(cudaGetLastError());
         ++it;
     }
