@@ -90,45 +90,36 @@ __device__ __forceinline__ void node_keys_ray(const float4 *nodes, int node, con
     kk[1] = e1 <= x1 ? e1 : __int_as_float(0x7f800000);
 }
 
-// Continue at the nearest child with h[c] (ties: the lower child index) and
-// push the others, farthest first.  Returns false if no child is taken.
-template <int kBW>
-__device__ __forceinline__ bool take_children(const float *k, const int *r, const bool *h, int &ref, int *stack,
-                                              float *skey, int &sp, int *err) {
-    float kk[kBW];
-    int rr[kBW], n = 0;
-#pragma unroll
-    for (int c = 0; c < kBW; ++c) {
-        kk[c] = h[c] ? k[c] : __int_as_float(0x7f800000);
-        rr[c] = r[c];
-        n += h[c] ? 1 : 0;
+// Traversal stack of a lane (2D): key and node or leaf in one 8-byte entry
+struct LaneStack {
+    uint2 e[kStack];
+    int sp = 0;
+    __device__ __forceinline__ void push(float key, int ref, int *err) {
+        if (sp < kStack) e[sp++] = make_uint2(__float_as_uint(key), (unsigned)ref);
+        else atomicOr(err, 1);
     }
-    if (n == 0) return false;
-    auto cs = [&](int i, int j) {
-        if (kk[j] < kk[i]) {
-            float tk = kk[i]; kk[i] = kk[j]; kk[j] = tk;
-            int tr = rr[i]; rr[i] = rr[j]; rr[j] = tr;
+    // the top entry whose key is within best; false if there is none
+    __device__ __forceinline__ bool pop(float best, int &ref) {
+        while (sp > 0) {
+            const uint2 t = e[--sp];
+            if (__uint_as_float(t.x) <= best) { ref = (int)t.y; return true; }
         }
-    };
-    if (kBW == 2) {
-        cs(0, 1);
-    } else {
-        cs(0, 1); cs(2, 3); cs(0, 2); cs(1, 3); cs(1, 2);
+        return false;
     }
-#pragma unroll
-    for (int i = kBW - 1; i >= 1; --i) {
-        if (i < n) {
-            if (sp < kStack) {
-                stack[sp] = rr[i];
-                skey[sp] = kk[i];
-                ++sp;
-            } else {
-                atomicOr(err, 1);
-            }
-        }
+};
+
+// Continue at the nearer of the two children with h[c] (ties: the first) and
+// push the other.  Returns false if no child is taken.
+__device__ __forceinline__ bool take_children(const float *k, const int *r, const bool *h, int &ref, LaneStack &st,
+                                              int *err) {
+    if (h[0] && h[1]) {
+        const bool second = k[1] < k[0];
+        st.push(second ? k[0] : k[1], second ? r[0] : r[1], err);
+        ref = second ? r[1] : r[0];
+        return true;
     }
-    ref = rr[0];
-    return true;
+    if (h[0] || h[1]) ref = h[0] ? r[0] : r[1];
+    return h[0] || h[1];
 }
 
 // ---- oriented caps ------------------------------------------------------------
@@ -289,16 +280,6 @@ __device__ __forceinline__ void load_tri(const float4 *__restrict__ P, int s, fl
 // pops its stack if needed.  Lanes that diverge inside an iteration
 // re-converge at its end, instead of drifting apart for the rest of the
 // traversal.
-#define WOST_POP(stack, sd, sp, ref, done, best)               \
-    do {                                                       \
-        bool found_ = false;                                   \
-        while (sp > 0) {                                       \
-            --sp;                                              \
-            if (sd[sp] <= best) { ref = stack[sp]; found_ = true; break; } \
-        }                                                      \
-        if (!found_) done = true;                              \
-    } while (0)
-
 // ---- closest Dirichlet primitive (2D) ---------------------------------------
 // returns the leaf slot of the closest primitive (-1 if none); best = squared distance
 __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const float4 *caps, const float *x, float &best,
@@ -308,9 +289,8 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
     int best_slot = -1, best_id = 0x7fffffff;
-    int stack[kStack];
-    float sd[kStack];
-    int sp = 0, ref = 0;
+    LaneStack st;
+    int ref = 0;
     bool done = false;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
@@ -329,7 +309,7 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
             if (vis) vis->nodes++;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
-            if (!take_children<kBW>(k, r, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, best);
+            if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
@@ -342,7 +322,7 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
                     if (d2 < best || id < best_id) { best = d2; best_slot = s; best_id = id; }
                 }
             }
-            WOST_POP(stack, sd, sp, ref, done, best);
+            done = !st.pop(best, ref);
         }
     }
     return best_slot;
@@ -452,9 +432,8 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
     int best_slot = -1, best_id = 0x7fffffff;
-    int stack[kStack];
-    float sd[kStack];
-    int sp = 0, ref = 0;
+    LaneStack st;
+    int ref = 0;
     bool done = false;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
@@ -466,7 +445,7 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
             bool h[kBW];
             node_keys_sil(bv.nodes, facing, ref, x, best, tau, k, r, h);
             if (vis) vis->nodes++;
-            if (!take_children<kBW>(k, r, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, best);
+            if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
@@ -478,7 +457,7 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
                     if (d2 < best || id < best_id) { best = d2; best_slot = s; best_id = id; }
                 }
             }
-            WOST_POP(stack, sd, sp, ref, done, best);
+            done = !st.pop(best, ref);
         }
     }
     return best_slot;
@@ -600,9 +579,8 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
     for (int k = 0; k < 2; ++k) inv[k] = 1.f / v[k];   // +-inf for a zero component is fine in the slab test
     float best = tmax;
     int best_slot = -1, best_id = 0x7fffffff;
-    int stack[kStack];
-    float st[kStack];
-    int sp = 0, ref = 0;
+    LaneStack st;
+    int ref = 0;
     bool done = false;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
@@ -616,7 +594,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
             if (vis) vis->nodes++;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
-            if (!take_children<kBW>(k, r, h, ref, stack, st, sp, err)) WOST_POP(stack, st, sp, ref, done, best);
+            if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
@@ -628,7 +606,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
                     if (t < best || id < best_id) { best = t; best_slot = s; best_id = id; }
                 }
             }
-            WOST_POP(stack, st, sp, ref, done, best);
+            done = !st.pop(best, ref);
         }
     }
     thit = best;
@@ -680,11 +658,10 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
     const unsigned mask = __activemask();
     int best_slot = -1, best_id = 0x7fffffff;
     float best_key = __int_as_float(0x7f800000);
-    int stack[kStack];
-    float sd[kStack];
-    int sp = 0, ref = 0;
+    LaneStack st;
+    int ref = 0;
     bool done = false;
-    float lim = r2;   // the search radius never shrinks: WOST_POP compares keys with it
+    const float lim = r2;   // the search radius never shrinks
     while (__any_sync(mask, !done)) {
         while (__any_sync(mask, !done && ref >= 0)) {
             if (done || ref < 0) continue;
@@ -695,7 +672,7 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
             if (vis) vis->nodes++;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] < r2;
-            if (!take_children<kBW>(k, rr, h, ref, stack, sd, sp, err)) WOST_POP(stack, sd, sp, ref, done, lim);
+            if (!take_children(k, rr, h, ref, st, err)) done = !st.pop(lim, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
@@ -708,7 +685,7 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
                 W += w;
                 if (key < best_key || (key == best_key && id < best_id)) { best_key = key; best_slot = s; best_id = id; }
             }
-            WOST_POP(stack, sd, sp, ref, done, lim);
+            done = !st.pop(lim, ref);
         }
     }
     return best_slot;
@@ -723,8 +700,8 @@ __device__ inline int ray_count(const DevBVH &bv, const float *o, const float *v
 #pragma unroll
     for (int k = 0; k < 2; ++k) inv[k] = 1.f / v[k];
     const float big = 3.0e38f;
-    int cnt = 0, stack[kStack], sp = 0, ref = 0;
-    float skey[kStack];
+    int cnt = 0, ref = 0;
+    LaneStack st;
     bool done = false;
     while (__any_sync(mask, !done)) {
         if (done) continue;
@@ -736,7 +713,7 @@ __device__ inline int ray_count(const DevBVH &bv, const float *o, const float *v
             node_keys_ray(bv.nodes, ref, o, inv, big, k, r, 0.f);
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] <= big;
-            if (!take_children<kBW>(k, r, h, ref, stack, skey, sp, err)) pop = true;
+            if (!take_children(k, r, h, ref, st, err)) pop = true;
         } else {
             int s0 = leaf_start(ref), c = leaf_count(ref);
             for (int s = s0; s < s0 + c; ++s) {
@@ -745,10 +722,7 @@ __device__ inline int ray_count(const DevBVH &bv, const float *o, const float *v
             }
             pop = true;
         }
-        if (pop) {
-            if (sp == 0) done = true;
-            else ref = stack[--sp];
-        }
+        if (pop) done = !st.pop(big, ref);
     }
     return cnt;
 }

@@ -376,9 +376,20 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
                     float w[1 << D];
                     level_corners<D>(a.f, l, u, idx, w);
                     const size_t lo = (size_t)a.f.level_off[l] + copy_off[l];
-                    for (int m = 0; m < (1 << D); ++m) {
-                        float *gp = a.g_grid + (lo + idx[m]) * 2;
-                        atomicAdd(reinterpret_cast<float2 *>(gp), make_float2(w[m] * dx[2 * l], w[m] * dx[2 * l + 1]));
+                    // corners along x that share an aligned pair of entries
+                    // (half of them, see encode_row_pairs) take one 16-byte add
+                    for (int m = 0; m < (1 << D); m += 2) {
+                        const size_t i0 = lo + idx[m], i1 = lo + idx[m + 1];
+                        const float2 v0 = make_float2(w[m] * dx[2 * l], w[m] * dx[2 * l + 1]);
+                        const float2 v1 = make_float2(w[m + 1] * dx[2 * l], w[m + 1] * dx[2 * l + 1]);
+                        if ((i0 ^ i1) == 1) {
+                            const bool odd = i0 & 1;
+                            atomicAdd(reinterpret_cast<float4 *>(a.g_grid) + (i0 >> 1),
+                                      make_float4(odd ? v1.x : v0.x, odd ? v1.y : v0.y, odd ? v0.x : v1.x, odd ? v0.y : v1.y));
+                        } else {
+                            atomicAdd(reinterpret_cast<float2 *>(a.g_grid) + i0, v0);
+                            atomicAdd(reinterpret_cast<float2 *>(a.g_grid) + i1, v1);
+                        }
                     }
                 }
             }

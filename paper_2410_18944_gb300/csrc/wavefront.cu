@@ -41,6 +41,7 @@ constexpr int kWfChunk = 8;             // iterations between host checks
 // 3D: walks per warp of the step kernel (icosphere, 64k walks: 109 / 79 / 67 ms
 // with 32 / 16 / 8)
 constexpr int kWfLanes3 = 8;
+constexpr unsigned kWfMinLanes(int d) { return d == 2 ? 4 : 1; }
 constexpr int wf_walks_per_block(int d) { return kWfBlock / 32 * (d == 2 ? 32 : kWfLanes3); }
 
 // Iteration k's step kernel reads the decode list of iteration k-1 (entry j
@@ -58,7 +59,7 @@ struct WfSlots {
     __half *theta;     // [rows][kThetaStride] decoded outputs of the last list
     int2 *ended;       // recording launches: (records, terminal value bits) of the slot's ended walk
     int nslots;
-    int warps;         // 3D: warps of the step kernel the GPU holds at once
+    int warps;         // warps of the step kernel the GPU holds at once
 };
 
 struct WfSoloArgs {
@@ -99,13 +100,11 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
     // one thread per entry of the previous iteration's decode list (or per
     // slot in the first iteration); blocks past the list's end leave at once
     const unsigned n_in = first ? (unsigned)S.nslots : S.dcount[parity ^ 1];
-    // 3D: at most kWfLanes3 entries per warp, fewer once the list is short
-    // (a warp answers four to eight queries at a time, coop.cuh)
-    unsigned L = 32;
-    if (D == 3) {
-        L = kWfLanes3;
-        while (L > 1 && n_in * 2u <= L * (unsigned)S.warps) L >>= 1;
-    }
+    // entries per warp: 32 (2D) or kWfLanes3 (3D: a warp answers four to eight
+    // queries at a time, coop.cuh), fewer once the list is short, so that a
+    // warp waits for fewer walks
+    unsigned L = D == 2 ? 32 : kWfLanes3;
+    while (L > kWfMinLanes(D) && n_in * 2u <= L * (unsigned)S.warps) L >>= 1;
     const unsigned j = (blockIdx.x * (kWfBlock / 32) + threadIdx.x / 32) * L + threadIdx.x % 32;
     if (blockIdx.x * (kWfBlock / 32) * L >= n_in) return;
     const bool valid = threadIdx.x % 32 < L && j < n_in;
@@ -341,6 +340,7 @@ wost_status wavefront_run(wost_scene *sc, wost_field *f, const WalkArgs &a, cons
             if (D == 2) {
                 WOST_CUDA(cudaFuncSetAttribute(wf_decode_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCtaTilesSmem));
                 grid_dec[D] = occupancy_grid(wf_decode_kernel<2>, 256, kCtaTilesSmem);
+                step_warps[D] = occupancy_grid(wf_step_kernel<2>, kWfBlock, 0) * (kWfBlock / 32);
             } else {
                 WOST_CUDA(cudaFuncSetAttribute(wf_decode_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCtaTilesSmem));
                 grid_dec[D] = occupancy_grid(wf_decode_kernel<3>, 256, kCtaTilesSmem);
