@@ -182,13 +182,15 @@ __device__ __forceinline__ void encode_row(const DevField &f, const float *x, ui
 // training step's two passes over 2^18 3D records 1473 -> 1338 us per call).  Costs 8 more registers per
 // level in flight, which the walkers of the warp-specialised kernel do not
 // have.  Same features bit for bit: the corners are added in the same order.
+// (levels [first, last), multiples of four)
 template <int D>
-__device__ __forceinline__ void encode_row_pairs(const DevField &f, const float *x, uint8_t *xtile, int row) {
+__device__ __forceinline__ void encode_row_pairs(const DevField &f, const float *x, uint8_t *xtile, int row, int first = 0,
+                                                 int last = kMaxLevels) {
     float u[D];
     unit_coords<D>(f, x, u);
     constexpr int P = 1 << (D - 1);
 #pragma unroll 1
-    for (int l4 = 0; l4 < kMaxLevels; l4 += 4) {
+    for (int l4 = first; l4 < last; l4 += 4) {
         float feat[8];
 #pragma unroll
         for (int h = 0; h < 4; h += 2) {

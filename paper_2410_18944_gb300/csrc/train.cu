@@ -43,7 +43,12 @@ __host__ __device__ constexpr int tile_bytes(int KM) { return kTX + 2 * kTH + 2 
 // 128-record tiles per CTA: two for KM = 8 (226 KB of shared memory); one for
 // KM = 16, whose tile and TMEM columns (128 + 3 x 64) do not fit twice
 __host__ __device__ constexpr int train_tiles(int KM) { return KM <= kMaxK ? 2 : 1; }
-__host__ __device__ constexpr int train_block(int KM) { return 128 * train_tiles(KM); }
+// Two threads per record: thread `half` of a row takes half of the levels,
+// hidden columns and lobes.  The tiles leave room for one CTA per SM, and with
+// one thread per record its 8 warps left the SM idle 84% of the time behind
+// the chain of gathers, MMAs and atomics; 16 warps also halve each thread's
+// part of that chain.
+__host__ __device__ constexpr int train_block(int KM) { return 256 * train_tiles(KM); }
 // TMEM columns of the scratch accumulator s0 of a tile (the layer-3 outputs)
 __host__ __device__ constexpr int s0cols(int KM) { return tile_tmem_cols(KM); }
 constexpr int kTrainCtl = 128;   // mbarriers, TMEM address, per-level gradient copy offsets
@@ -115,7 +120,7 @@ template <class F>
 __device__ __forceinline__ bool tt_issue_wait(TTile &t, bool issuer, F issue, int *err) {
     fence_async_smem();
     tc_fence_before();
-    named_sync(t.bar, 128);
+    named_sync(t.bar, 256);
     if (issuer) {
         tc_fence_after();
         issue();
@@ -124,8 +129,8 @@ __device__ __forceinline__ bool tt_issue_wait(TTile &t, bool issuer, F issue, in
     bool ok = mbar_wait_bounded(t.mbar, t.phase);
     t.phase ^= 1u;
     tc_fence_after();
-    ok = !named_or(t.bar, 128, !ok);   // tile-uniform give-up decision
-    if (!ok && (threadIdx.x & 127) == 0) atomicOr(err, 2);
+    ok = !named_or(t.bar, 256, !ok);   // tile-uniform give-up decision
+    if (!ok && (threadIdx.x & 255) == 0) atomicOr(err, 2);
     return ok;
 }
 
@@ -141,6 +146,22 @@ __device__ __forceinline__ void st_row8_split(uint8_t *hi, uint8_t *lo, int r, i
     st_row8_bf16(lo, r, c8, C, l);
 }
 
+// 4 values of a row (half a core-matrix row), likewise
+__device__ __forceinline__ void st_row4_split(uint8_t *hi, uint8_t *lo, int r, int c4, int C, const float *v) {
+    float l[4];
+    __nv_bfloat162 h[2], q[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        const float2 f = __bfloat1622float2(h[i]);
+        l[2 * i] = v[2 * i] - f.x;
+        l[2 * i + 1] = v[2 * i + 1] - f.y;
+        q[i] = __floats2bfloat162_rn(l[2 * i], l[2 * i + 1]);
+    }
+    *reinterpret_cast<uint2 *>(hi + cm_offset(r, c4, C)) = *reinterpret_cast<const uint2 *>(h);
+    *reinterpret_cast<uint2 *>(lo + cm_offset(r, c4, C)) = *reinterpret_cast<const uint2 *>(q);
+}
+
 __device__ __forceinline__ void ld_cols(uint32_t taddr, int row, int ncols, float *v) {
     for (int c = 0; c < ncols; c += 16) {
         tmem_ld16(lane_addr(taddr, row, c), v + c);
@@ -148,77 +169,119 @@ __device__ __forceinline__ void ld_cols(uint32_t taddr, int row, int ncols, floa
     }
 }
 
-// loss and gradient w.r.t. the raw outputs (internal layout of KM lobes) for
-// one record
+// Loss and gradient w.r.t. the raw outputs of one record, for one half of the
+// lobes (internal layout of KM lobes): lobes [half KH, half KH + KH), KH = KM / 2;
+// half 0 also takes the selection logit and the loss.  mu, kap: this half's
+// raw outputs; lam: all lobes'; c: the logit.  Returns pg's share in `part`;
+// the caller adds the other half's and calls finish.
 template <int D, int KM>
-__device__ __forceinline__ float record_grad(const TrainArgs &a, const float *rec, const float *raw, float inv_n,
-                                             float *draw) {
-    constexpr int K = KM;
-    Mixture<D, KM> m;
-    theta_map<D, KM>(raw, m);
-    const float c = a.c_mode ? a.c_fixed : m.c;
-    float nu[2][3], nrm[3];
-    for (int i = 0; i < 3; ++i) { nu[0][i] = rec[3 + i]; nrm[i] = rec[6 + i]; }
-    const bool onN = rec[9] != 0.f;
-    const float q = rec[10], pt = rec[11];
-    int nd = 1;
-    if (onN && a.reflect) {
-        float t = 2.f * (nu[0][0] * nrm[0] + nu[0][1] * nrm[1] + (D == 3 ? nu[0][2] * nrm[2] : 0.f));
-        for (int i = 0; i < D; ++i) nu[1][i] = nu[0][i] - t * nrm[i];
-        nd = 2;
-    }
-    float v[2][KM], pg = 0.f;
+struct RecordGrad {
+    static constexpr int KH = KM / 2;
+    float mu[KH * D], inv[KH], kappa[KH], kp[KH], lam[KH], v[2][KH];
+    float nu[2][D], c, pu, wt;
+    int nd;
+    bool live;
+
+    __device__ __forceinline__ float part(const TrainArgs &a, const float *rec, const float *rmu, const float *rkap,
+                                          const float *rlam, float rc, int half) {
+        // normalisation map (Tab. reg_map, theta_map)
+        float mx = rlam[0];
 #pragma unroll
-    for (int j = 0; j < K; ++j) {
+        for (int i = 1; i < KM; ++i) mx = fmaxf(mx, rlam[i]);
         float s = 0.f;
-        for (int d2 = 0; d2 < nd; ++d2) {
-            v[d2][j] = __expf(m.lognorm[j] - m.kappa[j] * half_dist2<D>(m.mu + j * D, nu[d2]));
-            s += v[d2][j];
-        }
-        pg += m.lam[j] * s;
-    }
-    const float area = D == 2 ? 2.f * WOST_PI : 4.f * WOST_PI;
-    const float pu = (onN ? 2.f : 1.f) / area;
-    const float ptil = c * pg + (1.f - c) * pu;
-    for (int i = 0; i < out_pad(KM); ++i) draw[i] = 0.f;
-    if (!(pt > 0.f) || !(q > 0.f)) return 0.f;
-    const float wt = pt / q;
-    const float pgs = fmaxf(pg, 1e-30f);
-    float loss = -wt * (__logf(pgs) + (a.c_mode == 0 ? a.e_sel * __logf(ptil) : 0.f));
-    const float dpg = -wt / pgs * inv_n;
 #pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const float *mu = m.mu + j * D;
-        float sj = 0.f, dk = 0.f, dm[3] = {0.f, 0.f, 0.f};
-        const float A = vmf_mean_cos<D>(m.kappa[j]);
-        for (int d2 = 0; d2 < nd; ++d2) {
-            float cm = 0.f;
-            for (int i = 0; i < D; ++i) cm += mu[i] * nu[d2][i];
-            sj += v[d2][j];
-            dk += v[d2][j] * (cm - A);
-            for (int i = 0; i < D; ++i) dm[i] += v[d2][j] * (nu[d2][i] - cm * mu[i]);
+        for (int i = 0; i < KM; ++i) {
+            const float e = __expf(rlam[i] - mx);
+            s += e;
+            if (i < KH && half == 0) lam[i % KH] = e;
+            if (i >= KH && half == 1) lam[i % KH] = e;
         }
-        draw[K * D + K + j] = dpg * m.lam[j] * (sj - pg);
-        float kp = raw[K * D + j];
-        if (kp > -8.f && kp < 8.f) draw[K * D + j] = dpg * m.lam[j] * m.kappa[j] * dk;
-        float nn = 0.f;
-        for (int i = 0; i < D; ++i) nn += raw[j * D + i] * raw[j * D + i];
-        if (nn > 0.f) {
-            float inv = rsqrtf(nn);
-            for (int i = 0; i < D; ++i) draw[j * D + i] = dpg * m.lam[j] * m.kappa[j] * dm[i] * inv;
+        const float is = 1.f / s;
+        c = a.c_mode ? a.c_fixed : 1.f / (1.f + __expf(-rc));
+        const bool onN = rec[9] != 0.f;
+        nd = 1;
+#pragma unroll
+        for (int i = 0; i < D; ++i) nu[0][i] = nu[1][i] = rec[3 + i];
+        if (onN && a.reflect) {
+            const float t = 2.f * (rec[3] * rec[6] + rec[4] * rec[7] + (D == 3 ? rec[5] * rec[8] : 0.f));
+#pragma unroll
+            for (int i = 0; i < D; ++i) nu[1][i] = rec[3 + i] - t * rec[6 + i];
+            nd = 2;
         }
+        const float area = D == 2 ? 2.f * WOST_PI : 4.f * WOST_PI;
+        pu = (onN ? 2.f : 1.f) / area;
+        live = rec[11] > 0.f && rec[10] > 0.f;
+        wt = live ? rec[11] / rec[10] : 0.f;
+        float pg = 0.f;
+#pragma unroll
+        for (int j = 0; j < KH; ++j) {
+            lam[j] *= is;
+            float n2 = 0.f;
+#pragma unroll
+            for (int i = 0; i < D; ++i) n2 += rmu[j * D + i] * rmu[j * D + i];
+            inv[j] = n2 > 0.f ? rsqrtf(n2) : 0.f;
+#pragma unroll
+            for (int i = 0; i < D; ++i) mu[j * D + i] = n2 > 0.f ? rmu[j * D + i] * inv[j] : (i == 0 ? 1.f : 0.f);
+            kp[j] = rkap[j];
+            kappa[j] = __expf(fminf(fmaxf(kp[j], -8.f), 8.f));
+            const float ln = vmf_lognorm<D>(kappa[j]);
+            v[0][j] = __expf(ln - kappa[j] * half_dist2<D>(mu + j * D, nu[0]));
+            v[1][j] = nd == 2 ? __expf(ln - kappa[j] * half_dist2<D>(mu + j * D, nu[1])) : 0.f;
+            pg += lam[j] * (v[0][j] + v[1][j]);
+        }
+        return pg;
     }
-    if (a.c_mode == 0) draw[K * (D + 2)] = -a.e_sel * wt * (pg - pu) / ptil * inv_n * c * (1.f - c);
-    return loss;
-}
+
+    // pg: of all lobes.  dmu, dkap, dlam: gradients of this half's outputs; dc
+    // and the returned loss are half 0's (0 on the other).
+    __device__ __forceinline__ float finish(const TrainArgs &a, float pg, float inv_n, int half, float *dmu, float *dkap,
+                                            float *dlam, float &dc) {
+        dc = 0.f;
+#pragma unroll
+        for (int j = 0; j < KH; ++j) {
+            dkap[j] = dlam[j] = 0.f;
+#pragma unroll
+            for (int i = 0; i < D; ++i) dmu[j * D + i] = 0.f;
+        }
+        if (!live) return 0.f;
+        const float ptil = c * pg + (1.f - c) * pu;
+        const float pgs = fmaxf(pg, 1e-30f);
+        const float dpg = -wt / pgs * inv_n;
+#pragma unroll
+        for (int j = 0; j < KH; ++j) {
+            const float *m = mu + j * D;
+            float sj = 0.f, dk = 0.f, dm[D] = {};
+            const float A = vmf_mean_cos<D>(kappa[j]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (q >= nd) continue;
+                float cm = 0.f;
+#pragma unroll
+                for (int i = 0; i < D; ++i) cm += m[i] * nu[q][i];
+                sj += v[q][j];
+                dk += v[q][j] * (cm - A);
+#pragma unroll
+                for (int i = 0; i < D; ++i) dm[i] += v[q][j] * (nu[q][i] - cm * m[i]);
+            }
+            dlam[j] = dpg * lam[j] * (sj - pg);
+            if (kp[j] > -8.f && kp[j] < 8.f) dkap[j] = dpg * lam[j] * kappa[j] * dk;
+#pragma unroll
+            for (int i = 0; i < D; ++i) dmu[j * D + i] = dpg * lam[j] * kappa[j] * dm[i] * inv[j];
+        }
+        if (half) return 0.f;
+        if (a.c_mode == 0) dc = -a.e_sel * wt * (pg - pu) / ptil * inv_n * c * (1.f - c);
+        return -wt * (__logf(pgs) + (a.c_mode == 0 ? a.e_sel * __logf(ptil) : 0.f));
+    }
+};
 
 template <int D, int KM>
 __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) {
     constexpr int TPC = train_tiles(KM), OUT = out_pad(KM), GC = gcols(KM), Z2 = z2col(KM), S0C = s0cols(KM);
     constexpr int kImg = wimg_bytes(KM), kTileB = tile_bytes(KM);
     extern __shared__ __align__(1024) uint8_t sm[];
-    const int tid = threadIdx.x, tl = tid >> 7, row = tid & 127;
-    const bool issuer = row == 0;
+    const int tid = threadIdx.x, tl = tid >> 8, half = (tid >> 7) & 1, row = tid & 127;
+    const bool issuer = (tid & 255) == 0;
+    constexpr int KH = KM / 2, HC = kHid / 2;
     uint8_t *wimg = sm;
     uint8_t *tb = sm + kImg + tl * kTileB;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(sm + kImg + TPC * kTileB);
@@ -266,43 +329,82 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
             rec[0] = r0.x; rec[1] = r0.y; rec[2] = r0.z; rec[3] = r0.w;
             rec[4] = r1.x; rec[5] = r1.y; rec[6] = r1.z; rec[7] = r1.w;
             rec[8] = r2.x; rec[9] = r2.y; rec[10] = r2.z; rec[11] = r2.w;
-            // (the 16-lobe kernel has no registers for the pairs: 968 -> 1012 us)
-            if constexpr (KM <= kMaxK) encode_row_pairs<D>(a.f, rec, t.X, row);
-            else encode_row<D>(a.f, rec, t.X, row);
+            encode_row_pairs<D>(a.f, rec, t.X, row, half * (kMaxLevels / 2), (half + 1) * (kMaxLevels / 2));
         } else {
             for (int i = 0; i < 12; ++i) rec[i] = 0.f;
-            for (int c = 0; c < kFeat; c += 8) *reinterpret_cast<uint4 *>(t.X + cm_offset(row, c, kFeat)) = make_uint4(0, 0, 0, 0);
+            for (int c = half * (kFeat / 2); c < (half + 1) * (kFeat / 2); c += 8) *reinterpret_cast<uint4 *>(t.X + cm_offset(row, c, kFeat)) = make_uint4(0, 0, 0, 0);
         }
         // ---- forward recomputation ----
         ok = tt_issue_wait(t, issuer, [&] { umma_gemm(t.s0, t.X, 0, kFeat, t.w, 0, kFeat, kHid, kFeat, false); }, a.err);
         if (!ok) break;
-        float h[kHid];
-        ld_cols(t.s0, row, kHid, h);
-        for (int c = 0; c < kHid; c += 8) {
+        // (this thread's half of the hidden columns)
+        const int hc = half * HC;
+        float h[HC];
+        ld_cols(t.s0 + hc, row, HC, h);
+        for (int c = 0; c < HC; c += 8) {
             float v8[8];
             for (int i = 0; i < 8; ++i) v8[i] = fmaxf(h[c + i], 0.f);
-            st_row8_bf16(t.H1, row, c, kHid, v8);
+            st_row8_bf16(t.H1, row, hc + c, kHid, v8);
         }
         ok = tt_issue_wait(t, issuer, [&] { umma_gemm(t.s0, t.H1, 0, kHid, t.w + kW1Bytes, 0, kHid, kHid, kHid, false); }, a.err);
         if (!ok) break;
-        ld_cols(t.s0, row, kHid, h);
-        for (int c = 0; c < kHid; c += 8) {
+        ld_cols(t.s0 + hc, row, HC, h);
+        for (int c = 0; c < HC; c += 8) {
             float v8[8];
             for (int i = 0; i < 8; ++i) v8[i] = fmaxf(h[c + i], 0.f);
-            st_row8_bf16(t.H2, row, c, kHid, v8);
+            st_row8_bf16(t.H2, row, hc + c, kHid, v8);
         }
         ok = tt_issue_wait(t, issuer, [&] { umma_gemm(t.s0, t.H2, 0, kHid, t.w + kW1Bytes + kW2Bytes, 0, kHid, OUT, kHid, false); }, a.err);
         if (!ok) break;
-        float raw[OUT];
-        ld_cols(t.s0, row, OUT, raw);
-        for (int i = 0; i < OUT; ++i) raw[i] += __ldg(a.f.b3 + i);
-        // ---- loss gradient at the raw outputs ----
-        float dy[OUT];
-        if (valid) loss_local += record_grad<D, KM>(a, rec, raw, inv_n, dy);
-        else for (int i = 0; i < OUT; ++i) dy[i] = 0.f;
-        if (a.loss_only) continue;   // uniform over the tile: no backward pass
-        for (int c = 0; c < OUT; c += 8) st_row8_split(t.G, t.Gl, row, c, GC, dy + c);
+        // ---- loss gradient at the raw outputs: this half's lobes ----
+        const int cmu = half * KH * D, ckap = KM * D + half * KH, clam = KM * D + KM, cc = KM * (D + 2);
+        RecordGrad<D, KM> g;
+        float pg = 0.f;
         {
+            float rmu[KH * D], rkap[KH], rlam[KM], rc[4];
+#pragma unroll
+            for (int c = 0; c < KH * D; c += 4) tmem_ld4(lane_addr(t.s0, row, cmu + c), rmu + c);
+#pragma unroll
+            for (int c = 0; c < KH; c += 4) tmem_ld4(lane_addr(t.s0, row, ckap + c), rkap + c);
+#pragma unroll
+            for (int c = 0; c < KM; c += 4) tmem_ld4(lane_addr(t.s0, row, clam + c), rlam + c);
+            tmem_ld4(lane_addr(t.s0, row, cc), rc);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < KH * D; ++i) rmu[i] += __ldg(a.f.b3 + cmu + i);
+#pragma unroll
+            for (int i = 0; i < KH; ++i) rkap[i] += __ldg(a.f.b3 + ckap + i);
+#pragma unroll
+            for (int i = 0; i < KM; ++i) rlam[i] += __ldg(a.f.b3 + clam + i);
+            rc[0] += __ldg(a.f.b3 + cc);
+            pg = g.part(a, rec, rmu, rkap, rlam, rc[0], half);
+        }
+        // the halves exchange their shares of the density through the gradient
+        // tile: each finds the other's in columns that it writes itself below
+        *reinterpret_cast<float *>(t.Gl + cm_offset(row, (1 - half) * KH * D, GC)) = pg;
+        named_sync(t.bar, 256);
+        const float other = *reinterpret_cast<const float *>(t.Gl + cm_offset(row, cmu, GC));
+        pg = half == 0 ? pg + other : other + pg;
+        float dmu[KH * D], dkap[KH], dlam[KH], dc[4] = {0.f, 0.f, 0.f, 0.f};
+        const float rl = g.finish(a, pg, inv_n, half, dmu, dkap, dlam, dc[0]);
+        if (valid) loss_local += rl;
+        if (a.loss_only) {
+            named_sync(t.bar, 256);   // the exchanged values have been read
+            continue;                 // uniform over the tile: no backward pass
+        }
+        // (rows without a record have zero targets, so zero gradients)
+#pragma unroll
+        for (int c = 0; c < KH * D; c += 4) st_row4_split(t.G, t.Gl, row, cmu + c, GC, dmu + c);
+#pragma unroll
+        for (int c = 0; c < KH; c += 4) {
+            st_row4_split(t.G, t.Gl, row, ckap + c, GC, dkap + c);
+            st_row4_split(t.G, t.Gl, row, clam + half * KH + c, GC, dlam + c);
+        }
+        if (half == 0) {
+            st_row4_split(t.G, t.Gl, row, cc, GC, dc);
+            const float z4[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int c = cc + 4; c < OUT; c += 4) st_row4_split(t.G, t.Gl, row, c, GC, z4);
+        } else {
             float z8[8] = {0, 0, 0, 0, 0, 0, 0, 0};
             for (int c = OUT; c < Z2; c += 8) {
                 st_row8_bf16(t.G, row, c, GC, z8);
@@ -317,22 +419,19 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
         }, a.err);
         if (!ok) break;
         // bias gradient: column sums of the dY tiles (hi + lo, what the MMAs see)
-        if (row < OUT) {
+        if (half == 1 && row < OUT) {
             float s = 0.f;
             for (int r = 0; r < 128; ++r)
                 s += __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(t.G + cm_offset(r, row, GC))) +
                      __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(t.Gl + cm_offset(r, row, GC)));
             db3 += s;
         }
-        ld_cols(t.s0, row, kHid, h);
-        {
-            float h2[kHid];
-            for (int c = 0; c < kHid; c += 8) ld_row8_bf16(t.H2, row, c, kHid, h2 + c);
-            for (int c = 0; c < kHid; c += 8) {
-                float v8[8];
-                for (int i = 0; i < 8; ++i) v8[i] = h2[c + i] > 0.f ? h[c + i] : 0.f;
-                st_row8_split(t.G, t.Gl, row, Z2 + c, GC, v8);
-            }
+        ld_cols(t.s0 + hc, row, HC, h);
+        for (int c = 0; c < HC; c += 8) {
+            float v8[8];
+            ld_row8_bf16(t.H2, row, hc + c, kHid, v8);
+            for (int i = 0; i < 8; ++i) v8[i] = v8[i] > 0.f ? h[c + i] : 0.f;
+            st_row8_split(t.G, t.Gl, row, Z2 + hc + c, GC, v8);
         }
         // dW3 (+)= [dY|..]^T H2 over G's first 128 columns (rows 0..OUT-1 used);
         // dH1 = dZ2 W2
@@ -343,15 +442,12 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
             umma_gemm(t.s0, t.Gl + cm_offset(0, Z2, GC), 0, GC, t.w + kW1Bytes, 1, kHid, kHid, kHid, true);
         }, a.err);
         if (!ok) break;
-        ld_cols(t.s0, row, kHid, h);
-        {
-            float h1[kHid];
-            for (int c = 0; c < kHid; c += 8) ld_row8_bf16(t.H1, row, c, kHid, h1 + c);
-            for (int c = 0; c < kHid; c += 8) {
-                float v8[8];
-                for (int i = 0; i < 8; ++i) v8[i] = h1[c + i] > 0.f ? h[c + i] : 0.f;
-                st_row8_split(t.G, t.Gl, row, c, GC, v8);
-            }
+        ld_cols(t.s0 + hc, row, HC, h);
+        for (int c = 0; c < HC; c += 8) {
+            float v8[8];
+            ld_row8_bf16(t.H1, row, hc + c, kHid, v8);
+            for (int i = 0; i < 8; ++i) v8[i] = v8[i] > 0.f ? h[c + i] : 0.f;
+            st_row8_split(t.G, t.Gl, row, hc + c, GC, v8);
         }
         // dW2 (+)= G[:, Z2-64 .. Z2+64)^T H1 (rows 64..127 = dZ2^T H1), dW1 (+)=
         // G[:, 0..128)^T X (rows 0..63 = dZ1^T X), dX = dZ1 W1
@@ -366,12 +462,15 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
         if (!ok) break;
         have_acc = true;
         {
-            float dx[kFeat];
-            ld_cols(t.s0, row, kFeat, dx);   // warp-uniform TMEM load
+            // this thread's half of the levels
+            constexpr int HL = kMaxLevels / 2;
+            float dx[kFeat / 2];
+            ld_cols(t.s0 + half * (kFeat / 2), row, kFeat / 2, dx);   // warp-uniform TMEM load
             if (valid) {
                 float u[D];
                 unit_coords<D>(a.f, rec, u);
-                for (int l = 0; l < a.f.L; ++l) {
+                for (int j = 0; j < HL; ++j) {
+                    const int l = half * HL + j;
                     uint32_t idx[1 << D];
                     float w[1 << D];
                     level_corners<D>(a.f, l, u, idx, w);
@@ -380,8 +479,8 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
                     // (half of them, see encode_row_pairs) take one 16-byte add
                     for (int m = 0; m < (1 << D); m += 2) {
                         const size_t i0 = lo + idx[m], i1 = lo + idx[m + 1];
-                        const float2 v0 = make_float2(w[m] * dx[2 * l], w[m] * dx[2 * l + 1]);
-                        const float2 v1 = make_float2(w[m + 1] * dx[2 * l], w[m + 1] * dx[2 * l + 1]);
+                        const float2 v0 = make_float2(w[m] * dx[2 * j], w[m] * dx[2 * j + 1]);
+                        const float2 v1 = make_float2(w[m + 1] * dx[2 * j], w[m + 1] * dx[2 * j + 1]);
                         if ((i0 ^ i1) == 1) {
                             const bool odd = i0 & 1;
                             atomicAdd(reinterpret_cast<float4 *>(a.g_grid) + (i0 >> 1),
@@ -398,16 +497,17 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
     // flush TMEM accumulators (each warp reads its own 32 lanes)
     if (have_acc && ok) {
         // TMEM loads are warp-collective: every lane loads, then stores conditionally
-        float v[kHid];
-        ld_cols(t.acc3, row, kHid, v);
+        const int hc = half * HC;
+        float v[HC];
+        ld_cols(t.acc3 + hc, row, HC, v);
         // internal output row -> exchange row (padding and disabled lobes: none)
         const int er = row < OUT ? out_row_to_exchange(row, a.f.dim, a.f.K, KM) : -1;
-        if (er >= 0) for (int i = 0; i < kHid; ++i) atomicAdd(a.g_W3 + (size_t)er * kHid + i, v[i]);
-        ld_cols(t.acc2, row, kHid, v);
-        if (row >= 64) for (int i = 0; i < kHid; ++i) atomicAdd(a.g_W2 + (size_t)(row - 64) * kHid + i, v[i]);
-        ld_cols(t.acc1, row, kFeat, v);
-        if (row < 64) for (int i = 0; i < kFeat; ++i) atomicAdd(a.g_W1 + (size_t)row * kFeat + i, v[i]);
-        if (er >= 0) atomicAdd(a.g_b3 + er, db3);
+        if (er >= 0) for (int i = 0; i < HC; ++i) atomicAdd(a.g_W3 + (size_t)er * kHid + hc + i, v[i]);
+        ld_cols(t.acc2 + hc, row, HC, v);
+        if (row >= 64) for (int i = 0; i < HC; ++i) atomicAdd(a.g_W2 + (size_t)(row - 64) * kHid + hc + i, v[i]);
+        ld_cols(t.acc1 + half * (kFeat / 2), row, kFeat / 2, v);
+        if (row < 64) for (int i = 0; i < kFeat / 2; ++i) atomicAdd(a.g_W1 + (size_t)row * kFeat + half * (kFeat / 2) + i, v[i]);
+        if (half == 1 && er >= 0) atomicAdd(a.g_b3 + er, db3);
     }
     // loss: warp reduction then one atomic per warp
     for (int o = 16; o; o >>= 1) loss_local += __shfl_xor_sync(0xffffffffu, loss_local, o);
