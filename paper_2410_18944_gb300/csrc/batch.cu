@@ -51,7 +51,7 @@ struct BatchGuidedArgs {
 
 template <int D>
 __global__ void __launch_bounds__(kBatchPlainBlock) batch_plain_kernel(const __grid_constant__ BatchArgs b) {
-    plain_loop<D, true>(coop_shared<D, kBatchPlainBlock / 32>(), BatchSrc<D>{b}, b.stat);
+    plain_loop<D, kModeMulti>(coop_shared<D, kBatchPlainBlock / 32>(), BatchSrc<D>{b}, b.stat);
 }
 
 template <int D, int W>
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128) batch_classify_kernel(const DevJob *jobs,
     const bool act = i < n;
     const DevJob &J = jobs[find_job(jobs, njobs, act ? i : n - 1)];
     double val;
-    const uint8_t st = classify_point<D, true>(coop_shared<D, 4>(), J.sc, J.eps64, J.points + (i - J.point_off) * D, act, err, val);
+    const uint8_t st = classify_point<D, kModeMulti>(coop_shared<D, 4>(), J.sc, J.eps64, J.points + (i - J.point_off) * D, act, err, val);
     if (!act) return;
     status[i] = st;
     shell[i] = val;

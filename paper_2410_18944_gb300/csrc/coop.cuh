@@ -16,12 +16,12 @@
 // a leaf is one or a few round trips, and so is a node.
 //
 // Closest points: groups of eight lanes over eight-wide nodes of oriented
-// caps (geom.cuh), nearest node first.  The caps carry a margin above the
+// caps and boxes (geom.cuh), nearest node first.  The bounds carry a margin above the
 // rounding of the distances, so the search returns the minimum over all
 // primitives (ties to the smaller id) in whatever order it visits them.  The
 // query is defined by the box tree, though (coop_closest).
-// Silhouettes and rays: groups of four lanes over four-wide nodes of boxes,
-// depth first, children nearest first.  An edge's or a hit's FP32 value can
+// Silhouettes, rays, Neumann samples: groups of four or eight lanes over
+// four-wide nodes of boxes, depth first, children nearest first.  An edge's or a hit's FP32 value can
 // lie below its box's by rounding (a ray hit by its edge slack, ray_prim), so
 // the result can depend on which box was opened first, and the summed weight of
 // the Neumann sample on the order of its terms: the order of visits is part of
@@ -54,6 +54,20 @@ __device__ __forceinline__ CoopWarp *coop_shared() {
 __host__ __device__ constexpr int coop_bytes(int D, int warps) { return D == 3 ? warps * (int)sizeof(CoopWarp) : 0; }
 
 enum : int { kCoopPoint = 0, kCoopPointBox = 1, kCoopSil = 2, kCoopExit = 3, kCoopAny = 4, kCoopCount = 5, kCoopPick = 6 };
+
+// What the lanes of a calling warp hold: walks of one scene, walks whose scenes
+// may differ (a pointer per lane), or few walks of one scene (the wavefront)
+enum : int { kModeSolo = 0, kModeMulti = 1, kModeFew = 2 };
+
+// Lanes per group.  Closest points: one per child and leaf primitive.
+// Silhouettes and rays: one per child, four rounds for a leaf of 16; with few
+// walks per warp the longer chain costs more than the shared visits save
+// (silhouettes, eight lanes: guided icosphere 63.2 -> 59.2 ms, plain icosphere
+// 80 -> 82).  The Neumann sample's leaves are long (a philox draw and a log
+// per primitive): flux slab 19.6 -> 18.8 ms with eight.
+__host__ __device__ constexpr int group_lanes(int kind, int mode) {
+    return kind == kCoopPoint || kind == kCoopPick || (kind == kCoopSil && mode == kModeFew) ? 8 : 4;
+}
 
 // monotonic map of a float (not NaN) to an int
 __device__ __forceinline__ int order_key(float f) {
@@ -93,8 +107,7 @@ __device__ __forceinline__ const DevBVH &coop_bvh(const DevScene &sc, bool diric
 //   kCoopCount  crossings along v (returned), aux != 0: of the Dirichlet BVH
 //   kCoopPick   neumann_pick: best_io: in r^2, out W; v: the bits of point, walk
 //               and step, aux and key1: the key
-// Returns the leaf slot (-1: none within the bound).  kMulti: the lanes'
-// scenes may differ.
+// Returns the leaf slot (-1: none within the bound).
 // Out of line: the walk's state is saved once around the call instead of
 // competing with the traversal for registers (the kernels run at 64 to 96 per
 // thread).
@@ -103,7 +116,7 @@ struct CoopResult {
     float best;
     uint32_t nodes, prims;   // visits of the queries this lane's group answered (its first lane counts)
 };
-template <int kKind, bool kMulti>
+template <int kKind, int kMode>
 __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *scene_p, bool want, float x0, float x1,
                                               float x2, float v0, float v1, float v2, float best_io, int aux, uint32_t key1,
                                               int *err) {
@@ -113,7 +126,9 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
     CoopResult res{kKind == kCoopCount ? 0 : -1, best_io, 0u, 0u};
     constexpr unsigned kFull = 0xffffffffu;
     constexpr bool kRay = kKind >= kCoopExit && kKind <= kCoopCount;
-    constexpr int G = kKind == kCoopPoint ? 8 : 4, NG = 32 / G;   // lanes per group, groups
+    constexpr bool kMulti = kMode == kModeMulti;
+    constexpr int G = group_lanes(kKind, kMode), NG = 32 / G;   // lanes per group, groups
+    constexpr int NW = kKind == kCoopPoint ? 8 : 4;   // children per node
     const int lane = threadIdx.x & 31, sub = lane & (G - 1), g = lane / G, base = g * G;
     uint2 *stack = sh.stack[g];
     want = want && coop_bvh<kKind>(scene, aux != 0).nprims > 0;
@@ -252,15 +267,19 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
             float key = 0.f;
             int cref = kEmptyRef;
             bool ok = false;
-            if (at) {
+            if (at && (G == NW || sub < NW)) {
                 if constexpr (kKind == kCoopPoint) {
                     const float4 *p = sc.dir_caps + (size_t)cap_f4(3) * ref;
-                    cref = reinterpret_cast<const int *>(p + 2 * G)[sub];
-                    key = cap_d2_3(ldn(p + sub), ldn(p + G + sub), gx);
+                    const float4 bl = ldn(p + 2 * G + sub), bh = ldn(p + 3 * G + sub);   // lo.xyz, hi.x | hi.yz
+                    const float ex = fmaxf(fmaxf(bl.x - gx[0], gx[0] - bl.w), 0.f);
+                    const float ey = fmaxf(fmaxf(bl.y - gx[1], gx[1] - bh.x), 0.f);
+                    const float ez = fmaxf(fmaxf(bl.z - gx[2], gx[2] - bh.y), 0.f);
+                    key = fmaxf(cap_d2_3(ldn(p + sub), ldn(p + G + sub), gx), ex * ex + ey * ey + ez * ez);
+                    cref = __float_as_int(bh.z);
                     ok = cref != kEmptyRef && key <= best;
                 } else {
                     const float4 *p = bv.nodes + (size_t)node_f4<3>() * ref + sub;
-                    const float4 a = ldn(p), b = ldn(p + G);   // lo.xyz, hi.x | hi.yz, child, -
+                    const float4 a = ldn(p), b = ldn(p + NW);   // lo.xyz, hi.x | hi.yz, child, -
                     cref = __float_as_int(b.z);
                     const float lo[3] = {a.x, a.y, a.z}, hi[3] = {a.w, b.x, b.y};
                     if constexpr (kRay) {
@@ -288,7 +307,7 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                         if constexpr (kKind == kCoopSil) {
                             const float4 *fp = sc.sil_facing + (size_t)facing_f4(3) * ref;
                             const float4 f = ldn(fp + sub);   // axis, d0
-                            const float2 h = reinterpret_cast<const float2 *>(fp + G)[sub];   // d1, s^2
+                            const float2 h = reinterpret_cast<const float2 *>(fp + NW)[sub];   // d1, s^2
                             const float q = -(f.x * u[0] + f.y * u[1] + f.z * u[2]);
                             ok = ok && !facing_prunes(q, f.w, h.x, h.y, far2, sc.tau);
                         }
@@ -313,8 +332,8 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                     const int ro = __shfl_sync(kFull, cref, base + other);
                     if (sub < other ? ko < kk : (sub > other && kk < ko)) { kk = ko; cref = ro; }
                 };
-                swap(sub ^ 1);
-                swap(sub ^ 2);
+                swap(G == NW || sub < NW ? sub ^ 1 : sub);
+                swap(G == NW || sub < NW ? sub ^ 2 : sub);
                 swap(sub == 1 || sub == 2 ? 3 - sub : sub);
                 key = kk;
                 nref = __shfl_sync(kFull, cref, base);
@@ -409,10 +428,10 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
 }
 
 // the call, with the visits added to the lane's counters
-template <int kKind, bool kMulti>
+template <int kKind, int kMode>
 __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool want, const float *x, const float *v,
                                         float &best, int aux, int *err, Visits *vis, uint32_t key1 = 0) {
-    const CoopResult r = coop_query<kKind, kMulti>((uint32_t)__cvta_generic_to_shared(&sh), &sc, want, x[0], x[1], x[2],
+    const CoopResult r = coop_query<kKind, kMode>((uint32_t)__cvta_generic_to_shared(&sh), &sc, want, x[0], x[1], x[2],
                                                    v[0], v[1], v[2], best, aux, key1, err);
     best = r.best;
     if (vis) {
@@ -432,11 +451,11 @@ __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool w
 // caps is therefore the boxes' answer whenever the primitive's distance is not
 // below that of its own bounding box, which its leaf's box contains; the rest
 // (about one in 10^5) are searched again in the boxes.
-template <bool kMulti>
+template <int kMode>
 __device__ __forceinline__ int coop_closest(CoopWarp &sh, const DevScene &sc, bool want, const float *x, float &d2,
                                             int *err, Visits *vis) {
     d2 = __int_as_float(0x7f800000);
-    int slot = coop_run<kCoopPoint, kMulti>(sh, sc, want, x, x, d2, -1, err, vis);
+    int slot = coop_run<kCoopPoint, kMode>(sh, sc, want, x, x, d2, -1, err, vis);
     bool again = false;
     if (slot >= 0) {
         float a[3], b[3], c[3], dd[3];
@@ -450,7 +469,7 @@ __device__ __forceinline__ int coop_closest(CoopWarp &sh, const DevScene &sc, bo
     }
     if (__any_sync(0xffffffffu, again)) {
         float e2 = __int_as_float(0x7f800000);
-        const int e = coop_run<kCoopPointBox, kMulti>(sh, sc, again, x, x, e2, -1, err, vis);
+        const int e = coop_run<kCoopPointBox, kMode>(sh, sc, again, x, x, e2, -1, err, vis);
         if (again) { slot = e; d2 = e2; }
     }
     return slot;

@@ -474,7 +474,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
                 if (D == 2 && !active) return;
                 nsteps += active;
                 bool trunc = false;
-                if (step_geometry<D, kMulti>(sh, w, src.env(w), active, r, S, gv, trunc, &vis)) {
+                if (step_geometry<D, kMulti ? kModeMulti : kModeSolo>(sh, w, src.env(w), active, r, S, gv, trunc, &vis)) {
                     src.finish(w);
                     ended = true;
                     ntrunc += trunc;
@@ -585,7 +585,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
                 }
             }
             if (o.record) suffix(live && zero_density, S);
-            step_move<D, kMulti>(sh, w, src.env(w), live && !zero_density, nu, r, &vis);
+            step_move<D, kMulti ? kModeMulti : kModeSolo>(sh, w, src.env(w), live && !zero_density, nu, r, &vis);
         }
         if (failed) atomicOr(o.err, 2);
         __syncwarp();

@@ -265,7 +265,7 @@ struct WorkCursor {
 // after each query (2D: a lane without a walk is predicated off; 3D: it takes
 // part in the queries of the others, coop.cuh).
 // ---------------------------------------------------------------------------
-template <int D, bool kMulti, class Src>
+template <int D, int kMode, class Src>
 __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigned long long *stat) {
     Walk<D> w;
     Visits vis;
@@ -293,7 +293,7 @@ __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigne
         const StepEnv env = src.env(w);
         float r = 0.f, S, gv;
         bool trunc = false;
-        bool ended = step_geometry<D, kMulti>(sh, w, env, active, r, S, gv, trunc, &vis);
+        bool ended = step_geometry<D, kMode>(sh, w, env, active, r, S, gv, trunc, &vis);
         float nu[D] = {};
         if (active && !ended) {
             U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_DIR, env.key0, env.key1);
@@ -309,7 +309,7 @@ __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigne
             ntrunc += trunc;
             active = false;
         }
-        step_move<D, kMulti>(sh, w, env, active, nu, r, &vis);
+        step_move<D, kMode>(sh, w, env, active, nu, r, &vis);
     }
     flush_stats(stat, nsteps, ntrunc, nwalks, vis);
 }

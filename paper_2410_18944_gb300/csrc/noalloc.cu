@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128) static_classify_kernel(WalkArgs a, double
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool act = i < a.npoints;
     double val;
-    const uint8_t st = classify_point<D, false>(coop_shared<D, 4>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
+    const uint8_t st = classify_point<D, kModeSolo>(coop_shared<D, 4>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
     if (!act) return;
     const_cast<uint8_t *>(a.status)[i] = st;
     shell_value[i] = val;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(128) static_classify_kernel(WalkArgs a, double
 // the plain persistent walk loop, on the static scratch
 template <int D>
 __global__ void __launch_bounds__(128) static_walk_kernel(const __grid_constant__ WalkArgs a) {
-    plain_loop<D, false>(coop_shared<D, 4>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
+    plain_loop<D, kModeSolo>(coop_shared<D, 4>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
 }
 
 __global__ void static_finalize_kernel(const uint8_t *status, const double *shell_value, const double *sum,

@@ -446,8 +446,12 @@ struct Builder {
                 o[k] = make_float4(c.c[0], c.c[1], c.c[2], c.h);
                 o[8 + k] = make_float4(c.a[0], c.a[1], c.a[2], c.r);
             }
-            for (int k = 0; k < 8; k += 4)
-                o[16 + k / 4] = make_float4(bits(ch[k].ref), bits(ch[k + 1].ref), bits(ch[k + 2].ref), bits(ch[k + 3].ref));
+            const float grow = std::nextafterf((float)margin, INFINITY);
+            for (int k = 0; k < 8; ++k) {
+                const Box &bx = ch[k].box;
+                o[16 + k] = make_float4(bx.lo[0] - grow, bx.lo[1] - grow, bx.lo[2] - grow, bx.hi[0] + grow);
+                o[24 + k] = make_float4(bx.hi[1] + grow, bx.hi[2] + grow, bits(ch[k].ref), 0.f);
+            }
         });
         return out;
     }

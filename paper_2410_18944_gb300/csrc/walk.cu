@@ -83,7 +83,7 @@ constexpr int kPlainBlock = 128;
 
 template <int D>
 __global__ void __launch_bounds__(kPlainBlock, D == 3 ? 8 : 0) plain_walk_kernel(const __grid_constant__ WalkArgs a) {
-    plain_loop<D, false>(coop_shared<D, kPlainBlock / 32>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
+    plain_loop<D, kModeSolo>(coop_shared<D, kPlainBlock / 32>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
 }
 
 // status of every query point: 2 outside (odd/even crossing count of a ray
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kPlainBlock) classify_kernel(WalkArgs a, doubl
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool act = i < a.npoints;
     double val;
-    const uint8_t st = classify_point<D, false>(coop_shared<D, kPlainBlock / 32>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
+    const uint8_t st = classify_point<D, kModeSolo>(coop_shared<D, kPlainBlock / 32>(), a.sc, a.eps64, a.points + i * D, act, a.err, val);
     if (!act) return;
     const_cast<uint8_t *>(a.status)[i] = st;
     shell_value[i] = val;
@@ -116,7 +116,7 @@ __global__ void q_closest_kernel(DevScene sc, const double *p, int64_t n, int32_
     if (act)
         for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
     float b;
-    const int s = query_dirichlet<D, false>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
+    const int s = query_dirichlet<D, kModeSolo>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
     if (!act) return;
     oid[i] = s >= 0 ? sc.dir.ids[s] : -1;
     od[i] = sqrtf(b);
@@ -132,7 +132,7 @@ __global__ void q_sil_kernel(DevScene sc, const int64_t *keys, const double *p, 
     if (act)
         for (int k = 0; k < D; ++k) x[k] = (float)p[i * D + k];
     float b = __int_as_float(0x7f800000);
-    const int s = query_silhouette<D, false>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
+    const int s = query_silhouette<D, kModeSolo>(coop_shared<D, kPlainBlock / 32>(), sc, act, x, b, err, nullptr);
     if (!act) return;
     oid[i] = s >= 0 ? keys[s] : -1;
     od[i] = s >= 0 ? sqrtf(b) : b;
@@ -158,13 +158,13 @@ __global__ void q_ray_kernel(DevScene sc, const double *o, const double *v, cons
         tm = (float)tmax[i];
     }
     if (kExit) {
-        s = query_exit<D, false>(sh, sc, act, x, d, tm, skip, t, err, nullptr);
+        s = query_exit<D, kModeSolo>(sh, sc, act, x, d, tm, skip, t, err, nullptr);
     } else {
         if constexpr (D == 2) {
             s = ray_neumann<false>(sc.neu, x, d, tm, skip, t, err);
         } else {
             t = tm;
-            s = coop_run<kCoopAny, false>(*sh, sc, act, x, d, t, skip, err, nullptr);
+            s = coop_run<kCoopAny, kModeSolo>(*sh, sc, act, x, d, t, skip, err, nullptr);
         }
         if (s >= 0) {
             double t64;

@@ -143,7 +143,7 @@ __device__ __forceinline__ void finish_walk(const WalkArgs &a, uint32_t pid, flo
 //                                      (1 / |z - x| - 1 / r) / 4 pi  (3D),
 // h the flux along the normal into the domain, alpha = 1/2 on a Neumann point.
 // Lanes with `act` (3D: the whole warp calls).
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ float neumann_term(CoopWarp *sh, const Walk<D> &w, const DevScene &sc, bool act, float r,
                                               uint32_t k0, uint32_t k1, int *err, Visits *vis) {
     float W;
@@ -153,7 +153,7 @@ __device__ __forceinline__ float neumann_term(CoopWarp *sh, const Walk<D> &w, co
     } else {
         const float ctr[3] = {__uint_as_float(w.pid), __uint_as_float(w.wid), __int_as_float(w.k)};
         W = r * r;
-        js = coop_run<kCoopPick, kMulti>(*sh, sc, act, w.x, ctr, W, (int)k0, err, vis, k1);
+        js = coop_run<kCoopPick, kMode>(*sh, sc, act, w.x, ctr, W, (int)k0, err, vis, k1);
     }
     if (js < 0) return 0.f;
     U4 u = philox(w.pid, w.wid, (uint32_t)w.k, P_NEU, k0, k1);
@@ -184,28 +184,27 @@ __device__ __forceinline__ float neumann_term(CoopWarp *sh, const Walk<D> &w, co
 }
 
 // The queries of a step: per lane in 2D (called by the lanes that want one),
-// by groups of lanes in 3D (called by the whole warp).  kMulti: the lanes'
-// scenes may differ.
-template <int D, bool kMulti>
+// by groups of lanes in 3D (called by the whole warp).  kMode: coop.cuh.
+template <int D, int kMode>
 __device__ __forceinline__ int query_dirichlet(CoopWarp *sh, const DevScene &sc, bool want, const float *x, float &d2,
                                                int *err, Visits *vis) {
     if constexpr (D == 2) {
         return closest_dirichlet(sc.dir, sc.dir_caps, x, d2, err, vis);
     } else {
-        return coop_closest<kMulti>(*sh, sc, want, x, d2, err, vis);
+        return coop_closest<kMode>(*sh, sc, want, x, d2, err, vis);
     }
 }
 
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ int query_silhouette(CoopWarp *sh, const DevScene &sc, bool want, const float *x, float &d2,
                                                  int *err, Visits *vis) {
     if constexpr (D == 2) return closest_silhouette(sc.sil, x, sc.tau, d2, err, sc.sil_facing, vis);
-    else return coop_run<kCoopSil, kMulti>(*sh, sc, want, x, x, d2, -1, err, vis);
+    else return coop_run<kCoopSil, kMode>(*sh, sc, want, x, x, d2, -1, err, vis);
 }
 
 // first exit through the Neumann boundary within tmax, re-tested in FP64 when
 // the FP32 hit lies within its rounding band below tmax
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ int query_exit(CoopWarp *sh, const DevScene &sc, bool want, const float *x, const float *v,
                                           float tmax, int skip, float &th, int *err, Visits *vis) {
     const float tneg = kRoundBand * sc.scale;
@@ -214,7 +213,7 @@ __device__ __forceinline__ int query_exit(CoopWarp *sh, const DevScene &sc, bool
         hit = ray_neumann<true>(sc.neu, x, v, tmax, skip, th, err, vis, tneg);
     } else {
         th = tmax;
-        hit = coop_run<kCoopExit, kMulti>(*sh, sc, want, x, v, th, skip, err, vis);
+        hit = coop_run<kCoopExit, kMode>(*sh, sc, want, x, v, th, skip, err, vis);
     }
     if (hit >= 0 && tmax - th <= kRoundBand * (sc.scale + tmax)) {
         double t64;
@@ -228,13 +227,13 @@ __device__ __forceinline__ int query_exit(CoopWarp *sh, const DevScene &sc, bool
 // roulette draw).  On return false: r (star radius) and S (this step's source
 // and Neumann terms, times the step's roulette scale, as the suffix pass of a
 // recorded walk takes them).
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const StepEnv &a, bool act, float &r, float &S,
                                               float &term_value, bool &truncated, Visits *vis) {
     if (D == 2 && !act) return false;
     const DevScene &sc = a.sc;
     float bd2;
-    const int slot = query_dirichlet<D, kMulti>(sh, sc, act, w.x, bd2, a.err, vis);
+    const int slot = query_dirichlet<D, kMode>(sh, sc, act, w.x, bd2, a.err, vis);
     const float RD = sqrtf(bd2);
     bool ended = false;
     if (act) {
@@ -268,7 +267,7 @@ __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const St
     if (D == 2 && ended) return true;
     const bool go = act && !ended;
     float bs = RD * RD;
-    query_silhouette<D, kMulti>(sh, sc, go, w.x, bs, a.err, vis);
+    query_silhouette<D, kMode>(sh, sc, go, w.x, bs, a.err, vis);
     if (go) {
         float R = fminf(sqrtf(bs), RD);
         r = fmaxf(R, a.eps);
@@ -284,7 +283,7 @@ __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const St
             rho = D == 2 ? r * sqrtf(u01(u.z) * u01(u.w)) : r * beta22_inv(u01(u.z));
         }
         float th;
-        const int hs = query_exit<D, kMulti>(sh, sc, source, w.x, vs, rho, w.prim, th, a.err, vis);
+        const int hs = query_exit<D, kMode>(sh, sc, source, w.x, vs, rho, w.prim, th, a.err, vis);
         if (source) {
             if (hs < 0) {
                 float y[3];
@@ -297,7 +296,7 @@ __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const St
     }
     const bool flux = go && sc.has_flux;
     if (D == 2 ? flux : __any_sync(0xffffffffu, flux)) {
-        const float N = neumann_term<D, kMulti>(sh, w, sc, flux, r, a.key0, a.key1, a.err, vis);
+        const float N = neumann_term<D, kMode>(sh, w, sc, flux, r, a.key0, a.key1, a.err, vis);
         if (flux) {
             S -= N;
             w.acc += w.T * S;
@@ -309,13 +308,13 @@ __device__ __forceinline__ bool step_geometry(CoopWarp *sh, Walk<D> &w, const St
 
 // Step 5 of the lanes with `act` (3D: the whole warp calls): ray cast within
 // r and move.
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ void step_move(CoopWarp *sh, Walk<D> &w, const StepEnv &a, bool act, const float *nu, float r,
                                           Visits *vis) {
     if (D == 2 && !act) return;
     const DevScene &sc = a.sc;
     float th;
-    const int hit = query_exit<D, kMulti>(sh, sc, act, w.x, nu, r, w.prim, th, a.err, vis);
+    const int hit = query_exit<D, kMode>(sh, sc, act, w.x, nu, r, w.prim, th, a.err, vis);
     if (!act) return;
     if (hit >= 0) {
         // an exit hit arrives from the inside, the side the walk is on, so
@@ -341,15 +340,15 @@ __device__ __forceinline__ void step_move(CoopWarp *sh, Walk<D> &w, const StepEn
 }
 
 // crossings of the ray x + t v (t > 0) with the whole boundary
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ int count_crossings(CoopWarp *sh, const DevScene &sc, bool want, const float *x,
                                                const float *v, int *err) {
     if constexpr (D == 2) {
         return ray_count(sc.dir, x, v, err) + ray_count(sc.neu, x, v, err);
     } else {
         float far = 3.0e38f;
-        const int n = coop_run<kCoopCount, kMulti>(*sh, sc, want, x, v, far, 1, err, nullptr);
-        return n + coop_run<kCoopCount, kMulti>(*sh, sc, want, x, v, far, 0, err, nullptr);
+        const int n = coop_run<kCoopCount, kMode>(*sh, sc, want, x, v, far, 1, err, nullptr);
+        return n + coop_run<kCoopCount, kMode>(*sh, sc, want, x, v, far, 0, err, nullptr);
     }
 }
 
@@ -357,7 +356,7 @@ __device__ __forceinline__ int count_crossings(CoopWarp *sh, const DevScene &sc,
 // ray against all primitives), 1 inside the epsilon-shell (val = g at the
 // closest Dirichlet point, FP64 distance test), 0 to be walked.
 // (3D: the whole warp calls, `act`: the lanes with a point)
-template <int D, bool kMulti>
+template <int D, int kMode>
 __device__ __forceinline__ uint8_t classify_point(CoopWarp *sh, const DevScene &sc, double eps64, const double *p,
                                                   bool act, int *err, double &val) {
     float x[D] = {};
@@ -368,7 +367,7 @@ __device__ __forceinline__ uint8_t classify_point(CoopWarp *sh, const DevScene &
     for (int k = 0; k < D; ++k) { v[k] = dir[k]; nn += v[k] * v[k]; }
     for (int k = 0; k < D; ++k) v[k] *= rsqrtf(nn);
     if (D == 2 && !act) return 0;
-    const int c = count_crossings<D, kMulti>(sh, sc, act, x, v, err);
+    const int c = count_crossings<D, kMode>(sh, sc, act, x, v, err);
     val = 0.0;
     const bool inside = act && (c & 1) != 0;
     if (D == 2 && !inside) {
@@ -376,7 +375,7 @@ __device__ __forceinline__ uint8_t classify_point(CoopWarp *sh, const DevScene &
         return 2;
     }
     float bd2;
-    const int slot = query_dirichlet<D, kMulti>(sh, sc, inside, x, bd2, err, nullptr);
+    const int slot = query_dirichlet<D, kMode>(sh, sc, inside, x, bd2, err, nullptr);
     if (!inside) {
         val = __longlong_as_double(0x7ff8000000000000LL);
         return 2;

@@ -94,7 +94,7 @@ __device__ __forceinline__ void store_walk(const WfSlots &S, int s, const Walk<D
     S.ids[s] = make_int4((int)w.pid, (int)w.wid, w.k, w.prim);
 }
 
-template <int D, bool kMulti, class Src>
+template <int D, int kMode, class Src>
 __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const WsOpts &o, const WfSlots &S,
                                              int parity, bool first) {
     // one thread per entry of the previous iteration's decode list (or per
@@ -184,7 +184,7 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
             w.T *= wgt;
         }
     }
-    if (D == 2 ? active : !first) step_move<D, kMulti>(sh, w, src.env(w), active, nu, r, &vis);
+    if (D == 2 ? active : !first) step_move<D, kMode>(sh, w, src.env(w), active, nu, r, &vis);
     // ---- the next step's geometry; an ended walk hands its slot to the next item ----
     bool settled = !valid;   // this lane's geometry is done, or there is no work for it
     for (;;) {
@@ -199,7 +199,7 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
         nsteps += run;
         float gv;
         bool trunc = false;
-        if (step_geometry<D, kMulti>(sh, w, src.env(w), run, r, Sx, gv, trunc, &vis)) {
+        if (step_geometry<D, kMode>(sh, w, src.env(w), run, r, Sx, gv, trunc, &vis)) {
             src.finish(w);
             // the suffix pass of a recorded walk waits for the end of the
             // launch (a recording launch gives every slot one walk, so its
@@ -232,7 +232,7 @@ __global__ void wf_suffix_kernel(RecDest rd, const float *scratch, int scratch_s
 
 template <int D>
 __global__ void __launch_bounds__(kWfBlock) wf_step_kernel(const __grid_constant__ WfSoloArgs g) {
-    wf_step_body<D, false>(coop_shared<D, kWfBlock / 32>(), SoloSrc<D>{g.w, &g.f, g.rd, &g.w.sc}, g.o, g.S, g.parity,
+    wf_step_body<D, kModeFew>(coop_shared<D, kWfBlock / 32>(), SoloSrc<D>{g.w, &g.f, g.rd, &g.w.sc}, g.o, g.S, g.parity,
                            g.first != 0);
 }
 
