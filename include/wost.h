@@ -179,7 +179,7 @@ typedef struct {
     int32_t walker_warps;      /* guided launches of the warp-specialised kernel: walker warps
                                   per CTA beside its 4 decode-server warps, 0 (automatic), 16 or
                                   28 (WOST_ERR_INVALID_ARG otherwise).  Automatic: wost_solve takes
-                                  28 when the scene's traversal data (BVH nodes, cones,
+                                  28 when the scene's traversal data (BVH nodes, bounds,
                                   primitives) exceeds 64 MB or, in 3D, when a launch holds at
                                   least two walks per lane of the 28-warp kernel, else 16;
                                   wost_batch_create lets its autotuner choose.  Results do not

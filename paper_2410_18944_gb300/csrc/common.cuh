@@ -128,7 +128,7 @@ struct DevScene {
     int has_flux;         // nonzero Neumann flux h and Neumann primitives
 };
 
-// BVH node, normal-cone and primitive loads: generic, as the arrays may
+// BVH node, bound and primitive loads: generic, as the arrays may
 // have been staged in shared memory by the kernel
 __device__ __forceinline__ float4 ldn(const float4 *p) { return *p; }
 

@@ -13,7 +13,9 @@
 // lane at another node, the warp waiting for its longest query), one L2
 // round trip per primitive of a leaf, and a launch lasted as long as its
 // slowest walk, 0.5-2 ms a step.  With groups all lanes of a visit do work,
-// a leaf is one or a few round trips, and so is a node.
+// a leaf is one or a few round trips, and so is a node.  What bounds it now: L2
+// round trips and instruction fetch (35% of issue slots, 20 active lanes of 32 on
+// the icosphere); figures at plain_walk_kernel.
 //
 // Closest points: groups of eight lanes over eight-wide nodes of oriented
 // caps and boxes (geom.cuh), nearest node first.  The bounds carry a margin above the
@@ -449,8 +451,8 @@ __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool w
 // the distance of its own box (both are rounded; an edge shared by triangles
 // of several leaves), where the order of visits decides.  The answer of the
 // caps is therefore the boxes' answer whenever the primitive's distance is not
-// below that of its own bounding box, which its leaf's box contains; the rest
-// (about one in 10^5) are searched again in the boxes.
+// below that of its own bounding box, which its leaf's box contains; the few
+// others are searched again in the boxes.
 template <int kMode>
 __device__ __forceinline__ int coop_closest(CoopWarp &sh, const DevScene &sc, bool want, const float *x, float &d2,
                                             int *err, Visits *vis) {

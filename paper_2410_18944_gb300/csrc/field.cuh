@@ -180,8 +180,8 @@ __device__ __forceinline__ void encode_row(const DevField &f, const float *x, ui
 // the rate of L1 lookups (one per lane and load, the table serves from L2), so
 // 1.25 loads per pair take the place of two (figures at decode_kernel; the
 // training step's two passes over 2^18 3D records 1473 -> 1338 us per call).  Costs 8 more registers per
-// level in flight, which the walkers of the warp-specialised kernel do not
-// have.  Same features bit for bit: the corners are added in the same order.
+// level in flight; the walkers of the warp-specialised kernel, which wait for
+// few rows at a time, are slower with it (star training batch 39.0 -> 41.2 ms).  Same features bit for bit: the corners are added in the same order.
 // (levels [first, last), multiples of four)
 template <int D>
 __device__ __forceinline__ void encode_row_pairs(const DevField &f, const float *x, uint8_t *xtile, int row, int first = 0,

