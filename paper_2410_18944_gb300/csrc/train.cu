@@ -7,8 +7,8 @@
 // Eq. one_sample_kld for Theta and Eq. one_sample_sp for c.  The mean over
 // records is back-propagated through the MLP and scattered onto the hash grid.
 //
-// One fused persistent kernel, two 128-record tiles per CTA (256 threads;
-// one tile of 128 threads for fields of 9..16 lobes, whose 96 outputs widen
+// One fused persistent kernel, two 128-record tiles per CTA (512 threads,
+// two per record; one tile of 256 threads for fields of 9..16 lobes, whose 96 outputs widen
 // the gradient tile and the TMEM columns beyond two tiles per SM):
 //   forward recomputation (3 tcgen05 MMAs) -> per-thread loss and d raw ->
 //   dH2 = dY W3, dZ2 = dH2 * [H2 > 0] -> dH1 = dZ2 W2 -> dZ1 -> dX = dZ1 W1
@@ -250,7 +250,8 @@ struct RecordGrad {
             for (int i = 0; i < D; ++i) dmu[j * D + i] = 0.f;
         }
         if (!live) return 0.f;
-        const float ptil = c * pg + (1.f - c) * pu;
+        // (the rounding spelled out, as the density's above)
+        const float ptil = __fmaf_rn(1.f - c, pu, __fmul_rn(c, pg));
         const float pgs = fmaxf(pg, 1e-30f);
         const float dpg = -wt / pgs * inv_n;
 #pragma unroll
