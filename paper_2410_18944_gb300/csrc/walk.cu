@@ -83,12 +83,12 @@ constexpr int kPlainBlock = 128;
 
 // Measured on one GB300, one query per lane (before) and now:
 //   3D (queries by lane groups, caps, facing bounds): icosphere of 82k triangles,
-//   376k walks, 231 / 78.5 ms; genus-3 solid of 994k, 131k walks, 316 / 58 ms;
+//   376k walks, 231 / 78.5 ms; genus-3 solid of 994k, 131k walks, 326 / 60 ms;
 //   flux slab, 131k walks, 30.2 / 16.4 ms.  Eight CTAs per SM (64 registers): the
 //   queries are calls, so the walk's state spills around them, not inside; six
 //   CTAs (80 registers) 88 against 82 ms on the icosphere, four 100.
 //   2D (caps, facing bounds, 8-byte stack entries): star of 4096 segments, 1.39 M
-//   walks, 41.5 / 20.3 ms; 64 segments, 52k walks, 490 / 380 us.
+//   walks, 41.5 / 20.3 ms; 64 segments, 52k walks, 490 / 345 us (whole call).
 template <int D>
 __global__ void __launch_bounds__(kPlainBlock, D == 3 ? 8 : 0) plain_walk_kernel(const __grid_constant__ WalkArgs a) {
     plain_loop<D, kModeSolo>(coop_shared<D, kPlainBlock / 32>(), SoloSrc<D>{a, nullptr, RecDest{}, &a.sc}, a.stat);
