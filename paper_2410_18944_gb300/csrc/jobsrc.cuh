@@ -231,13 +231,14 @@ struct BatchSrc {
 // 3D: round the warps, the lanes of a warp that hold walks: a warp has four to
 // eight queries in flight at a time, so more walks than that only amortise the
 // step logic, but a warp that is left with many long walks holds up the end of
-// the launch; half the lanes where there are fewer than two walks per lane.
-// Measured on one GB300, 16 / 32 lanes: genus-3 (27 walks per warp) 66 / 72
-// ms, icosphere (77 per warp) 83 / 79 ms.
+// the launch; half the lanes where there are fewer than two walks per lane,
+// all of them where every step has a Neumann sample too.  Measured on one GB300,
+// 16 / 32 lanes: genus-3 (27 walks per warp) 59 / 64 ms, icosphere (77 per warp)
+// 86 / 78 ms, flux slab (27 per warp) 16.1 / 15.0 ms.
 inline int plain_lanes(const DevScene &s, unsigned long long total, long long warps) {
     const unsigned long long lanes = 32ull * (unsigned long long)warps;
     if (s.dim == 2) return total <= lanes ? 32 : 0;
-    return total >= 2 * lanes ? 32 : 16;
+    return s.has_flux || total >= 2 * lanes ? 32 : 16;
 }
 
 // A lane's next work item: from the launch's counter, warp-aggregated, after

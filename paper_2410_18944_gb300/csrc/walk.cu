@@ -84,7 +84,7 @@ constexpr int kPlainBlock = 128;
 // Measured on one GB300, one query per lane (before) and now:
 //   3D (queries by lane groups, caps, facing bounds): icosphere of 82k triangles,
 //   376k walks, 231 / 78.5 ms; genus-3 solid of 994k, 131k walks, 326 / 60 ms;
-//   flux slab, 131k walks, 30.2 / 16.4 ms.  Eight CTAs per SM (64 registers): the
+//   flux slab, 131k walks, 30.2 / 15.0 ms.  Eight CTAs per SM (64 registers): the
 //   queries are calls, so the walk's state spills around them, not inside; six
 //   CTAs (80 registers) 88 against 82 ms on the icosphere, four 100.
 //   2D (caps, facing bounds, 8-byte stack entries): star of 4096 segments, 1.39 M
