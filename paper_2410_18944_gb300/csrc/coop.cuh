@@ -326,7 +326,7 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                 nref = __shfl_sync(kFull, cref, base + near);
                 pos = ok && sub != near ? sp + __popc(m & ~(1u << near) & ((1u << sub) - 1u)) : -1;
             } else {
-                // sort the children by key (take_children's network: strict
+                // sort the children by key (a network of four: strict
                 // comparisons, children not taken last)
                 float kk = ok ? key : __int_as_float(0x7f800000);
                 auto swap = [&](int other) {
