@@ -142,12 +142,12 @@ __device__ __forceinline__ bool take_children(const float *k, const int *r, cons
 __host__ __device__ constexpr int cap_f4(int d) { return d == 2 ? 4 : 32; }
 
 // squared distance from x to the cap (c, a as loaded; 2D: c = (c.xy, a.xy))
-__device__ __forceinline__ float cap_d2_2(float4 c, float h, float r, const float *x) {
+__host__ __device__ __forceinline__ float cap_d2_2(float4 c, float h, float r, const float *x) {
     const float ux = x[0] - c.x, uy = x[1] - c.y;
     const float s = fmaxf(fabsf(c.z * ux + c.w * uy) - h, 0.f), l = fmaxf(fabsf(c.z * uy - c.w * ux) - r, 0.f);
     return s * s + l * l;
 }
-__device__ __forceinline__ float cap_d2_3(float4 c, float4 a, const float *x) {
+__host__ __device__ __forceinline__ float cap_d2_3(float4 c, float4 a, const float *x) {
     const float u[3] = {x[0] - c.x, x[1] - c.y, x[2] - c.z};
     const float q = a.x * u[0] + a.y * u[1] + a.z * u[2];
     const float n = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];

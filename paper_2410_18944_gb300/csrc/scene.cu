@@ -143,12 +143,22 @@ Cap cap_of(const std::vector<float> &P, const std::vector<float> &N, int b, int 
         for (int j = 0; j < d; ++j) c += 0.5 * (lo[j] + hi[j]) * f[j][k];
         o.c[k] = (float)c;
     }
+    // The radius comes from the components across the axis: n - q^2 (n the
+    // squared length, q the part along the axis) would lose a radius below
+    // about h / 3000 to the rounding of the FP32 axis' length.
     double h = 0, r2 = 0;
+    const double a2 = f[0][0] * f[0][0] + f[0][1] * f[0][1] + (d == 3 ? f[0][2] * f[0][2] : 0.0);
     for (size_t p = p0; p < p1; p += d) {
-        double q = 0, n = 0;
-        for (int k = 0; k < d; ++k) { const double u = P[p + k] - (double)o.c[k]; q += f[0][k] * u; n += u * u; }
+        double u[3], q = 0, w2 = 0;
+        for (int k = 0; k < d; ++k) { u[k] = P[p + k] - (double)o.c[k]; q += f[0][k] * u[k]; }
+        if (d == 2) {
+            const double w = f[1][0] * u[0] + f[1][1] * u[1];   // (as cap_d2_2)
+            w2 = w * w;
+        } else {
+            for (int k = 0; k < d; ++k) { const double w = u[k] - q / a2 * f[0][k]; w2 += w * w; }
+        }
         h = std::max(h, std::fabs(q));
-        r2 = std::max(r2, n - q * q);
+        r2 = std::max(r2, w2);
     }
     o.h = std::nextafterf((float)(h + margin), INFINITY);
     o.r = std::nextafterf((float)(std::sqrt(r2) * (1 + 1e-6) + margin), INFINITY);
