@@ -131,9 +131,13 @@ __device__ __forceinline__ bool take_children(const float *k, const int *r, cons
 // to its axis-aligned box falls short by about r, and a search from afar has
 // to open every patch whose box is nearer than the closest point: patches
 // within about sqrt(r R) of it (R: the walk's distance) instead of a few r.
-// h and r carry a margin of 1e-6 x the scene's extent, more than the rounding
-// of this distance and of a primitive's own: every primitive at or below the
-// bound is tested, whatever the order of visits.
+// h and r carry a margin of 1e-6 x the scene's extent and its distance from the
+// origin, and the axis is 1e-6 short of unit length, so that the distance is
+// too, for points far outside the scene (rounding grows with their distance):
+// together more than the rounding of this distance and of a primitive's own.
+// Every primitive at or below the bound is tested, whatever the order of visits
+// (3D, outside the scene by more than a few extents: but for the last units of
+// a box's own distance).
 // Per node: 2D (2 children) (c.xy, a.xy) of each, (h0, r0, h1, r1), (ref0,
 // ref1, -, -); 3D (8 children) 8 x (c.xyz, h), 8 x (a.xyz, r), and the children's
 // boxes grown by the margin with the references, 8 x (lo.xyz, hi.x), 8 x (hi.yz,
@@ -151,8 +155,9 @@ __host__ __device__ __forceinline__ float cap_d2_3(float4 c, float4 a, const flo
     const float u[3] = {x[0] - c.x, x[1] - c.y, x[2] - c.z};
     const float q = a.x * u[0] + a.y * u[1] + a.z * u[2];
     const float n = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    // squared distance to the axis, less the rounding of n and q^2
-    const float w = fmaxf(n * (1.f - 2e-6f) - q * q, 1e-30f);
+    // squared distance to the axis, less the axis' 2e-6 of q^2 and the rounding
+    // of n and q^2
+    const float w = fmaxf(n * (1.f - 4e-6f) - q * q, 1e-30f);
     const float s = fmaxf(fabsf(q) - c.w, 0.f), l = fmaxf(w * rsqrtf(w) - a.w, 0.f);
     return s * s + l * l;
 }

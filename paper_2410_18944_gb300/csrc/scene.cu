@@ -103,8 +103,9 @@ Facing facing_bound(const std::vector<SilData> &el, int b, int e, int d, const f
 
 // Oriented cap around primitives [b, e) (geom.cuh, cap_d2): centre c, axis a,
 // half thickness h along a, radius r across it.  The axis is the mean normal
-// (any axis bounds, that one is thin).  P: vertices in leaf order (d points
-// of d floats per primitive), N: unit normals.  margin: see cap_d2.
+// (any axis bounds, that one is thin), 1e-6 short of unit length.  P: vertices
+// in leaf order (d points of d floats per primitive), N: unit normals.  Margin
+// and length: see cap_f4.
 struct Cap { float c[3] = {0, 0, 0}, a[3] = {1, 0, 0}, h = 0, r = 0; };
 
 Cap cap_of(const std::vector<float> &P, const std::vector<float> &N, int b, int e, int d, double margin) {
@@ -114,10 +115,13 @@ Cap cap_of(const std::vector<float> &P, const std::vector<float> &N, int b, int 
         for (int k = 0; k < d; ++k) ax[k] += N[(size_t)i * d + k];
     for (int k = 0; k < d; ++k) L += ax[k] * ax[k];
     L = std::sqrt(L);
+    // frame: the unit axis and (2D) its perpendicular, or (3D) two axes across
+    double f[3][3] = {{1, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     if (L > 1e-3 * (e - b))
-        for (int k = 0; k < d; ++k) o.a[k] = (float)(ax[k] / L);
-    // frame: the axis and (2D) its perpendicular, or (3D) two axes across
-    double f[3][3] = {{o.a[0], o.a[1], o.a[2]}, {-o.a[1], o.a[0], 0}, {0, 0, 0}};
+        for (int k = 0; k < d; ++k) f[0][k] = ax[k] / L;
+    for (int k = 0; k < d; ++k) o.a[k] = (float)((1 - 1e-6) * f[0][k]);
+    f[1][0] = -f[0][1];
+    f[1][1] = f[0][0];
     if (d == 3) {
         const int m = std::fabs(f[0][0]) < std::fabs(f[0][1]) ? (std::fabs(f[0][0]) < std::fabs(f[0][2]) ? 0 : 2)
                                                               : (std::fabs(f[0][1]) < std::fabs(f[0][2]) ? 1 : 2);
@@ -143,19 +147,20 @@ Cap cap_of(const std::vector<float> &P, const std::vector<float> &N, int b, int 
         for (int j = 0; j < d; ++j) c += 0.5 * (lo[j] + hi[j]) * f[j][k];
         o.c[k] = (float)c;
     }
-    // The radius comes from the components across the axis: n - q^2 (n the
-    // squared length, q the part along the axis) would lose a radius below
-    // about h / 3000 to the rounding of the FP32 axis' length.
-    double h = 0, r2 = 0;
-    const double a2 = f[0][0] * f[0][0] + f[0][1] * f[0][1] + (d == 3 ? f[0][2] * f[0][2] : 0.0);
+    // extents along and across the axis as stored.  The radius comes from the
+    // components across it: n - q^2 (n the squared length, q the part along the
+    // axis) would lose a radius below about h / 3000 to the rounding of the FP32
+    // axis' length.
+    double h = 0, r2 = 0, a2 = 0;
+    for (int k = 0; k < d; ++k) a2 += (double)o.a[k] * o.a[k];
     for (size_t p = p0; p < p1; p += d) {
         double u[3], q = 0, w2 = 0;
-        for (int k = 0; k < d; ++k) { u[k] = P[p + k] - (double)o.c[k]; q += f[0][k] * u[k]; }
+        for (int k = 0; k < d; ++k) { u[k] = P[p + k] - (double)o.c[k]; q += o.a[k] * u[k]; }
         if (d == 2) {
-            const double w = f[1][0] * u[0] + f[1][1] * u[1];   // (as cap_d2_2)
+            const double w = o.a[0] * u[1] - o.a[1] * u[0];   // (as cap_d2_2)
             w2 = w * w;
         } else {
-            for (int k = 0; k < d; ++k) { const double w = u[k] - q / a2 * f[0][k]; w2 += w * w; }
+            for (int k = 0; k < d; ++k) { const double w = u[k] - q / a2 * o.a[k]; w2 += w * w; }
         }
         h = std::max(h, std::fabs(q));
         r2 = std::max(r2, w2);

@@ -2,7 +2,7 @@
 // runs on any machine): the cap that the scene builder puts around a patch of
 // primitives lies at or below the distance of every primitive in it, less what
 // FP32 rounds off that distance, for needles and slabs of any aspect at any
-// rotation.  Prints "ok" and exits 0 when every check holds.
+// rotation, seen from inside the scene and from far outside it.  Prints "ok" and exits 0 when every check holds.
 #include <cstdio>
 #include <random>
 
@@ -84,11 +84,14 @@ int check_caps(int d, int patches, double reach, std::mt19937_64 &rng) {
         }
         const Cap c = cap_of(P, N, 0, n, d, 1e-6 * far);
         for (int q = 0; q < 16; ++q) {
-            const double radius = q < 5 ? reach : (q < 10 ? len : 4 * len / aspect);
+            const double radius = q < 6 ? reach : (q < 11 ? len : 4 * len / aspect);
             float x[3] = {0, 0, 0};
             double xd[3] = {0, 0, 0};
             const int at = (int)(unit(rng) * n * d) * d;
-            for (int k = 0; k < d; ++k) xd[k] = x[k] = (float)(P[at + k] + radius * (2 * unit(rng) - 1));
+            for (int k = 0; k < d; ++k) {   // (two along the cap's axis)
+                const double step = q < 2 ? (double)c.a[k] * (q ? 1 : -1) : 2 * unit(rng) - 1;
+                xd[k] = x[k] = (float)(P[at + k] + radius * step);
+            }
             const double key = d == 2 ? cap_d2_2(make_float4(c.c[0], c.c[1], c.a[0], c.a[1]), c.h, c.r, x)
                                       : cap_d2_3(make_float4(c.c[0], c.c[1], c.c[2], c.h),
                                                  make_float4(c.a[0], c.a[1], c.a[2], c.r), x);
@@ -113,7 +116,8 @@ int check_caps(int d, int patches, double reach, std::mt19937_64 &rng) {
 int main() {
     std::mt19937_64 rng(11);
     int bad = 0;
-    for (int d = 2; d <= 3; ++d) bad += check_caps(d, 20000, 1.0, rng);
+    for (double reach : {1.0, 30.0, 1000.0})   // from points of the scene, and from outside
+        for (int d = 2; d <= 3; ++d) bad += check_caps(d, 20000, reach, rng);
     if (bad) {
         std::printf("%d bounds above their primitives\n", bad);
         return 1;
