@@ -386,8 +386,17 @@ extern "C" wost_status wost_train_grad(wost_field *f, const wost_exec *exec, flo
     if (!f->rec || !f->rec_ctr) { set_error("wost_train_grad: no training records"); return WOST_ERR_INVALID_ARG; }
     cudaStream_t st = exec ? (cudaStream_t)exec->stream : 0;
     if (exec) f->t_samples = exec->train_samples;
-    // the grid's gradient is accumulated in the caller's array where it can be
+    // the grid's gradient is accumulated in the caller's array where it can be,
+    // in order after the legacy stream's work on that array, as the copies are
     const bool direct = g_grid && on_device(g_grid, f->device, 16);
+    if (direct && st) {
+        cudaEvent_t ready;
+        WOST_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+        cudaError_t e = cudaEventRecord(ready, cudaStreamLegacy);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ready, 0);
+        cudaEventDestroy(ready);
+        if (e != cudaSuccess) return cuda_status(e, "wost_train_grad");
+    }
     wost_status rc = train_grad_launch(f, f->desc.dim, st, -1, false, direct ? g_grid : nullptr);
     if (rc != WOST_OK) return rc;
     if (direct) g_grid = nullptr;
