@@ -82,9 +82,8 @@ class FieldLoss(torch.autograd.Function):
         grads = [torch.empty_like(t) for t in params]
         loss = C.c_float()
         check(lib.wost_train_grad(ctx.field._h, C.byref(_exec(lib)), C.byref(loss), *[_fp(g) for g in grads]))
-        if torch.is_grad_enabled() and gout.requires_grad:   # a graph of the gradients is asked for
-            return (None,) + tuple(gout * g for g in grads)
-        return (None,) + tuple(g.mul_(gout) for g in grads)
+        # (not in place: gout may be batched, vmap, or carry a graph)
+        return (None,) + tuple(gout * g for g in grads)
 
 
 def field_loss(field, grid, W1, W2, W3, b3):
