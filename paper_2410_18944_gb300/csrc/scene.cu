@@ -5,9 +5,10 @@
 // run on a linear BVH in the paper; here the hierarchy is built once on the
 // host (not timed) and traversed in the persistent walk kernel.
 #include <algorithm>
+#include <atomic>
+#include <cfloat>
 #include <cmath>
 #include <cstring>
-#include <atomic>
 #include <numeric>
 #include <system_error>
 #include <thread>
@@ -291,7 +292,7 @@ struct Builder {
             BNode r;
             r.ref[0] = leaf_ref(0, n);
             r.ref[1] = leaf_ref(0, 1);
-            r.box[0] = range_box(0, n);   // r.box[1] stays empty (inverted): never entered
+            r.box[0] = range_box(0, n);   // r.box[1] stays empty (inverted)
             r.range[0][0] = 0; r.range[0][1] = n;
             r.range[1][0] = 0; r.range[1][1] = 0;
             nodes.push_back(r);
@@ -387,7 +388,10 @@ struct Builder {
     std::vector<float4> pack_binary() const {
         std::vector<float4> out;
         for (const BNode &nd : nodes) {
-            const Box &a = nd.box[0], &b = nd.box[1];
+            const Box &a = nd.box[0];
+            Box b = nd.box[1];
+            if (nd.range[1][1] <= nd.range[1][0])   // the unused child of a one-leaf tree: a point out of any ray's reach
+                for (int k = 0; k < 2; ++k) b.lo[k] = b.hi[k] = FLT_MAX;
             out.push_back(make_float4(a.lo[0], a.lo[1], a.hi[0], a.hi[1]));
             out.push_back(make_float4(b.lo[0], b.lo[1], b.hi[0], b.hi[1]));
             int r[2];
