@@ -200,8 +200,8 @@ typedef struct {
     int64_t walk_launches;     /* of which walk kernels */
     int64_t node_visits;       /* BVH nodes visited by all walk-step queries */
     int64_t prim_visits;       /* primitives / silhouette elements tested */
-    double alg_bytes;          /* algorithmic bytes of the walk kernels: visited BVH nodes and
-                                  primitives, hash-grid corner reads, query points, FP64
+    double alg_bytes;          /* algorithmic bytes of the walk kernels: visited BVH nodes (with
+                                  the bounds that the query reads) and primitives, hash-grid corner reads, query points, FP64
                                   accumulator updates, training-record writes and suffix pass */
     int64_t dir_prim_visits;   /* of prim_visits: Dirichlet primitives (closest point) */
     int64_t sil_prim_visits;   /* silhouette elements (closest silhouette) */

@@ -39,7 +39,7 @@ constexpr int kBatchGuidedSmem = ws_smem_bytes(true);
 static_assert(kBatchGuidedSmem % alignof(CoopWarp) == 0, "query workspaces follow the tiles");
 constexpr int batch_guided_smem(int D, int W) { return kBatchGuidedSmem + coop_bytes(D, W); }
 // counter block of a plan (unsigned long long words)
-constexpr int kCtrStat = 8;       // [8, 15): launch statistics
+constexpr int kCtrStat = 8;       // [8, 16): launch statistics
 constexpr int kCtrRec = 16;       // [16, 18): records appended / dropped over all rounds
 constexpr int kCtrCalib = 23;     // work counter of calibration launches
 constexpr int kCtrWork = 24;      // [24, 24 + launches): work counter per launch

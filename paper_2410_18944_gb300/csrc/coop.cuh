@@ -432,16 +432,14 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
 // the call, with the visits added to the lane's counters
 template <int kKind, int kMode>
 __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool want, const float *x, const float *v,
-                                        float &best, int aux, int *err, Visits *vis, uint32_t key1 = 0) {
+                                        float &best, int aux, int *err, volatile Visits *vis, uint32_t key1 = 0) {
     const CoopResult r = coop_query<kKind, kMode>((uint32_t)__cvta_generic_to_shared(&sh), &sc, want, x[0], x[1], x[2],
                                                    v[0], v[1], v[2], best, aux, key1, err);
     best = r.best;
-    if (vis) {
-        vis->nodes += r.nodes;
-        if (kKind == kCoopPoint || kKind == kCoopPointBox) vis->dprims += r.prims;
-        else if (kKind == kCoopSil) vis->sprims += r.prims;
-        else vis->nprims += r.prims;
-    }
+    if (kKind == kCoopPoint) add_visits(vis, &Visits::dnodes, r.nodes, &Visits::dprims, r.prims);
+    else if (kKind == kCoopPointBox) add_visits(vis, &Visits::nodes, r.nodes, &Visits::dprims, r.prims);
+    else if (kKind == kCoopSil) add_visits(vis, &Visits::snodes, r.nodes, &Visits::sprims, r.prims);
+    else add_visits(vis, &Visits::nodes, r.nodes, &Visits::nprims, r.prims);
     return r.slot;
 }
 
@@ -455,7 +453,7 @@ __device__ __forceinline__ int coop_run(CoopWarp &sh, const DevScene &sc, bool w
 // others are searched again in the boxes.
 template <int kMode>
 __device__ __forceinline__ int coop_closest(CoopWarp &sh, const DevScene &sc, bool want, const float *x, float &d2,
-                                            int *err, Visits *vis) {
+                                            int *err, volatile Visits *vis) {
     d2 = __int_as_float(0x7f800000);
     int slot = coop_run<kCoopPoint, kMode>(sh, sc, want, x, x, d2, -1, err, vis);
     bool again = false;

@@ -44,10 +44,21 @@ __host__ __device__ constexpr int node_f4() {
     return D == 2 ? 3 : 8;
 }
 
-// per-thread visit counts of the traversals (algorithmic-traffic accounting)
+// Per-thread visit counts of the traversals (algorithmic-traffic accounting):
+// nodes of caps (closest point), of boxes with facing bounds (silhouettes) and
+// of boxes alone, primitives.  A query counts in registers of its own and adds
+// to these at its end.  They are volatile, kept in memory: totals that stayed in
+// registers cost the traversals more than the adds per query (training batch of
+// the star, counted per visit in registers 51.9 ms, so 50.9).
 struct Visits {
-    uint32_t nodes = 0, dprims = 0, sprims = 0, nprims = 0;
+    uint32_t dnodes = 0, snodes = 0, nodes = 0, dprims = 0, sprims = 0, nprims = 0;
 };
+__device__ __forceinline__ void add_visits(volatile Visits *vis, uint32_t Visits::*nodes, uint32_t nv, uint32_t Visits::*prims,
+                                           uint32_t pv) {
+    if (!vis) return;
+    vis->*nodes = vis->*nodes + nv;
+    vis->*prims = vis->*prims + pv;
+}
 
 // squared distance from the distances along the axes, with its rounding
 // spelled out: whether a box is opened is decided on this value
@@ -291,7 +302,7 @@ __device__ __forceinline__ void load_tri(const float4 *__restrict__ P, int s, fl
 // ---- closest Dirichlet primitive (2D) ---------------------------------------
 // returns the leaf slot of the closest primitive (-1 if none); best = squared distance
 __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const float4 *caps, const float *x, float &best,
-                                                         int *err, Visits *vis = nullptr) {
+                                                         int *err, volatile Visits *vis = nullptr) {
     constexpr int kBW = 2;
     best = __int_as_float(0x7f800000);
     if (bv.nprims == 0) return -1;
@@ -300,6 +311,7 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
     LaneStack st;
     int ref = 0;
     bool done = false;
+    uint32_t nv = 0, pv = 0;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
     while (__any_sync(mask, !done)) {
@@ -314,14 +326,14 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
             k[1] = cap_d2_2(ldn(p + 1), hr.z, hr.w, x);
             r[0] = __float_as_int(q.x);
             r[1] = __float_as_int(q.y);
-            if (vis) vis->nodes++;
+            ++nv;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
             if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
-            if (vis) vis->dprims += cnt;
+            pv += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 float4 p = ldn(bv.prims + s);
                 const float d2 = seg_d2_fast(p, x);
@@ -333,6 +345,7 @@ __device__ inline WOST_QUERY_FN int closest_dirichlet(const DevBVH &bv, const fl
             done = !st.pop(best, ref);
         }
     }
+    add_visits(vis, &Visits::dnodes, nv, &Visits::dprims, pv);
     return best_slot;
 }
 
@@ -435,7 +448,7 @@ __device__ __forceinline__ bool sil_elem(const float4 *prims, int s, const float
 }
 
 __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const float *x, float tau, float &best, int *err,
-                                   const float4 *facing, Visits *vis = nullptr) {
+                                   const float4 *facing, volatile Visits *vis = nullptr) {
     constexpr int kBW = 2;
     if (bv.nprims == 0) return -1;
     const unsigned mask = __activemask();
@@ -443,6 +456,7 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
     LaneStack st;
     int ref = 0;
     bool done = false;
+    uint32_t nv = 0, pv = 0;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
     while (__any_sync(mask, !done)) {
@@ -452,12 +466,12 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
             int r[kBW];
             bool h[kBW];
             node_keys_sil(bv.nodes, facing, ref, x, best, tau, k, r, h);
-            if (vis) vis->nodes++;
+            ++nv;
             if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
-            if (vis) vis->sprims += cnt;
+            pv += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 float d2;
                 if (sil_elem<2>(bv.prims, s, x, tau, best, d2)) {
@@ -468,6 +482,7 @@ __device__ inline WOST_QUERY_FN int closest_silhouette(const DevBVH &bv, const f
             done = !st.pop(best, ref);
         }
     }
+    add_visits(vis, &Visits::snodes, nv, &Visits::sprims, pv);
     return best_slot;
 }
 
@@ -577,7 +592,7 @@ __device__ __forceinline__ bool ray_prim64(const DevBVH &bv, int s, const float 
 // slot or -1 (kExit: exit hits only, from t > -tneg, see ray_prim)
 template <bool kExit = false>
 __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const float *v, float tmax, int skip, float &thit,
-                           int *err, Visits *vis = nullptr, float tneg = 0.f) {
+                           int *err, volatile Visits *vis = nullptr, float tneg = 0.f) {
     constexpr int kBW = 2;
     thit = tmax;
     if (bv.nprims == 0) return -1;
@@ -590,6 +605,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
     LaneStack st;
     int ref = 0;
     bool done = false;
+    uint32_t nv = 0, pv = 0;
     // while-while: descend inner nodes together until every lane holds a
     // leaf (or is done), then test the leaves together
     while (__any_sync(mask, !done)) {
@@ -599,14 +615,14 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
             int r[kBW];
             bool h[kBW];
             node_keys_ray(bv.nodes, ref, o, inv, best, k, r, kExit ? tneg : 0.f);
-            if (vis) vis->nodes++;
+            ++nv;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] <= best;
             if (!take_children(k, r, h, ref, st, err)) done = !st.pop(best, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
-            if (vis) vis->nprims += cnt;
+            pv += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 float t;
                 if (s != skip && ray_prim<2, kExit>(bv.prims, s, o, v, t, tneg) && t <= best) {
@@ -618,6 +634,7 @@ __device__ WOST_QUERY_FN int ray_neumann(const DevBVH &bv, const float *o, const
         }
     }
     thit = best;
+    add_visits(vis, &Visits::nodes, nv, &Visits::nprims, pv);
     return best_slot;
 }
 
@@ -658,7 +675,7 @@ __device__ __forceinline__ float neumann_key(int id, float w, uint32_t pid, uint
 
 // 2D (one query per lane; 3D: kCoopPick, coop.cuh)
 __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, uint32_t pid, uint32_t wid, uint32_t step,
-                                   uint32_t k0, uint32_t k1, float &W, int *err, Visits *vis = nullptr) {
+                                   uint32_t k0, uint32_t k1, float &W, int *err, volatile Visits *vis = nullptr) {
     constexpr int kBW = 2;
     W = 0.f;
     if (bv.nprims == 0) return -1;
@@ -669,6 +686,7 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
     LaneStack st;
     int ref = 0;
     bool done = false;
+    uint32_t nv = 0, pv = 0;
     const float lim = r2;   // the search radius never shrinks
     while (__any_sync(mask, !done)) {
         while (__any_sync(mask, !done && ref >= 0)) {
@@ -677,14 +695,14 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
             int rr[kBW];
             bool h[kBW];
             node_keys_d2(bv.nodes, ref, x, k, rr);
-            if (vis) vis->nodes++;
+            ++nv;
 #pragma unroll
             for (int c = 0; c < kBW; ++c) h[c] = k[c] < r2;
             if (!take_children(k, rr, h, ref, st, err)) done = !st.pop(lim, ref);
         }
         if (!done && ref < 0) {
             int s0 = leaf_start(ref), cnt = leaf_count(ref);
-            if (vis) vis->nprims += cnt;
+            pv += cnt;
             for (int s = s0; s < s0 + cnt; ++s) {
                 const float w = neumann_weight<2>(bv, s, x, r2);
                 if (!(w > 0.f)) continue;
@@ -696,6 +714,7 @@ __device__ inline int neumann_pick(const DevBVH &bv, const float *x, float r, ui
             done = !st.pop(lim, ref);
         }
     }
+    add_visits(vis, &Visits::nodes, nv, &Visits::nprims, pv);
     return best_slot;
 }
 

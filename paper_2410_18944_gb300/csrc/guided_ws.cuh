@@ -282,7 +282,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
     tc_fence_after();
     const uint32_t tmem0 = ctl->tmem;
 
-    Visits vis;
+    volatile Visits vis;
     unsigned long long nsteps = 0, ntrunc = 0, nwalks = 0;
 
     if (warp < kWsServerWarps) {
@@ -590,7 +590,7 @@ __device__ __forceinline__ void guided_ws_body(const Src &src, const WsOpts &o, 
         __syncwarp();
         if (lane == 0) atomicSub(&ctl->alive, 1);
     }
-    flush_stats(o.stat, nsteps, ntrunc, nwalks, vis);
+    flush_stats<D>(o.stat, nsteps, ntrunc, nwalks, vis);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

@@ -269,7 +269,7 @@ struct WorkCursor {
 template <int D, int kMode, class Src>
 __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigned long long *stat) {
     Walk<D> w;
-    Visits vis;
+    volatile Visits vis;
     bool active = false, exhausted = false;
     unsigned long long nsteps = 0, ntrunc = 0, nwalks = 0;
     if (D == 3) {   // lanes without a walk take part in the groups' queries
@@ -312,7 +312,7 @@ __device__ __forceinline__ void plain_loop(CoopWarp *sh, const Src &src, unsigne
         }
         step_move<D, kMode>(sh, w, env, active, nu, r, &vis);
     }
-    flush_stats(stat, nsteps, ntrunc, nwalks, vis);
+    flush_stats<D>(stat, nsteps, ntrunc, nwalks, vis);
 }
 
 }  // namespace wost

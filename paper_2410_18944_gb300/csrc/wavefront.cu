@@ -113,7 +113,7 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
     __shared__ __half rows[kWfBlock * kYStride];
     __half *myrow = rows + threadIdx.x * kYStride;
     const float area = D == 2 ? 2.f * WOST_PI : 4.f * WOST_PI;
-    Visits vis;
+    volatile Visits vis;
     unsigned long long nsteps = 0, ntrunc = 0, nwalks = 0;
     const int s = valid ? (first ? (int)j : S.dlist[parity ^ 1][j]) : 0;
     Walk<D> w;
@@ -218,7 +218,7 @@ __device__ __forceinline__ void wf_step_body(CoopWarp *sh, const Src &src, const
         S.rS[s] = make_float2(r, Sx);
         S.dlist[parity][warp_append(S.dcount + parity)] = s;
     }
-    flush_stats(o.stat, nsteps, ntrunc, nwalks, vis);
+    flush_stats<D>(o.stat, nsteps, ntrunc, nwalks, vis);
 }
 
 // suffix passes of the walks of a recording launch (one per slot, a warp each)
