@@ -99,8 +99,8 @@ __device__ __forceinline__ const DevBVH &coop_bvh(const DevScene &sc, bool diric
 }
 
 // One query per lane that wants one; all lanes of the warp call.
-//   kCoopPoint  best_io: in the bound (squared), out the squared distance;
-//               aux: leaf slot whose squared distance best_io is, or -1
+//   kCoopPoint  best_io: in the bound (squared), out the squared distance
+//               (kCoopPointBox: the same over the box tree)
 //   kCoopSil    best_io: in the bound (squared), out the squared distance
 //   kCoopExit   first exit through the Neumann boundary along v within
 //               best_io, from t > -(rounding band of a position)
@@ -197,11 +197,6 @@ __device__ __noinline__ CoopResult coop_query(uint32_t sh_addr, const DevScene *
                 lb = __int_as_float(0x7f800000);
                 ls = -1;
                 lid = kKind == kCoopCount ? 0 : INT_MAX;
-                if (kKind == kCoopPoint && sub == 0 && a0 >= 0) {
-                    lb = b0;
-                    ls = a0;
-                    lid = __ldg(gs->dir.ids + a0);
-                }
             }
         }
         if (!__any_sync(kFull, busy)) break;
