@@ -201,8 +201,9 @@ typedef struct {
     int64_t node_visits;       /* BVH nodes visited by all walk-step queries */
     int64_t prim_visits;       /* primitives / silhouette elements tested */
     double alg_bytes;          /* algorithmic bytes of the walk kernels: visited BVH nodes (with
-                                  the bounds that the query reads) and primitives, hash-grid corner reads, query points, FP64
-                                  accumulator updates, training-record writes and suffix pass */
+                                  the bounds that the query reads) and primitives, hash-grid
+                                  corner reads, query points, FP64 accumulator updates,
+                                  training-record writes and suffix pass */
     int64_t dir_prim_visits;   /* of prim_visits: Dirichlet primitives (closest point) */
     int64_t sil_prim_visits;   /* silhouette elements (closest silhouette) */
     int64_t neu_prim_visits;   /* Neumann primitives (ray casts and the Neumann-flux sample) */

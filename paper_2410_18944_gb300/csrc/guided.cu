@@ -26,16 +26,15 @@ struct GuidedArgs {
 };
 
 // Walker warps of the single-scene kernel (exec walker_warps 0): kWsWalkerWarps
-// (16) when the scene's traversal data (BVH nodes, facing bounds, primitives) fits
-// comfortably in L2 or shared memory, kWsWalkersWide beside the 4 servers
-// when it does not.
-// Measured on one GB300, one recording round: genus-3 solid (about 300 MB of
-// traversal data) 1057 ms with 12 walker warps, 964 with 14, 798 with 20,
-// 729 with 24, 695 with 28 (32 warps, the 1024-thread limit); icosphere of
-// 82k triangles (about 20 MB) 168, 172, 174 ms with 12, 14, 20.  More
-// walkers hide the latency of BVH loads that miss L2; with the scene in L2
-// the register cap they impose (64 per thread at 1024 threads, with spills)
-// costs more than it hides.
+// (16) when the scene's traversal data (BVH nodes, caps, facing bounds,
+// primitives) fits comfortably in L2 or shared memory, kWsWalkersWide beside the
+// 4 servers when it does not: more walkers hide the latency of BVH loads that
+// miss L2; with the scene in L2 the register cap they impose (64 per thread at
+// 1024 threads, with spills) costs more than it hides.  Measured on one GB300,
+// walks of a recording round with 16 / 28 walker warps: genus-3 solid (about 300
+// MB of traversal data) 131k walks 82 / 77 ms, 510k 204 / 156, 1.02 M 409 / 317;
+// icosphere of 82k triangles (about 20 MB) 47k walks 35 / 45 ms, 188k 74 / 82;
+// star 174k walks 13.3 / 14.7, 696k 38.7 / 43.0.
 #ifndef WOST_WS_WIDE_MB
 #define WOST_WS_WIDE_MB 64
 #endif
@@ -66,12 +65,11 @@ static size_t traversal_bytes(const DevScene &s) {
 // the walker-warp count of a scene's guided launches of `walks` walks
 // (`req`: the caller's choice, 0 = automatic): the wide kernel where the
 // scene's traversal data misses L2, or, in 3D, where a launch gives each of
-// its lanes about two walks or more (3D steps are long chains of dependent
-// loads that more warps hide; a launch with fewer walks leaves the wide
-// kernel's lanes idle and its register cap costs more).  Measured on one
-// GB300: icosphere of 82k triangles, batches of 8 walks per point (376k
-// walks) 400 ms with 12 walker warps, 357 with 28; one walk per point
-// (47k walks) 168 / 174 ms with 12 / 20; the 2D star equal (58 / 59 ms).
+// its lanes about two walks or more (a launch with fewer walks leaves the wide
+// kernel's lanes idle and its register cap costs more).  The second line was
+// drawn for queries of one lane each; with the queries answered by lane groups
+// the two kernels are level there (icosphere, 376k walks: 121 / 123 ms with 16 /
+// 28).
 static int ws_walkers_for(const DevScene &s, int req, unsigned long long walks) {
     if (req > 0) return req;
     if (traversal_bytes(s) > ((size_t)WOST_WS_WIDE_MB << 20)) return kWsWalkersWide;

@@ -55,11 +55,10 @@ namespace wost {
 
 constexpr int kWsServerWarps = 4;
 // Walker warps of the standard variant (640 threads, 102 registers each).
-// Measured on one GB300, training batches of the bench: 2D star 58.1 /
-// 55.0 / 55.2 / 57.5 / 59.5 ms with 12 / 16 / 20 / 24 / 28 walker warps,
-// icosphere 403 / 340 / 335 / 341 / 334-357 ms (the latter run by the wide
-// variant); fewer warps hide less latency, more impose a register cap that
-// spills.
+// Measured on one GB300, training batches of the 2D star: 58.1 / 55.0 / 55.2 /
+// 57.5 / 59.5 ms with 12 / 16 / 20 / 24 / 28 walker warps (with box-bounded
+// searches; 16 and 28 with the present ones at guided_walk_kernel); fewer warps
+// hide less latency, more impose a register cap that spills.
 #ifndef WOST_WS_WALKERS
 #define WOST_WS_WALKERS 16
 #endif
@@ -78,9 +77,9 @@ static_assert(kWsServerWarps + kWsWalkersWide <= 32, "a CTA holds at most 32 war
 // threads of a CTA with W walker warps beside the decode servers
 __host__ __device__ constexpr int ws_threads(int W) { return 32 * (kWsServerWarps + W); }
 constexpr int kWsThreads = ws_threads(kWsWalkerWarps);
-// decode tile buffers.  Measured on one GB300: one buffer is 6% faster than
-// two on the 2D star and 3-5% on the icosphere (equal on the genus-3 solid);
-// three and four are slower still.  A walker warp that finds the buffer busy
+// decode tile buffers.  Measured on one GB300 (3D queries of one lane each): one
+// buffer is 6% faster than two on the 2D star and 3-5% on the icosphere (equal
+// on the genus-3 solid); three and four are slower still.  A walker warp that finds the buffer busy
 // waits for the tile in flight, so tiles fill fuller and the shared memory
 // the buffers do not take goes to the scene and to L1.
 constexpr int kNT = WOST_WS_TILES;
@@ -115,10 +114,10 @@ __host__ __device__ constexpr int ws_smem_bytes(bool multi, int KM = kMaxK) {
     return wimg_bytes(KM) * ws_weight_slots(multi) + kNT * kBufBytes + kWsCtrlBytes + (multi ? kNT * 128 * 4 : 0) +
            (ws_y_separate(multi, KM) ? kNT * ws_y_bytes(KM) : 0);
 }
-// Server polls before closing a partial tile.  Fuller tiles measured faster
-// (one GB300, training batches: icosphere 374 / 364 / 354 / 339-347 / 335 ms
-// with 1 / 32 / 256 / 1024 / 4096 polls, genus-3 708 / 703 / 696 / 688-691 /
-// 697, the 2D star 58 ms from 256 polls on and 65-67 below).
+// Server polls before closing a partial tile.  Measured on one GB300, walks of a
+// training batch with 32 / 256 / 1024 / 4096 polls: genus-3 (1.02 M walks) 337 /
+// 329 / 317 / 319 ms, icosphere (376k) 124 / 124 / 123 / 124, star (696k) 36.9 /
+// 38.6 / 38.7 / 39.1.
 #ifndef WOST_FLUSH_POLLS
 #define WOST_FLUSH_POLLS 1024
 #endif

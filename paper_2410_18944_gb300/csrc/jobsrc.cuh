@@ -233,8 +233,10 @@ struct BatchSrc {
 // step logic, but a warp that is left with many long walks holds up the end of
 // the launch; half the lanes where there are fewer than two walks per lane,
 // all of them where every step has a Neumann sample too.  Measured on one GB300,
-// 16 / 32 lanes: genus-3 (27 walks per warp) 59 / 64 ms, icosphere (77 per warp)
-// 86 / 78 ms, flux slab (27 per warp) 16.1 / 15.0 ms.
+// 16 / 32 lanes at 0.84, 1, 1.5, 1.9, 2.4 and 4 walks per lane: genus-3 60 / 67,
+// 70 / 80, 85 / 90, 101 / 105, 118 / 126, 180 / 182 ms; icosphere 42.8 / 42.0,
+// 46 / 50, 58.8 / 58.1, 70 / 67, 83 / 78, 128 / 110 ms; flux slab at 0.84 walks
+// 16.1 / 15.0 ms.
 inline int plain_lanes(const DevScene &s, unsigned long long total, long long warps) {
     const unsigned long long lanes = 32ull * (unsigned long long)warps;
     if (s.dim == 2) return total <= lanes ? 32 : 0;
@@ -246,6 +248,11 @@ inline int plain_lanes(const DevScene &s, unsigned long long total, long long wa
 // item l * warps + w; the counter then counts the items after those).  Long
 // walks come in runs of neighbouring points, or first where the launch is
 // ordered, and in 3D a warp that held a run of them would outlast all others.
+// The first items belong to their warps: a CTA that does not fit the GPU beside
+// the others holds its items until one of them leaves (correct, but a launch of
+// few walks then takes two waves; wost_solve_plain_static in 3D, whose kernel
+// fits four of its eight CTAs per SM: flux slab, 131k walks, 18.8 ms against the
+// 15.4 of wost_solve).
 struct WorkCursor {
     bool first = true;
     __device__ __forceinline__ unsigned long long next(unsigned long long *ctr, unsigned warp, unsigned warps,
