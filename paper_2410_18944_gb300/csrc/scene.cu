@@ -339,7 +339,6 @@ struct Builder {
         for (int i = 0; i < n; ++i) {
             Child c = ch[i];
             if (c.ref >= 0) c.ref = collapse(out, W, lf, c.ref);
-            else if (c.range[1] <= c.range[0]) c.ref = kEmptyRef;   // the unused child of a one-leaf tree
             out[id].ch[i] = c;
         }
         out[id].n = n;
@@ -358,7 +357,17 @@ struct Builder {
     // wide tree of at most W children per node and lf primitives per leaf
     std::vector<WNode> widen(int W, int lf) const {
         std::vector<WNode> out;
-        if (!nodes.empty()) collapse(out, W, lf, 0);
+        const int n = (int)items.size();
+        if (n > lf) {
+            collapse(out, W, lf, 0);
+        } else if (n > 0) {   // one leaf, although the binary tree may be split further
+            WNode root;
+            root.ch[0].box = range_box(0, n);
+            root.ch[0].ref = leaf_ref(0, n);
+            root.ch[0].range[1] = n;
+            root.n = 1;
+            out.push_back(root);
+        }
         return out;
     }
 

@@ -1,4 +1,7 @@
-"""Scenes whose trees are a single leaf or barely more: which points are inside."""
+"""Scenes whose trees are a single leaf or barely more: which points are inside,
+and which of several primitives at the same distance is the closest."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -52,3 +55,21 @@ def test_inside_and_outside(api, name):
     assert inside.any() and not inside.all()
     mean = api.solve(api.Scene(sc), pts, 1, maxsteps=8)[0]
     assert np.array_equal(~np.isnan(mean), inside)
+
+
+@pytest.mark.parametrize("reach", [1.0, 30.0, 1000.0])
+def test_ties_in_a_scene_of_one_leaf(api, reach):
+    """14 triangles, all tested together: a point whose nearest point is a vertex
+    is as far from all triangles there, and takes the smallest id."""
+    sc = wi.slab_box(1)
+    r = np.random.default_rng(5)
+    prims = np.concatenate([sc.prims[r.permutation(12)], sc.prims[:2]])
+    sc = dataclasses.replace(sc, prims=prims, bc=np.zeros(14, np.uint8))
+    lo, hi = sc.bbox
+    top = r.integers(0, 2, (2000, 3))
+    corner = np.where(top, hi, lo)
+    pts = (corner + r.uniform(0.02, 1, (2000, 3)) * reach * np.where(top, 1, -1)).astype(np.float32).astype(np.float64)
+    vertex = [np.flatnonzero((sc.verts == c).all(1))[0] for c in corner]
+    want = np.array([np.flatnonzero((prims == v).any(1))[0] for v in vertex])
+    got = api.Scene(sc).query_closest(pts)[0]
+    assert np.array_equal(got, want), (got != want).sum()
