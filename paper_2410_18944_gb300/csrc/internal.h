@@ -46,7 +46,7 @@ struct wost_scene {
     double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     wost::DevScene dev{};
     std::vector<void *> allocs;
-    int64_t *sil_key = nullptr;   // device: canonical silhouette element id per leaf slot
+    const int64_t *sil_key = nullptr;   // device: canonical silhouette element id per leaf slot
     int ndir = 0, nneu = 0, nsil = 0;
     int depth_dir = 0, depth_neu = 0, depth_sil = 0;
     // per-solve workspace (grown on demand)

@@ -46,6 +46,7 @@ struct Item {
     Box b;
     float c[3];
     int idx;
+    int bin;   // of the split in progress
 };
 
 // silhouette element: inward normals of the two adjacent Neumann primitives
@@ -238,6 +239,8 @@ struct Builder {
             if (cb.hi[k] - cb.lo[k] > cb.hi[axis] - cb.lo[axis]) axis = k;
         float ext = cb.hi[axis] - cb.lo[axis];
         int mid;
+        Box half[2];
+        bool boxed = false;   // `half` holds the children's boxes
         if (!(ext > 0.f)) {
             mid = (b + e) / 2;   // identical centroids: split by index
         } else if (depth > kSahDepth) {
@@ -245,30 +248,46 @@ struct Builder {
         } else {
             Box bb[kBins];
             int bn[kBins] = {0};
-            auto bin_of = [&](const Item &it) {
-                int k = (int)((it.c[axis] - cb.lo[axis]) / ext * kBins);
-                return std::min(std::max(k, 0), kBins - 1);
-            };
-            for (int i = b; i < e; ++i) { int k = bin_of(items[i]); bn[k]++; bb[k].grow(items[i].b); }
+            for (int i = b; i < e; ++i) {
+                int k = (int)((items[i].c[axis] - cb.lo[axis]) / ext * kBins);
+                k = std::min(std::max(k, 0), kBins - 1);
+                items[i].bin = k;
+                bn[k]++;
+                bb[k].grow(items[i].b);
+            }
+            // the boxes left and right of each split, one sweep each
+            Box R[kBins];
+            int nr[kBins];
+            R[kBins - 1] = bb[kBins - 1];
+            nr[kBins - 1] = bn[kBins - 1];
+            for (int s = kBins - 2; s > 0; --s) {
+                R[s] = R[s + 1];
+                R[s].grow(bb[s]);
+                nr[s] = nr[s + 1] + bn[s];
+            }
             float best = INFINITY;
-            int bestk = -1;
+            int bestk = -1, nl = 0;
+            Box L;
             for (int s = 1; s < kBins; ++s) {
-                Box L, R;
-                int nl = 0, nr = 0;
-                for (int k = 0; k < s; ++k) { L.grow(bb[k]); nl += bn[k]; }
-                for (int k = s; k < kBins; ++k) { R.grow(bb[k]); nr += bn[k]; }
-                if (!nl || !nr) continue;
-                float c = L.cost(d) * nl + R.cost(d) * nr;
-                if (c < best) { best = c; bestk = s; }
+                L.grow(bb[s - 1]);
+                nl += bn[s - 1];
+                if (!nl || !nr[s]) continue;
+                float c = L.cost(d) * nl + R[s].cost(d) * nr[s];
+                if (c < best) { best = c; bestk = s; half[0] = L; }
             }
             if (bestk < 0) {
                 mid = split_median(b, e, axis);
             } else {
                 auto it = std::partition(items.begin() + b, items.begin() + e,
-                                         [&](const Item &x) { return bin_of(x) < bestk; });
+                                         [&](const Item &x) { return x.bin < bestk; });
                 mid = (int)(it - items.begin());
-                if (mid == b || mid == e) mid = split_median(b, e, axis);
+                half[1] = R[bestk];
+                boxed = true;
             }
+        }
+        if (!boxed) {
+            half[0] = range_box(b, mid);
+            half[1] = range_box(mid, e);
         }
         int node = (int)nodes.size();
         nodes.push_back(BNode{});
@@ -276,8 +295,8 @@ struct Builder {
         int r = rec(mid, e, depth + 1, n <= kLeaf);
         nodes[node].ref[0] = l;
         nodes[node].ref[1] = r;
-        nodes[node].box[0] = range_box(b, mid);
-        nodes[node].box[1] = range_box(mid, e);
+        nodes[node].box[0] = half[0];
+        nodes[node].box[1] = half[1];
         nodes[node].range[0][0] = b; nodes[node].range[0][1] = mid;
         nodes[node].range[1][0] = mid; nodes[node].range[1][1] = e;
         return node;
@@ -485,21 +504,51 @@ struct Builder {
     }
 };
 
-template <class T>
-wost_status upload(wost_scene *s, const std::vector<T> &v, const T **out) {
-    *out = nullptr;
-    if (v.empty()) return WOST_OK;
-    void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, v.size() * sizeof(T));
-    if (e != cudaSuccess) {
-        set_error("cudaMalloc failed while uploading the scene");
-        return e == cudaErrorMemoryAllocation ? WOST_ERR_OOM : WOST_ERR_CUDA;
+// The scene's device arrays.  Each allocation and copy costs about 10 us, a
+// third of the creation of a small scene, so arrays of up to kPacked bytes go
+// into one allocation, with one copy (64 segments: 185 / 150 us); a larger one
+// is copied from where it is.
+struct Uploader {
+    static constexpr size_t kPacked = 256 << 10;
+    wost_scene *s;
+    std::vector<unsigned char> blob{};
+    std::vector<std::pair<const void **, size_t>> at{};   // pointers into the blob's device copy
+
+    wost_status send(const void *src, size_t bytes, const void **out) {
+        void *p = nullptr;
+        cudaError_t e = cudaMalloc(&p, bytes);
+        if (e != cudaSuccess) {
+            set_error("cudaMalloc failed while uploading the scene");
+            return e == cudaErrorMemoryAllocation ? WOST_ERR_OOM : WOST_ERR_CUDA;
+        }
+        s->allocs.push_back(p);
+        WOST_CUDA(cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice));
+        *out = p;
+        return WOST_OK;
     }
-    s->allocs.push_back(p);
-    WOST_CUDA(cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
-    *out = reinterpret_cast<const T *>(p);
-    return WOST_OK;
-}
+    template <class T>
+    wost_status add(const std::vector<T> &v, const T **out) {
+        *out = nullptr;
+        const size_t bytes = v.size() * sizeof(T);
+        const void **o = reinterpret_cast<const void **>(out);
+        if (bytes == 0) return WOST_OK;
+        if (bytes > kPacked) return send(v.data(), bytes, o);
+        const size_t off = (blob.size() + 255) / 256 * 256;
+        blob.resize(off + bytes);
+        std::memcpy(blob.data() + off, v.data(), bytes);
+        at.push_back({o, off});
+        return WOST_OK;
+    }
+    // the packed arrays (their pointers are set here)
+    wost_status finish() {
+        if (blob.empty()) return WOST_OK;
+        const void *base = nullptr;
+        const wost_status st = send(blob.data(), blob.size(), &base);
+        if (st != WOST_OK) return st;
+        for (auto &x : at) *x.first = static_cast<const unsigned char *>(base) + x.second;
+        return WOST_OK;
+    }
+};
 
 bool valid_fn(const wost_fn &f) {
     if (f.kind < 0 || f.kind > 10) return false;
@@ -595,6 +644,7 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
     }
 
     auto fv = [&](int64_t vi, int k) { return (float)V[vi * d + k]; };
+    Uploader up{s};
 
     // ---- primitive BVHs (Dirichlet, Neumann) ----
     auto build_prims = [&](int bcv, DevBVH &bv, int &count, int &depth, std::vector<int> *slot_of) -> wost_status {
@@ -602,6 +652,7 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
         B.d = d;
         // (the caps' smaller leaves subdivide those of the boxes)
         B.leaf = bcv == 0 ? kLeafCaps : kLeaf;
+        B.items.reserve(bcv == 0 ? ndir : np - ndir);
         for (int64_t i = 0; i < np; ++i) {
             if (desc->bc[i] != bcv) continue;
             Item it;
@@ -651,7 +702,7 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
             }
         }
         wost_status st;
-        if ((st = upload(s, d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK) return st;
+        if ((st = up.add(d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK) return st;
         bv.nnodes = (int)(d == 2 ? B.nodes.size() : (bcv == 0 ? caps.size() : wide.size()));
         bv.need = caps.empty() ? 0 : Builder::stack_need(caps, 0);
         if (bcv == 0) {
@@ -664,12 +715,12 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
             }
             double far = diag;
             for (int k = 0; k < d; ++k) far = std::max(far, std::max(std::fabs(lo[k]), std::fabs(hi[k])));
-            if ((st = upload(s, d == 2 ? B.caps_binary(vp, vn, 1e-6 * far) : Builder::caps_wide(caps, vp, vn, 1e-6 * far),
+            if ((st = up.add(d == 2 ? B.caps_binary(vp, vn, 1e-6 * far) : Builder::caps_wide(caps, vp, vn, 1e-6 * far),
                              &s->dev.dir_caps)) != WOST_OK) return st;
         }
-        if ((st = upload(s, prims, &bv.prims)) != WOST_OK) return st;
-        if ((st = upload(s, ids, &bv.ids)) != WOST_OK) return st;
-        if ((st = upload(s, p64, &bv.prims64)) != WOST_OK) return st;
+        if ((st = up.add(prims, &bv.prims)) != WOST_OK) return st;
+        if ((st = up.add(ids, &bv.ids)) != WOST_OK) return st;
+        if ((st = up.add(p64, &bv.prims64)) != WOST_OK) return st;
         bv.nprims = count;
         return WOST_OK;
     };
@@ -685,7 +736,7 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
         for (int64_t i = 0; i < np; ++i)
             if (neu_slot[i] >= 0)
                 for (int k = 0; k < d; ++k) nn[(size_t)neu_slot[i] * d + k] = (float)nin[(size_t)i * d + k];
-        if ((st = upload(s, nn, &s->dev.nin_neu)) != WOST_OK) { delete s; return st; }
+        if ((st = up.add(nn, &s->dev.nin_neu)) != WOST_OK) { delete s; return st; }
     }
 
     // ---- silhouette elements ----
@@ -770,17 +821,15 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
         }
         DevBVH &bv = s->dev.sil;
         const double tau = (float)(1e-6 * diag);
-        if ((st = upload(s, d == 2 ? B.facing_binary(data, tau) : Builder::facing_wide(data, wide, tau), &s->dev.sil_facing)) != WOST_OK) { delete s; return st; }
-        if ((st = upload(s, d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK ||
-            (st = upload(s, prims, &bv.prims)) != WOST_OK || (st = upload(s, ids, &bv.ids)) != WOST_OK) {
+        if ((st = up.add(d == 2 ? B.facing_binary(data, tau) : Builder::facing_wide(data, wide, tau), &s->dev.sil_facing)) != WOST_OK) { delete s; return st; }
+        if ((st = up.add(d == 2 ? B.pack_binary() : Builder::pack_wide(wide), &bv.nodes)) != WOST_OK ||
+            (st = up.add(prims, &bv.prims)) != WOST_OK || (st = up.add(ids, &bv.ids)) != WOST_OK) {
             delete s;
             return st;
         }
         bv.nnodes = (int)(d == 2 ? B.nodes.size() : wide.size());
         bv.need = 0;
-        const int64_t *kp = nullptr;
-        if ((st = upload(s, keys, &kp)) != WOST_OK) { delete s; return st; }
-        s->sil_key = const_cast<int64_t *>(kp);
+        if ((st = up.add(keys, &s->sil_key)) != WOST_OK) { delete s; return st; }
         bv.prims64 = nullptr;
         bv.nprims = s->nsil;
     }
@@ -792,6 +841,7 @@ extern "C" wost_status wost_create_scene(const wost_scene_desc *desc, wost_scene
     s->dev.has_source = desc->f.kind != 0;
     s->dev.h = to_dev(desc->h);
     s->dev.has_flux = desc->h.kind != 0 && s->nneu > 0;
+    if ((st = up.finish()) != WOST_OK) { delete s; return st; }
     *out = s;
     return WOST_OK;
 }
