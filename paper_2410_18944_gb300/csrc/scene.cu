@@ -9,9 +9,10 @@
 #include <cfloat>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <numeric>
-#include <system_error>
 #include <thread>
+#include <utility>
 
 #include "coop.cuh"
 #include "internal.h"
@@ -186,11 +187,12 @@ void parallel_for(int n, F fn) {
             for (int j = i; j < std::min(n, i + 16); ++j) fn(j);
     };
     std::vector<std::thread> th;
+    th.reserve(nt);
     for (int t = 1; t < nt; ++t) {
         try {
             th.emplace_back(work);
-        } catch (const std::system_error &) {
-            break;   // no more threads to be had: those there are do the work
+        } catch (const std::exception &) {
+            break;   // no more threads (or memory for one) to be had: those there are do the work
         }
     }
     work();
